@@ -106,7 +106,8 @@ def _bitmap(case, generator):
     return packed.cpu().numpy().astype(np.uint32)
 
 
-def prepare(case, seed):
+def _inputs(case, seed):
+    """q, k, v on the GPU and the bitmap's words (None for the other masks), from the seed alone."""
     g = torch.Generator(device="cuda")
     g.manual_seed(seed)
     b, hq, hkv, sq, skv, d = (case[x] for x in ("batch", "heads_q", "heads_kv", "seq_q", "seq_kv", "head_dim"))
@@ -121,7 +122,12 @@ def prepare(case, seed):
     q, k, v = normal(hq, sq), normal(hkv, skv), normal(hkv, skv)
     # heads differ in how peaked their scores are
     q *= (0.5 + torch.rand((hq, 1, 1), generator=g, device="cuda")).to(torch.bfloat16)
-    bitmap = _bitmap(case, g) if case["mask"] == "bitmap" else None
+    return q, k, v, _bitmap(case, g) if case["mask"] == "bitmap" else None
+
+
+def prepare(case, seed):
+    q, k, v, bitmap = _inputs(case, seed)
+    b, hq, hkv, sq, skv, d = (case[x] for x in ("batch", "heads_q", "heads_kv", "seq_q", "seq_kv", "head_dim"))
     args = (b, hq, hkv, sq, skv, d, 1.0 / math.sqrt(d), FLAGS[case["mask"]])
     state = {"entry": case["entry"], "q": q, "k": k, "v": v}
     if case["entry"] == "run":
@@ -183,3 +189,43 @@ def tolerance(case):
     # listed and of drawn cases is off by 2.0e-3 to 2.4e-3 (2-norm) and by at most 0.035 of the larger of the
     # value and the root mean square; LSE by 2e-6.  Four times that.
     return {"rel": 1e-2, "max": 0.14}
+
+
+def exact(case, seed):
+    """O and LSE in float64 from the same operands: explicit scores, mask and softmax over blocks of query rows."""
+    b, hq, hkv, sq, skv, d = (case[x] for x in ("batch", "heads_q", "heads_kv", "seq_q", "seq_kv", "head_dim"))
+    if 1.0 * b * hq * sq * skv * d > 2e13:  # over about 20 s
+        return None
+    q, k, v, bitmap = _inputs(case, seed)
+    o = torch.empty((b, hq, sq, d), dtype=torch.float64, device="cuda")
+    lse = torch.empty((b, hq, sq), dtype=torch.float64, device="cuda")
+    keys = torch.arange(skv, device="cuda")
+    rows = max(1, min(sq, (1 << 28) // skv))
+    for i0 in range(0, sq, rows):
+        i1 = min(i0 + rows, sq)
+        # a key block's end bounds what these rows see under a causal mask; the first key, under a window
+        pos = torch.arange(i0, i1, device="cuda") + (skv - sq)
+        end = skv if case["mask"] == "dense" else min(skv, i1 + skv - sq)
+        begin = max(0, i0 + skv - sq - case["window"] + 1) if case["mask"] == "window" else 0
+        seen = torch.ones((i1 - i0, end - begin), dtype=torch.bool, device="cuda")
+        if case["mask"] != "dense":
+            seen &= keys[None, begin:end] <= pos[:, None]
+        if case["mask"] == "window":
+            seen &= pos[:, None] - keys[None, begin:end] < case["window"]
+        for n in range(b):
+            for h in range(hq):
+                kept = seen
+                if bitmap is not None:
+                    words = torch.from_numpy(bitmap[h].astype(np.int64)).cuda()
+                    n_j = -(-end // case["block"])
+                    j = torch.arange(n_j, device="cuda")
+                    i_blocks = torch.arange(i0, i1, device="cuda") // case["block"]
+                    bits = ((words[i_blocks][:, j >> 5] >> (j & 31)) & 1).bool()
+                    kept = seen & bits.repeat_interleave(case["block"], 1)[:, :end]
+                g = h // (hq // hkv)
+                s = q[n, h, i0:i1].double() @ k[n, g, begin:end].double().T
+                s *= 1.0 / math.sqrt(d)
+                s.masked_fill_(~kept, -math.inf)
+                lse[n, h, i0:i1] = torch.logsumexp(s, 1)
+                o[n, h, i0:i1] = s.sub_(lse[n, h, i0:i1, None]).exp_() @ v[n, g, begin:end].double()
+    return o, lse
