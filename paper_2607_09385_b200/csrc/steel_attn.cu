@@ -24,7 +24,6 @@ struct steel_attn {
   int32_t *d_cta_begin = nullptr;
   StepPair *d_steps = nullptr;
   int32_t *d_status = nullptr;
-  long long *d_trace = nullptr;  // debug builds only
   long long *d_clock_probe = nullptr;
   long long timeout_cycles = kDefaultTimeoutCycles;
   int32_t stall_cta = -1;
@@ -187,7 +186,6 @@ steel_status_t steel_attn_run(steel_attn_t *h, const void *q, const void *k, con
   kp.cta_begin = h->d_cta_begin;
   kp.steps = h->d_steps;
   kp.status = h->d_status;
-  kp.trace = h->d_trace;
   kp.clock_probe = h->d_clock_probe;
   kp.timeout_cycles = h->timeout_cycles;
   kp.stall_cta = h->stall_cta;
@@ -249,15 +247,6 @@ steel_status_t steel_attn_plan_host(const steel_attn_params_t *params, steel_att
   if (n_tiles) *n_tiles = n;
   return STEEL_OK;
 }
-
-#ifdef STEEL_TRACE
-// Debug builds: device buffer of gridDim.x * 32 counters filled by the kernel's roles.
-steel_status_t steel_attn_set_trace(steel_attn_t *h, long long *device_buffer) {
-  if (!h) return STEEL_ERR_INVALID_ARG;
-  h->d_trace = device_buffer;
-  return STEEL_OK;
-}
-#endif
 
 steel_status_t steel_attn_debug_clock_probe(steel_attn_t *h, int64_t *device_pair) {
   if (!h || (reinterpret_cast<uintptr_t>(device_pair) & 7u)) return STEEL_ERR_INVALID_ARG;

@@ -11,16 +11,26 @@
 //                     the First Stage, the Second Stage, and the rescale of the Third.)
 //   warp 8          : TMA producer and scheduler.  Walks the items, loads Q once per item and K_j / V_j
 //                     for executed tiles only into a shared-memory ring (a tile wanted by both slots
-//                     in the same step is loaded once), and publishes one command word per slot-step
-//                     for the MMA issuer, with ring slots, barrier phases and release flags worked out.
-//   warp 9          : MMA issuer.  Pops commands and issues S = Q K^T (both operands in shared memory)
-//                     and O += P V (P from TMEM, V from shared memory) on tcgen05 with fp32
-//                     accumulators in TMEM.  Its loop time is the kernel's period, so it does nothing else.
-//   warps 10-11     : idle (they only keep the warpgroup complete for the register re-split).
+//                     in the same step is loaded once), and publishes one command word per product
+//                     for its MMA issuer, with ring slots, barrier phases and release flags worked out.
+//   warps 9-11      : MMA issuers on tcgen05 with fp32 accumulators in TMEM: warp 9 issues S = Q K^T of
+//                     both slots (both operands in shared memory), warp 10 / 11 O += P V of slot 0 / 1 (P
+//                     from TMEM, V from shared memory).
 // Tensor memory (512 columns): one S buffer that the slots use in turn (128), P of each slot
-// (2 x 64), O of each slot (2 x head_dim).  S(s, t + 1) is issued before PV(s, t), so a slot's next
+// (2 x 64), O of each slot (2 x head_dim).  S(s, t + 1) does not wait for PV(s, t), so a slot's next
 // scores are computed while its softmax warps still work on the current tile.  (At head_dim 64 the
-// columns would allow an S buffer per slot; measured, that layout was 9 % slower.)
+// columns would allow an S buffer per slot; measured, that layout is slower: 32 heads of 8192 tokens
+// 419 us against 382 us.  The shared buffer keeps the slots half a tile apart, so that one computes
+// exponentials while the other reads scores and searches its maximum.)
+//
+// What bounds it: the chain S -> registers -> hand-back of the S buffer -> next S, and the softmax warps'
+// instruction stream (16 384 exponentials per tile: 1 024 cycles of the special-function unit at best, as
+// much as the tile's two products take on the tensor core at head_dim 128).  Three issuers instead of one,
+// because a tcgen05.commit returns only when the products before it have nearly drained: one thread that
+// issues everything spends 1 450 to 1 700 cycles per pair of products that take 1 024.  Measured, one
+// issuer -> three (kernel time): 32 heads x 4096 causal, head_dim 128: 136.5 -> 125.6 us; 16 heads x 32768,
+// bitmap 25 %: 1 027 -> 954 us; 32/8 heads x 16384 causal: 1 753 -> 1 635 us; 32 heads x 8192 causal,
+// head_dim 64: 408 -> 382 us.  Two issuers, one per slot with both its products: 126 / 968 / 1 636 / 395 us.
 // Every mbarrier and queue wait is bounded; on expiry the CTA sets the status word and all roles leave.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -33,7 +43,7 @@
 
 namespace steel {
 
-constexpr int kThreads = 384;        // softmax slot 0, softmax slot 1, {producer, MMA, 2 idle warps}
+constexpr int kThreads = 384;        // softmax slot 0, softmax slot 1, {producer, 3 MMA issuers}
 // Registers per thread after the warpgroups re-split the file.  2 * 128 * kRegsSoftmax + 128 *
 // kRegsOther must stay below the 65 536 registers of an SM with room to spare: setmaxnreg.inc waits,
 // without any bound, until the increase can be granted.
@@ -41,7 +51,7 @@ constexpr int kRegsSoftmax = 216;
 constexpr int kRegsOther = 72;
 static_assert(2 * 128 * kRegsSoftmax + 128 * kRegsOther <= 65536 - 1024, "register re-split needs slack");
 constexpr int kProducerWarp = 8;
-constexpr int kMmaWarp = 9;
+constexpr int kMmaWarp = 9;  // first of three: S of both slots, PV of slot 0, PV of slot 1
 constexpr float kRescaleThreshold = 8.0f;           // lazy rescale: P stays below 2^8
 constexpr int kMaxStages = 10;
 constexpr int kFifoDepth = 32;
@@ -63,37 +73,23 @@ struct Ctrl {
   uint64_t ring_full[kMaxStages], ring_empty[kMaxStages];
   uint64_t q_full[2], q_empty[2], s_full[2], p_full[2], p_free[2], o_full[2], o_empty[2];
   uint64_t s_free;     // the softmax warps that own the S buffer's content have it in registers
-  uint64_t drain;      // the MMA issuer's last commit when it leaves on an expired wait
-  uint32_t fifo[kFifoDepth];  // command words from the producer to the MMA issuer (0 = empty)
+  uint64_t drain[3];   // an MMA issuer's last commit when it leaves on an expired wait
+  uint32_t fifo[3][kFifoDepth];  // command words from the producer to the MMA issuers (0 = empty)
   uint32_t tmem_base;
   int abort;
   long long timeout_cycles;
 };
 
-// Command word (producer -> MMA issuer): one word carries S(s, t + 1), PV(s, t) or both (the usual
-// case: the first product of the next step is issued right before the second product of this one).
-constexpr uint32_t kCmdValid = 1u << 0, kCmdHasPV = 1u << 1, kCmdHasS = 1u << 2, kCmdSlot1 = 1u << 3,
-                   kCmdVRingShift = 4, kCmdKRingShift = 8,  // 4 bits each: ring slot of the V / K tile
-                   kCmdVPhase = 1u << 12, kCmdKPhase = 1u << 13, kCmdVSkipWait = 1u << 14, kCmdKSkipWait = 1u << 15,
-                   kCmdVFinal = 1u << 16, kCmdKFinal = 1u << 17,  // last user: release the ring slot
-                   kCmdWaitOEmpty = 1u << 18, kCmdOEmptyPhase = 1u << 19, kCmdWaitQFull = 1u << 20,
-                   kCmdQFullPhase = 1u << 21, kCmdAcc = 1u << 22, kCmdPPhase = 1u << 23, kCmdOEnd = 1u << 24,
-                   kCmdQEnd = 1u << 25, kCmdWaitSFree = 1u << 26, kCmdSFreePhase = 1u << 27, kCmdExit = 1u << 31;
-
-// Optional per-role wait accounting (compiled in with -DSTEEL_TRACE only): cycles per CTA, 32 slots.
-#ifdef STEEL_TRACE
-#define TRACE_T0() const long long trace_t0_ = clock64()
-#define TRACE_ADD(idx) trace_acc[idx] += clock64() - trace_t0_
-#define TRACE_DECL(n) long long trace_acc[n] = {}
-#define TRACE_FLUSH(base, n)                                                               \
-  if (p.trace)                                                                             \
-    for (int i_ = 0; i_ < (n); ++i_) p.trace[size_t(blockIdx.x) * 32 + (base) + i_] = trace_acc[i_]
-#else
-#define TRACE_T0()
-#define TRACE_ADD(idx)
-#define TRACE_DECL(n)
-#define TRACE_FLUSH(base, n)
-#endif
+// Command word (producer -> MMA issuer): one product, S(s, t) or PV(s, t).
+constexpr uint32_t kCmdValid = 1u << 0, kCmdSlot1 = 1u << 1,
+                   kCmdFirst = 1u << 2, kCmdLast = 1u << 3,  // of the slot's steps in this item
+                   kCmdRingShift = 4,  // 4 bits: ring slot of the K or V tile
+                   kCmdRingPhase = 1u << 8,
+                   kCmdUsePhase = 1u << 9,    // Q full (S), O empty (PV); read with kCmdFirst
+                   kCmdDepPhase = 1u << 10,   // S buffer free (S), P full (PV)
+                   kCmdWaitSFree = 1u << 11,  // not the CTA's first S
+                   kCmdFinal = 1u << 12,      // S: last reader of the K tile, release the ring slot
+                   kCmdExit = 1u << 31;
 
 __device__ __forceinline__ bool bounded_wait(uint64_t *bar, uint32_t parity, Ctrl &ctrl, int32_t *status) {
   if (mbar_test_wait(bar, parity)) return true;  // the common case: already complete, no suspension
@@ -112,12 +108,25 @@ __device__ __forceinline__ bool bounded_wait(uint64_t *bar, uint32_t parity, Ctr
   }
 }
 
-// One lane polls on behalf of its warp; the vote both broadcasts the outcome and orders the other
-// lanes after the observation.
+// Wait by a whole warp: every lane tests the same barrier and the vote both keeps the warp together and
+// orders its lanes after the observation.
 __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, Ctrl &ctrl, int32_t *status, int lane) {
-  bool ok = true;
-  if (lane == 0) ok = bounded_wait(bar, parity, ctrl, status);
-  return __all_sync(0xffffffffu, ok);
+  if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
+  const long long start = clock64();
+  uint32_t n = 0;
+  while (true) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if ((++n & 63u) == 0) {
+      const bool stop = *reinterpret_cast<volatile int *>(&ctrl.abort) != 0 || clock64() - start > ctrl.timeout_cycles;
+      if (__any_sync(0xffffffffu, stop)) {
+        if (lane == 0 && *reinterpret_cast<volatile int *>(&ctrl.abort) == 0) {
+          *reinterpret_cast<volatile int *>(&ctrl.abort) = 1;
+          atomicExch(status, 5);
+        }
+        return false;
+      }
+    }
+  }
 }
 
 // A work item unpacked into scalars (no indexable arrays, so everything stays in registers).
@@ -157,7 +166,7 @@ __device__ __forceinline__ uint2 load_step(const Item &w, const StepPair *steps,
 
 // The canonical order of an item's tensor-core operations S(s, t) = Q_s K_j^T and PV(s, t):
 // O_s += P_s V_j: the order in which the producer loads tiles (at their first use) and publishes
-// commands, and therefore the order in which the MMA issuer executes them.
+// commands, and therefore the order in which each MMA issuer executes its own.
 // For each step t: first S(s, t) of slots that start at t, then for each present slot S(s, t + 1)
 // followed by PV(s, t): the first product runs one step ahead of the second, so a slot's next scores
 // are computed while its softmax warps still work on the current ones (they hold them in registers;
@@ -222,8 +231,8 @@ __device__ __forceinline__ bool walk_item(const Item &w, const StepPair *steps, 
 // ------------------------------------------------------------------------------------------------
 // Bounded push into the single-producer single-consumer command queue in shared memory (the pop is
 // with the MMA issuer below).
-__device__ __forceinline__ bool fifo_push(Ctrl &ctrl, uint32_t &tail, uint32_t word, int32_t *status) {
-  volatile uint32_t *cell = &ctrl.fifo[tail];
+__device__ __forceinline__ bool fifo_push(Ctrl &ctrl, int s, uint32_t &tail, uint32_t word, int32_t *status) {
+  volatile uint32_t *cell = &ctrl.fifo[s][tail];
   if (*cell != 0) {
     const long long start = clock64();
     uint32_t n = 0;
@@ -243,8 +252,7 @@ __device__ __forceinline__ bool fifo_push(Ctrl &ctrl, uint32_t &tail, uint32_t w
   return true;
 }
 // The producer is also the scheduler: it walks the items, issues the TMA loads and publishes one
-// command word per slot-step (PV(s, t) fused with the S(s, t + 1) that follows it), so the MMA
-// issuer's own loop stays a few instructions long.
+// command word per product, so the MMA issuers' own loops stay a few instructions long.
 template <int D>
 __device__ void producer_role(const KernelParams &p, const CUtensorMap *map_q, const CUtensorMap *map_k,
                               const CUtensorMap *map_v, Ctrl &ctrl, uint8_t *smem_q, uint8_t *smem_ring) {
@@ -258,7 +266,7 @@ __device__ void producer_role(const KernelParams &p, const CUtensorMap *map_q, c
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(probe_t0));
   }
   RingPos ring{0, 0};
-  uint32_t n_use0 = 0, n_use1 = 0, n_sp0 = 0, n_sp1 = 0, n_s = 0, fills = 0, tail = 0, pending = 0;
+  uint32_t n_use0 = 0, n_use1 = 0, n_sp0 = 0, n_sp1 = 0, n_s = 0, fills = 0, tail_s = 0, tail_pv0 = 0, tail_pv1 = 0;
   bool ok = true;
   const bool stalled = p.stall_cta == int(blockIdx.x);
   const int k_end = p.cta_begin[blockIdx.x + 1];
@@ -282,6 +290,9 @@ __device__ void producer_role(const KernelParams &p, const CUtensorMap *map_q, c
     ok = walk_item<C::kStages>(w, p.steps, ring, [&](int s, int t, int j, bool is_s, Fill f, bool first, bool final_use) -> bool {
       if (first) {
         if (!bounded_wait(&ctrl.ring_empty[f.slot], f.phase ^ 1u, ctrl, p.status)) return false;
+        // a ring slot is free again after two arrivals: the issuers of both slots release a V tile that both
+        // want; K has one issuer, and a tile that one slot wants one reader
+        if (is_s || final_use) mbar_arrive(&ctrl.ring_empty[f.slot]);
         mbar_arrive_expect_tx(&ctrl.ring_full[f.slot], C::kTileBytes);
         const CUtensorMap *map = is_s ? map_k : map_v;
 #pragma unroll
@@ -292,36 +303,26 @@ __device__ void producer_role(const KernelParams &p, const CUtensorMap *map_q, c
       }
       // phase of this item's use of the slot: Q-full for S, O-empty (inverted) for PV
       const uint32_t use_phase = ((s ? n_use1 : n_use0) - 1u) & 1u;
+      uint32_t cmd = kCmdValid | (f.slot << kCmdRingShift) | (f.phase ? kCmdRingPhase : 0u) |
+                     (t == w.lo(s) ? kCmdFirst : 0u) | (t == w.hi(s) ? kCmdLast : 0u);
       if (is_s) {
         // the S buffer is shared: S number n may be issued once S number n - 1 has been loaded into registers
-        uint32_t part = kCmdHasS | (f.slot << kCmdKRingShift) | (f.phase ? kCmdKPhase : 0u) |
-                        (first ? 0u : kCmdKSkipWait) | (final_use ? kCmdKFinal : 0u) |
-                        (n_s > 0 ? kCmdWaitSFree : 0u) | (((n_s - 1u) & 1u) ? kCmdSFreePhase : 0u);
+        cmd |= (s ? kCmdSlot1 : 0u) | (use_phase ? kCmdUsePhase : 0u) | (final_use ? kCmdFinal : 0u) |
+               (n_s > 0 ? kCmdWaitSFree : 0u) | (((n_s - 1u) & 1u) ? kCmdDepPhase : 0u);
         ++n_s;
-        if (t == w.lo(s)) part |= kCmdWaitQFull | (use_phase ? kCmdQFullPhase : 0u);
-        if (t == w.hi(s)) part |= kCmdQEnd;
-        if (t == w.lo(s)) {
-          // first step of the slot: nothing of this slot to pair it with
-          if (stalled) return true;  // test hook: the issuer's bounded wait for this command must expire
-          return fifo_push(ctrl, tail, part | kCmdValid | (s ? kCmdSlot1 : 0u), p.status);
-        }
-        pending = part;  // completed by the PV(s, t - 1) that the walk visits next
-        return true;
+        if (stalled) return true;  // test hook: the issuer's bounded wait for this command must expire
+        return fifo_push(ctrl, 0, tail_s, cmd, p.status);
       }
       uint32_t &n_sp = s ? n_sp1 : n_sp0;
-      uint32_t part = kCmdHasPV | (f.slot << kCmdVRingShift) | (f.phase ? kCmdVPhase : 0u) |
-                      (first ? 0u : kCmdVSkipWait) | (final_use ? kCmdVFinal : 0u) | (t > w.lo(s) ? kCmdAcc : 0u) |
-                      ((n_sp & 1u) ? kCmdPPhase : 0u);
-      if (t == w.lo(s)) part |= kCmdWaitOEmpty | ((use_phase ^ 1u) ? kCmdOEmptyPhase : 0u);
-      if (t == w.hi(s)) part |= kCmdOEnd;
+      cmd |= ((use_phase ^ 1u) ? kCmdUsePhase : 0u) | ((n_sp & 1u) ? kCmdDepPhase : 0u);
       ++n_sp;
-      const uint32_t cmd = pending | part | kCmdValid | (s ? kCmdSlot1 : 0u);
-      pending = 0;
       if (stalled) return true;
-      return fifo_push(ctrl, tail, cmd, p.status);
+      return fifo_push(ctrl, 1 + s, s ? tail_pv1 : tail_pv0, cmd, p.status);
     });
   }
-  if (ok) ok = fifo_push(ctrl, tail, kCmdValid | kCmdExit, p.status);
+  if (ok) ok = fifo_push(ctrl, 0, tail_s, kCmdValid | kCmdExit, p.status);
+  if (ok) ok = fifo_push(ctrl, 1, tail_pv0, kCmdValid | kCmdExit, p.status);
+  if (ok) ok = fifo_push(ctrl, 2, tail_pv1, kCmdValid | kCmdExit, p.status);
   if (probe) {
     unsigned long long t1;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
@@ -368,8 +369,8 @@ __device__ __forceinline__ uint32_t warp_uniform(uint32_t word, int lane) {
 
 // Pop by the whole warp: every lane polls the same cell; the decision to leave is taken on the
 // voted word, so the lanes stay together.  Lane 0 empties the cell.
-__device__ __forceinline__ uint32_t fifo_pop_warp(Ctrl &ctrl, uint32_t &head, int32_t *status, int lane) {
-  volatile uint32_t *cell = &ctrl.fifo[head];
+__device__ __forceinline__ uint32_t fifo_pop_warp(Ctrl &ctrl, int s, uint32_t &head, int32_t *status, int lane) {
+  volatile uint32_t *cell = &ctrl.fifo[s][head];
   __syncwarp();
   uint32_t word = warp_uniform(*cell, lane);
   if (word == 0) {
@@ -396,8 +397,12 @@ __device__ __forceinline__ uint32_t fifo_pop_warp(Ctrl &ctrl, uint32_t &head, in
   return word;
 }
 
+// Three issuing warps: one for the first products of both slots, one for the second products of each
+// slot.  None of them waits for anything but the inputs of its own next product.  Accumulation chains
+// (O of a slot) stay within one thread, which is what tcgen05 orders.
 template <int D>
-__device__ void mma_role(const KernelParams &p, Ctrl &ctrl, uint8_t *smem_q, uint8_t *smem_ring, const int lane) {
+__device__ void mma_role(const KernelParams &p, Ctrl &ctrl, uint8_t *smem_q, uint8_t *smem_ring, const int who,
+                         const int lane) {
   using C = Cfg<D>;
   const uint32_t tmem = warp_uniform(ctrl.tmem_base, lane);
   const uint32_t idesc_s = make_idesc_bf16(kTile, kTile, 0, 0);
@@ -407,99 +412,56 @@ __device__ void mma_role(const KernelParams &p, Ctrl &ctrl, uint8_t *smem_q, uin
   const uint64_t desc_v0 = make_smem_desc(smem_u32(smem_ring), C::kBoxBytes, 1024);
   uint32_t head = 0;
   bool ok = true;
-  TRACE_DECL(8);
-#ifdef STEEL_TRACE
-  const long long role_t0 = clock64();
-#endif
-  uint32_t cmd = fifo_pop_warp(ctrl, head, p.status, lane);
+  auto wait = [&](uint64_t *bar, uint32_t parity) {
+    if (ok) ok = bounded_wait(bar, parity, ctrl, p.status);
+  };
+  uint32_t cmd = fifo_pop_warp(ctrl, who, head, p.status, lane);
   while (!(cmd & kCmdExit)) {
     // look at the next command now, so that its shared-memory latency hides behind this one's issue
-    volatile uint32_t *next_cell = &ctrl.fifo[head];
+    volatile uint32_t *next_cell = &ctrl.fifo[who][head];
     __syncwarp();
     const uint32_t next_raw = *next_cell;
-    const uint32_t s = (cmd & kCmdSlot1) ? 1u : 0u;
-    const uint32_t v_slot = (cmd >> kCmdVRingShift) & 0xFu, k_slot = (cmd >> kCmdKRingShift) & 0xFu;
-    const bool has_pv = (cmd & kCmdHasPV) != 0, has_s = (cmd & kCmdHasS) != 0;
-    constexpr uint32_t kRare = kCmdWaitOEmpty | kCmdWaitQFull | kCmdOEnd | kCmdQEnd;
-    const uint32_t rare = cmd & kRare;
-    // One elected lane does the barrier work and issues; the other lanes only keep the loop's
-    // control values uniform.
+    const uint32_t slot = (cmd >> kCmdRingShift) & 0xFu;
+    const uint32_t ring_phase = (cmd & kCmdRingPhase) ? 1u : 0u, use_phase = (cmd & kCmdUsePhase) ? 1u : 0u,
+                   dep_phase = (cmd & kCmdDepPhase) ? 1u : 0u;
     if (elect_one()) {
-      TRACE_T0();
-      // test the barriers the command depends on back to back, so their latencies overlap; only
-      // the ones not yet complete are then waited for
-      const bool need_v = has_pv && !(cmd & kCmdVSkipWait), need_k = has_s && !(cmd & kCmdKSkipWait);
-      const bool need_f = has_s && (cmd & kCmdWaitSFree);
-      uint64_t *s_free = &ctrl.s_free;
-      bool ok_f = !need_f || mbar_test_wait(s_free, (cmd & kCmdSFreePhase) ? 1u : 0u);
-      bool ok_k = !need_k || mbar_test_wait(&ctrl.ring_full[k_slot], (cmd & kCmdKPhase) ? 1u : 0u);
-      bool ok_v = !need_v || mbar_test_wait(&ctrl.ring_full[v_slot], (cmd & kCmdVPhase) ? 1u : 0u);
-      if (has_s) {
-        // S(s, t + 1) into the shared S buffer: its previous content must be in its owners' registers
-        if (rare | uint32_t(!ok_f) | uint32_t(!ok_k)) {
-          if (cmd & kCmdWaitQFull)
-            ok = bounded_wait(&ctrl.q_full[s], (cmd & kCmdQFullPhase) ? 1u : 0u, ctrl, p.status);
-          if (ok && !ok_f) {
-            TRACE_T0();
-            ok = bounded_wait(s_free, (cmd & kCmdSFreePhase) ? 1u : 0u, ctrl, p.status);
-            TRACE_ADD(0);
-          }
-          if (ok && !ok_k) {
-            TRACE_T0();
-            ok = bounded_wait(&ctrl.ring_full[k_slot], (cmd & kCmdKPhase) ? 1u : 0u, ctrl, p.status);
-            TRACE_ADD(1);
-          }
-        }
+      if (who == 0) {
+        const uint32_t s = (cmd & kCmdSlot1) ? 1u : 0u;
+        if (cmd & kCmdFirst) wait(&ctrl.q_full[s], use_phase);
+        wait(&ctrl.ring_full[slot], ring_phase);
+        if (cmd & kCmdWaitSFree) wait(&ctrl.s_free, dep_phase);
         if (ok) {
           tc_fence_after();
           const uint64_t dq = desc_q0 + uint64_t((s * C::kTileBytes) >> 4);
-          const uint64_t dk = desc_k0 + uint64_t((k_slot * C::kTileBytes) >> 4);
+          const uint64_t dk = desc_k0 + uint64_t((slot * C::kTileBytes) >> 4);
 #pragma unroll
           for (int kk = 0; kk < D / 16; ++kk) {
             const uint64_t off = uint64_t(((kk / 4) * C::kBoxBytes + (kk % 4) * 32) >> 4);
             mma_ss(tmem + C::kColS, dq + off, dk + off, idesc_s, kk > 0);
           }
+          tc_commit(&ctrl.s_full[s]);
+          tc_commit_if(&ctrl.ring_empty[slot], cmd & kCmdFinal);
+          tc_commit_if(&ctrl.q_empty[s], cmd & kCmdLast);
         }
-      }
-      // A commit does not return before the instructions it covers have nearly drained, so the
-      // test of the next group's barrier goes between issuing this group and committing it.
-      const uint32_t p_phase = (cmd & kCmdPPhase) ? 1u : 0u;
-      const bool ok_p = !has_pv || mbar_test_wait(&ctrl.p_full[s], p_phase);
-      if (ok && has_s) {
-        tc_commit(&ctrl.s_full[s]);
-        tc_commit_if(&ctrl.ring_empty[k_slot], cmd & kCmdKFinal);
-        if (rare) tc_commit_if(&ctrl.q_empty[s], cmd & kCmdQEnd);
-      }
-      if (ok && has_pv) {
-        // O_s += P_s V: P from its own TMEM columns, written by the softmax warps of slot s
-        if (rare | uint32_t(!ok_p) | uint32_t(!ok_v)) {
-          if (cmd & kCmdWaitOEmpty) ok = bounded_wait(&ctrl.o_empty[s], (cmd & kCmdOEmptyPhase) ? 1u : 0u, ctrl, p.status);
-          if (ok && !ok_v) {
-            TRACE_T0();
-            ok = bounded_wait(&ctrl.ring_full[v_slot], (cmd & kCmdVPhase) ? 1u : 0u, ctrl, p.status);
-            TRACE_ADD(2);
-          }
-          if (ok && !ok_p) {
-            TRACE_T0();
-            ok = bounded_wait(&ctrl.p_full[s], p_phase, ctrl, p.status);
-            TRACE_ADD(3);
-          }
-        }
+      } else {
+        const uint32_t s = who - 1;
+        if (cmd & kCmdFirst) wait(&ctrl.o_empty[s], use_phase);
+        wait(&ctrl.ring_full[slot], ring_phase);
+        wait(&ctrl.p_full[s], dep_phase);
         if (ok) {
+          // O_s += P_s V: P from its own TMEM columns, written by the softmax warps of slot s
           tc_fence_after();
-          const uint64_t dv = desc_v0 + uint64_t((v_slot * C::kTileBytes) >> 4);
-          const uint32_t t_p = tmem + C::kColP + s * (kTile / 2);
-          const uint32_t t_o = tmem + C::kColO + s * D;
-          const uint32_t acc0 = (cmd & kCmdAcc) ? 1u : 0u;
+          const uint64_t dv = desc_v0 + uint64_t((slot * C::kTileBytes) >> 4);
+          const uint32_t t_p = tmem + C::kColP + s * (kTile / 2), t_o = tmem + C::kColO + s * D;
+          const uint32_t acc0 = (cmd & kCmdFirst) ? 0u : 1u;
 #pragma unroll
           for (int kk = 0; kk < kTile / 16; ++kk)
             mma_ts(t_o, t_p + kk * 8, dv + uint64_t((kk * 2048) >> 4), idesc_pv, kk > 0 ? 1u : acc0);
           tc_commit(&ctrl.p_free[s]);
-          tc_commit_if(&ctrl.ring_empty[v_slot], cmd & kCmdVFinal);
-          if (rare) tc_commit_if(&ctrl.o_full[s], cmd & kCmdOEnd);
+          tc_commit(&ctrl.ring_empty[slot]);
+          tc_commit_if(&ctrl.o_full[s], cmd & kCmdLast);
         }
       }
-      TRACE_ADD(5);
     }
     const uint32_t next = warp_uniform(next_raw, lane);
     if (__any_sync(0xffffffffu, !ok)) break;
@@ -508,22 +470,16 @@ __device__ void mma_role(const KernelParams &p, Ctrl &ctrl, uint8_t *smem_q, uin
       head = (head + 1) & (kFifoDepth - 1);
       cmd = next;
     } else {
-      TRACE_T0();
-      cmd = fifo_pop_warp(ctrl, head, p.status, lane);
-      TRACE_ADD(4);
+      cmd = fifo_pop_warp(ctrl, who, head, p.status, lane);
     }
   }
-#ifdef STEEL_TRACE
-  trace_acc[7] = clock64() - role_t0;
-  if (elect_one()) { TRACE_FLUSH(0, 8); }
-#endif
   // Leaving on an expired wait: everything this warp issued must have retired before the CTA frees
   // its tensor memory, so commit to a spare barrier and wait for it (bounded).
   if (*reinterpret_cast<volatile int *>(&ctrl.abort)) {
     if (elect_one()) {
-      tc_commit(&ctrl.drain);
+      tc_commit(&ctrl.drain[who]);
       const long long start = clock64();
-      while (!mbar_try_wait(&ctrl.drain, 0) && clock64() - start < ctrl.timeout_cycles / 8) {
+      while (!mbar_try_wait(&ctrl.drain[who], 0) && clock64() - start < ctrl.timeout_cycles / 8) {
       }
     }
   }
@@ -590,12 +546,6 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
   const float2 scale2 = make_float2(scale_log2, scale_log2);
   __nv_bfloat16 *o_base = static_cast<__nv_bfloat16 *>(p.o);
   uint32_t n_sp = 0, n_use = 0;
-  TRACE_DECL(7);
-#ifdef STEEL_TRACE
-  const long long role_t0 = clock64();
-  unsigned long long gt0;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(gt0));
-#endif
 
   const int k_end = p.cta_begin[blockIdx.x + 1];
   for (int k = p.cta_begin[blockIdx.x]; k < k_end; ++k) {
@@ -607,21 +557,24 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
     const int lo = w.lo(s), hi = w.hi(s);
     const bool active = hi >= lo;
 
+    // Range items: tiles f_lo .. f_hi need no element-wise mask (case ii).  List items carry it in the entry.
+    int f_lo = 0, f_hi = p.seq_kv / kTile - 1;
+    if (causal) f_hi = min(f_hi, (w.qtile(s) * kTile + off + 1) / kTile - 1);
+    if (windowed) {
+      const int first = min(w.qtile(s) * kTile + kTile - 1, p.seq_q - 1) + off - p.window + 1;
+      f_lo = first > 0 ? (first + kTile - 1) / kTile : 0;
+    }
+    const uint32_t *entries = reinterpret_cast<const uint32_t *>(p.steps + w.list_off) + s;
+    uint32_t next_entry = (w.kind != 0 && active) ? __ldg(entries + 2 * lo) : 0u;
+
     for (int t = lo; t <= hi; ++t) {
       // which key tile, and does it need the element-wise mask (case iii)?
-      int j;
-      bool partial;
+      int j = w.j0 + t;
+      bool partial = j < f_lo || j > f_hi;
       uint32_t sub = 0xF;
-      if (w.kind == 0) {
-        j = w.j0 + t;
-        const int i0 = w.qtile(s) * kTile, i1 = min(i0 + kTile - 1, p.seq_q - 1);
-        const int j0 = j * kTile, j1 = min(j0 + kTile - 1, p.seq_kv - 1);
-        const bool full = (!causal || j1 <= i0 + off) && (!windowed || (i1 + off) - j0 < p.window) &&
-                          (j1 - j0 + 1 == kTile);
-        partial = !full;
-      } else {
-        const uint2 sp = __ldg(reinterpret_cast<const uint2 *>(p.steps + w.list_off + t));
-        const uint32_t e = s ? sp.y : sp.x;
+      if (w.kind != 0) {
+        const uint32_t e = next_entry;
+        next_entry = t < hi ? __ldg(entries + 2 * (t + 1)) : 0u;
         j = int(e & kEntryTileMask);
         partial = (e & kEntryPartial) != 0;
         sub = (e >> kEntrySubShift) & 0xF;
@@ -629,13 +582,10 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
 
       bool ok;
       {
-        TRACE_T0();
         ok = warp_wait(&ctrl.s_full[s], n_sp & 1u, ctrl, p.status, lane);
-        TRACE_ADD(0);
       }
       if (!ok) return;
       tc_fence_after();
-      TRACE_T0();
 
       float x[kTile];
 #pragma unroll
@@ -650,7 +600,6 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&ctrl.s_free);
-      TRACE_ADD(2);
 
       if (partial) {
         // visible columns of this row form one interval [c_lo, c_hi] of the tile
@@ -726,21 +675,17 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
       // The polynomial path returns 2^-125 rather than 0 for a masked (-inf) score: a row that has
       // not seen a visible key yet (m = -inf) must keep l = 0 exactly, so that it ends as O = 0.
       if (kEmu == 0 || m_ref != -CUDART_INF_F) l += acc.x + acc.y;
-      TRACE_ADD(3);
     }
 
     // epilogue: O / l and LSE = ln2 * (m + log2 l)
     if (active) {
       bool ok;
       {
-        TRACE_T0();
         ok = warp_wait(&ctrl.o_full[s], n_use & 1u, ctrl, p.status, lane);
-        TRACE_ADD(1);
       }
       if (!ok) return;
       ++n_use;
       tc_fence_after();
-      TRACE_T0();
       const float inv = l > 0.0f ? 1.0f / l : 0.0f;
 #pragma unroll
       for (int c = 0; c < D / 32; ++c) {
@@ -765,7 +710,6 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
       if (lane == 0) mbar_arrive(&ctrl.o_empty[s]);
       if (p.lse != nullptr && row < p.seq_q)
         p.lse[out_row] = l > 0.0f ? 0.6931471805599453f * (m_ref + log2f(l)) : -CUDART_INF_F;
-      TRACE_ADD(4);
     } else if (row < p.seq_q) {
       // no key tile is visible to this query tile
       uint4 *dst = reinterpret_cast<uint4 *>(o_base + out_row * D);
@@ -774,15 +718,6 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
       if (p.lse != nullptr) p.lse[out_row] = -CUDART_INF_F;
     }
   }
-#ifdef STEEL_TRACE
-  trace_acc[6] = clock64() - role_t0;
-  if (r == 0) {
-    unsigned long long gt1;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(gt1));
-    if (p.trace && s == 0) p.trace[size_t(blockIdx.x) * 32 + 15] = (long long)(gt1 - gt0);
-    TRACE_FLUSH(16 + 8 * s, 7);
-  }
-#endif
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -801,7 +736,7 @@ steel_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
   if (threadIdx.x == 0) {
     for (int i = 0; i < C::kStages; ++i) {
       mbar_init(&ctrl.ring_full[i], 1);
-      mbar_init(&ctrl.ring_empty[i], 1);
+      mbar_init(&ctrl.ring_empty[i], 2);
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(&ctrl.q_full[s], 1);
@@ -813,8 +748,8 @@ steel_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
       mbar_init(&ctrl.o_empty[s], 4);
     }
     mbar_init(&ctrl.s_free, 4);
-    mbar_init(&ctrl.drain, 1);
-    for (int i = 0; i < kFifoDepth; ++i) ctrl.fifo[i] = 0;
+    for (int i = 0; i < 3; ++i) mbar_init(&ctrl.drain[i], 1);
+    for (int i = 0; i < 3 * kFifoDepth; ++i) ctrl.fifo[0][i] = 0;
     ctrl.abort = 0;
     ctrl.timeout_cycles = p.timeout_cycles;
     fence_barrier_init();
@@ -839,8 +774,8 @@ steel_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     setmaxnreg_dec<kRegsOther>();
     if (warp == kProducerWarp) {
       if (lane == 0) producer_role<D>(p, &map_q, &map_k, &map_v, ctrl, smem_q, smem_ring);
-    } else if (warp == kMmaWarp) {
-      mma_role<D>(p, ctrl, smem_q, smem_ring, lane);
+    } else if (warp >= kMmaWarp) {
+      mma_role<D>(p, ctrl, smem_q, smem_ring, warp - kMmaWarp, lane);
     }
   }
 

@@ -113,7 +113,6 @@ extern "C" steel_status_t steel_attn_run_noalloc(const steel_attn_params_t *para
   kp.cta_begin = reinterpret_cast<const int32_t *>(base + kOffCtaBegin);
   kp.steps = reinterpret_cast<const StepPair *>(base + kOffSteps);
   kp.status = reinterpret_cast<int32_t *>(base + kOffStatus);
-  kp.trace = nullptr;
   kp.clock_probe = nullptr;
   kp.timeout_cycles = kDefaultTimeoutCycles;
   kp.stall_cta = -1;
