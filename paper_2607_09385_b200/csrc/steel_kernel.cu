@@ -610,8 +610,17 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
         const uint32_t half = (sub >> (2 * (r / 64))) & 3u;  // bit 0: keys 0-63 enabled, bit 1: keys 64-127
         if (!(half & 1u)) c_lo = max(c_lo, 64);
         if (!(half & 2u)) c_hi = min(c_hi, 63);
+        // As bits c_lo .. c_hi of four words: a bit test and a select per score instead of two comparisons
+        // and a select.  The code sits in the tile loop, so every tile gains (the instruction stream is what
+        // the softmax warps wait for most): 32 heads x 8192 causal d64 382 -> 367 us, batch 4 x 1777 92.5 ->
+        // 87 us, 64-token bitmap blocks (every tile partial), 4 heads x 2048: 30.5 -> 25.8 us.
 #pragma unroll
-        for (int c = 0; c < kTile; ++c) x[c] = (c >= c_lo && c <= c_hi) ? x[c] : -CUDART_INF_F;
+        for (int q = 0; q < 4; ++q) {
+          const int a = min(max(c_lo - 32 * q, 0), 32), b = min(max(c_hi + 1 - 32 * q, 0), 32);
+          const uint32_t keep = (b < 32 ? (1u << b) - 1u : 0xffffffffu) & ~(a < 32 ? (1u << a) - 1u : 0xffffffffu);
+#pragma unroll
+          for (int c = 0; c < 32; ++c) x[32 * q + c] = (keep >> c) & 1u ? x[32 * q + c] : -CUDART_INF_F;
+        }
       }
 
       float mx0 = fmax3(x[0], x[1], x[2]), mx1 = fmax3(x[3], x[4], x[5]);
@@ -638,7 +647,8 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
           tc_fence_after();
           const float v = need ? ex2_approx(m_ref - ms) : 1.0f;
           l *= v;
-#pragma unroll
+          // rare: kept short, so that the loop around it needs fewer instructions from the cache
+#pragma unroll 1
           for (int c = 0; c < D / 32; ++c) {
             uint32_t regs[32];
             tmem_ld32(t_o + c * 32, regs);
