@@ -24,6 +24,12 @@ struct steel_attn {
   int32_t *d_cta_begin = nullptr;
   StepPair *d_steps = nullptr;
   int32_t *d_status = nullptr;
+  SplitTile *d_split_tiles = nullptr;  // null: no query tile is split
+  int32_t *d_arrivals = nullptr;
+  size_t arrivals_bytes = 0;
+  float *d_parts = nullptr;
+  int32_t part_rows = 0;
+  bool packed = false;
   long long *d_clock_probe = nullptr;
   long long timeout_cycles = kDefaultTimeoutCycles;
   int32_t stall_cta = -1;
@@ -71,6 +77,9 @@ void free_device(steel_attn *h) {
   if (h->d_cta_begin) cudaFree(h->d_cta_begin);
   if (h->d_steps) cudaFree(h->d_steps);
   if (h->d_status) cudaFree(h->d_status);
+  if (h->d_split_tiles) cudaFree(h->d_split_tiles);
+  if (h->d_arrivals) cudaFree(h->d_arrivals);
+  if (h->d_parts) cudaFree(h->d_parts);
 }
 
 }  // namespace
@@ -78,7 +87,7 @@ void free_device(steel_attn *h) {
 namespace steel {
 
 // Encode the tensor maps for (q, k, v) unless `cache` holds them already, fill the problem fields
-// of `kp` (whose list and status pointers the caller has set) and enqueue the kernel.
+// of `kp` (whose list and status pointers and view of Q the caller has set) and enqueue the kernel.
 steel_status_t launch_with_params(const steel_attn_params_t &p, KernelParams kp, int grid, const void *q,
                                   const void *k, const void *v, void *o, float *lse, cudaStream_t stream,
                                   TensorMaps *cache) {
@@ -86,7 +95,7 @@ steel_status_t launch_with_params(const steel_attn_params_t &p, KernelParams kp,
   TensorMaps &m = cache ? *cache : local;
   if (m.q_ptr != q || m.k_ptr != k || m.v_ptr != v) {
     m.q_ptr = m.k_ptr = m.v_ptr = nullptr;
-    if (!make_map(&m.q, q, p.head_dim, p.seq_q, int64_t(p.batch) * p.heads_q) ||
+    if (!make_map(&m.q, q, p.head_dim, kp.rows_q, int64_t(p.batch) * kp.heads_q) ||
         !make_map(&m.k, k, p.head_dim, p.seq_kv, int64_t(p.batch) * p.heads_kv) ||
         !make_map(&m.v, v, p.head_dim, p.seq_kv, int64_t(p.batch) * p.heads_kv))
       return STEEL_ERR_CUDA;
@@ -96,7 +105,6 @@ steel_status_t launch_with_params(const steel_attn_params_t &p, KernelParams kp,
   }
   kp.o = o;
   kp.lse = lse;
-  kp.heads_q = p.heads_q;
   kp.heads_kv = p.heads_kv;
   kp.seq_q = p.seq_q;
   kp.seq_kv = p.seq_kv;
@@ -128,27 +136,44 @@ steel_status_t steel_attn_create(const steel_attn_params_t *params, steel_attn_t
   }
   if (prop.major != 10) return STEEL_ERR_CUDA;  // the kernel is built for sm_100a only
 
-  Plan plan;
-  try {
-    st = build_plan(params, prop.multiProcessorCount, &plan);
-  } catch (const std::bad_alloc &) {
-    return STEEL_ERR_ALLOC;
-  }
-  if (st != STEEL_OK) return st;
-
   steel_attn *h = new (std::nothrow) steel_attn();
   if (!h) return STEEL_ERR_ALLOC;
+  Plan plan;
+  for (bool spread : {true, false}) {
+    try {
+      st = build_plan(params, prop.multiProcessorCount, &plan, /*exec_stats=*/true, spread);
+    } catch (const std::bad_alloc &) {
+      st = STEEL_ERR_ALLOC;
+    }
+    if (st != STEEL_OK) {
+      delete h;
+      return st;
+    }
+    if (plan.split_tiles.empty()) break;
+    // part buffers; without memory for them the key ranges stay whole.  Rows in multiples of four: every
+    // part's buffer then starts on a 16-byte boundary.
+    h->part_rows = int32_t(std::min<int64_t>((plan_rows_q(*params, plan) + 3) / 4 * 4, kTile));
+    const size_t part_bytes = size_t(plan.n_parts) * size_t(h->part_rows) * size_t(params->head_dim + 2) * sizeof(float);
+    if (cudaMalloc(&h->d_parts, part_bytes) == cudaSuccess) break;
+    cudaGetLastError();
+    h->d_parts = nullptr;
+  }
   h->params = *params;
   h->params.mask.bitmap = nullptr;  // the caller's bitmap is not referenced after create
   h->stats = plan.stats;
   h->device = device;
   h->grid = plan.grid;
+  h->packed = plan.packed;
+  const size_t n_split = plan.split_tiles.size();
+  h->arrivals_bytes = n_split * 4 * sizeof(int32_t);
 
   const size_t n_items = plan.items.size() ? plan.items.size() : 1, n_steps = plan.steps.size() ? plan.steps.size() : 1;
   bool ok = cudaMalloc(&h->d_items, n_items * sizeof(WorkItem)) == cudaSuccess &&
             cudaMalloc(&h->d_cta_begin, plan.cta_begin.size() * sizeof(int32_t)) == cudaSuccess &&
             cudaMalloc(&h->d_steps, n_steps * sizeof(StepPair)) == cudaSuccess &&
-            cudaMalloc(&h->d_status, sizeof(int32_t)) == cudaSuccess;
+            cudaMalloc(&h->d_status, sizeof(int32_t)) == cudaSuccess &&
+            (n_split == 0 || (cudaMalloc(&h->d_split_tiles, n_split * sizeof(SplitTile)) == cudaSuccess &&
+                              cudaMalloc(&h->d_arrivals, h->arrivals_bytes) == cudaSuccess));
   if (!ok) {
     cudaGetLastError();
     free_device(h);
@@ -161,6 +186,9 @@ steel_status_t steel_attn_create(const steel_attn_params_t *params, steel_attn_t
                   cudaMemcpyHostToDevice) == cudaSuccess &&
        (plan.steps.empty() || cudaMemcpy(h->d_steps, plan.steps.data(), plan.steps.size() * sizeof(StepPair),
                                          cudaMemcpyHostToDevice) == cudaSuccess) &&
+       (n_split == 0 || (cudaMemcpy(h->d_split_tiles, plan.split_tiles.data(), n_split * sizeof(SplitTile),
+                                    cudaMemcpyHostToDevice) == cudaSuccess &&
+                         cudaMemset(h->d_arrivals, 0, h->arrivals_bytes) == cudaSuccess)) &&
        cudaMemset(h->d_status, 0, sizeof(int32_t)) == cudaSuccess && configure_kernels() == cudaSuccess &&
        cudaDeviceSynchronize() == cudaSuccess;
   if (!ok || !encode_fn()) {
@@ -186,6 +214,11 @@ steel_status_t steel_attn_run(steel_attn_t *h, const void *q, const void *k, con
   kp.cta_begin = h->d_cta_begin;
   kp.steps = h->d_steps;
   kp.status = h->d_status;
+  kp.split_tiles = h->d_split_tiles;
+  kp.parts = h->d_parts;
+  kp.part_rows = h->part_rows;
+  kp.arrivals = h->d_arrivals;
+  set_query_view(h->params, h->packed, &kp);
   kp.clock_probe = h->d_clock_probe;
   kp.timeout_cycles = h->timeout_cycles;
   kp.stall_cta = h->stall_cta;
@@ -199,7 +232,10 @@ steel_status_t steel_attn_last_status(steel_attn_t *h, void *cuda_stream) {
   if (cudaStreamSynchronize(stream) != cudaSuccess ||
       cudaMemcpy(&word, h->d_status, sizeof word, cudaMemcpyDeviceToHost) != cudaSuccess)
     return STEEL_ERR_CUDA;
-  if (word != 0 && cudaMemset(h->d_status, 0, sizeof(int32_t)) != cudaSuccess) return STEEL_ERR_CUDA;
+  // an interrupted call can leave some parts counted
+  if (word != 0 && (cudaMemset(h->d_status, 0, sizeof(int32_t)) != cudaSuccess ||
+                    (h->d_arrivals && cudaMemset(h->d_arrivals, 0, h->arrivals_bytes) != cudaSuccess)))
+    return STEEL_ERR_CUDA;
   return word == 0 ? STEEL_OK : STEEL_ERR_TIMEOUT;
 }
 

@@ -131,11 +131,14 @@ __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, Ctrl &
 
 // A work item unpacked into scalars (no indexable arrays, so everything stays in registers).
 struct Item {
-  int batch, kv_head, head0, head1, qtile0, qtile1, lo0, lo1, hi0, hi1, n_steps, kind, j0, list_off;
+  int batch, kv_head, head0, head1, qtile0, qtile1, lo0, lo1, hi0, hi1, n_steps, kind, j00, j01, split0, split1;
   __device__ __forceinline__ int lo(int s) const { return s ? lo1 : lo0; }
   __device__ __forceinline__ int hi(int s) const { return s ? hi1 : hi0; }
   __device__ __forceinline__ int head(int s) const { return s ? head1 : head0; }
   __device__ __forceinline__ int qtile(int s) const { return s ? qtile1 : qtile0; }
+  __device__ __forceinline__ int j0(int s) const { return s ? j01 : j00; }
+  __device__ __forceinline__ int split(int s) const { return s ? split1 : split0; }
+  __device__ __forceinline__ int list_off() const { return j00; }
   __device__ __forceinline__ bool active(int s) const { return head(s) >= 0 && hi(s) >= lo(s); }
 };
 
@@ -146,7 +149,7 @@ __device__ __forceinline__ Item load_item(const WorkItem *items, int k) {
   w.batch = a.x;  w.kv_head = a.y;  w.head0 = a.z;  w.head1 = a.w;
   w.qtile0 = b.x; w.qtile1 = b.y;   w.lo0 = b.z;    w.lo1 = b.w;
   w.hi0 = c.x;    w.hi1 = c.y;      w.n_steps = c.z; w.kind = c.w;
-  w.j0 = d.x;     w.list_off = d.y;
+  w.j00 = d.x;    w.j01 = d.y;      w.split0 = d.z; w.split1 = d.w;
   return w;
 }
 
@@ -155,11 +158,10 @@ __device__ __forceinline__ uint2 load_step(const Item &w, const StepPair *steps,
   uint2 e = make_uint2(0u, 0u);
   if (t >= w.n_steps) return e;
   if (w.kind == 0) {
-    const uint32_t v = uint32_t(w.j0 + t) | kEntryPresent;
-    if (w.active(0) && t >= w.lo0 && t <= w.hi0) e.x = v;
-    if (w.active(1) && t >= w.lo1 && t <= w.hi1) e.y = v;
+    if (w.active(0) && t >= w.lo0 && t <= w.hi0) e.x = uint32_t(w.j00 + t) | kEntryPresent;
+    if (w.active(1) && t >= w.lo1 && t <= w.hi1) e.y = uint32_t(w.j01 + t) | kEntryPresent;
   } else {
-    e = __ldg(reinterpret_cast<const uint2 *>(steps + w.list_off + t));
+    e = __ldg(reinterpret_cast<const uint2 *>(steps + w.list_off() + t));
   }
   return e;
 }
@@ -532,7 +534,116 @@ __device__ __forceinline__ void exp_half(const float (&x)[kTile], int base, floa
   }
 }
 
-template <int D, int kEmu>
+// ------------------------------------------------------------------------------------------------
+// Split query tiles.  Every part counts its arrival per warp (32 rows); the warp that arrives last combines
+// the parts of its rows, always in the order of the parts, so the result does not depend on who was last:
+//   O = sum_i w_i O_i / sum_i w_i l_i,  w_i = 2^(m_i - max m).
+// In fp32 throughout, as in TMEM.  Bound by the latency of its loads from L2 and, with full tiles, by what one
+// SM can read, so a batch of loads is in flight together and lanes beyond the rows in use take a share of the
+// columns.  (Loops over single parts: 500 queries on 12500 keys 103 us, as here 97 us.)
+template <int D>
+__device__ __forceinline__ float *part_buffer(const KernelParams &p, int n) {
+  return p.parts + size_t(n) * size_t(p.part_rows) * (D + 2);
+}
+
+// Columns c0, c0 + step, ... of one row (in units of four columns): kCols of them from kBatch parts at a time.
+template <int D, int kCols, int kBatch>
+__device__ __forceinline__ void combine_columns(const float4 *col, const float2 *stat, size_t stride, int part_rows,
+                                                int n_parts, int c0, int step, float m, float inv,
+                                                __nv_bfloat16 *o_row) {
+  float4 acc[kCols] = {};
+#pragma unroll 1
+  for (int i0 = 0; i0 < n_parts; i0 += kBatch) {
+    float2 ml[kBatch];
+    float4 v[kBatch][kCols];
+#pragma unroll
+    for (int b = 0; b < kBatch; ++b) {
+      const int i = min(i0 + b, n_parts - 1);
+      ml[b] = __ldcg(stat + i * (stride / 2));
+#pragma unroll
+      for (int k = 0; k < kCols; ++k)
+        v[b][k] = __ldcg(col + i * (stride / 4) + size_t(min(c0 + k * step, D / 4 - 1)) * part_rows);
+    }
+#pragma unroll
+    for (int b = 0; b < kBatch; ++b) {
+      const float w = (ml[b].y > 0.0f && i0 + b < n_parts) ? ex2_approx(ml[b].x - m) : 0.0f;
+#pragma unroll
+      for (int k = 0; k < kCols; ++k) {
+        acc[k].x = fmaf(w, v[b][k].x, acc[k].x);
+        acc[k].y = fmaf(w, v[b][k].y, acc[k].y);
+        acc[k].z = fmaf(w, v[b][k].z, acc[k].z);
+        acc[k].w = fmaf(w, v[b][k].w, acc[k].w);
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < kCols; ++k)
+    if (c0 + k * step < D / 4)
+      *reinterpret_cast<uint2 *>(o_row + (c0 + k * step) * 4) =
+          make_uint2(pack_bf16x2(acc[k].x * inv, acc[k].y * inv), pack_bf16x2(acc[k].z * inv, acc[k].w * inv));
+}
+
+template <int D>
+__device__ __forceinline__ void finish_part(const KernelParams &p, int split, int tile_row0, size_t tile_out_row,
+                                            int warp, int lane) {
+  const int used = min(32, p.rows_q - tile_row0 - warp * 32);
+  if (used <= 0) return;
+  const SplitTile tile = p.split_tiles[split >> 6];
+  int32_t *counter = p.arrivals + (split >> 6) * 4 + warp;
+  __syncwarp();
+  int before = 0;
+  if (lane == 0) before = atomic_add_acq_rel(counter, 1);
+  before = __shfl_sync(0xffffffffu, before, 0);
+  __syncwarp();
+  if (before != tile.n_parts - 1) return;
+  if (lane == 0) *counter = 0;  // for the next call
+  // `lanes` lanes share a row: lane = row + rows * share
+  const int rows = used > 16 ? 32 : used > 8 ? 16 : used > 4 ? 8 : used > 2 ? 4 : used > 1 ? 2 : 1, lanes = 32 / rows;
+  const int row = lane & (rows - 1), share = lane / rows;
+  if (row < used) {
+    const int r = warp * 32 + row;
+    const size_t stride = size_t(p.part_rows) * (D + 2);
+    const float *base = part_buffer<D>(p, tile.first);
+    const float2 *stat = reinterpret_cast<const float2 *>(base + size_t(D) * p.part_rows) + r;
+    constexpr int kBatch = 4;
+    float m = -CUDART_INF_F, l = 0.0f;
+#pragma unroll 1
+    for (int i0 = 0; i0 < tile.n_parts; i0 += kBatch) {
+      float2 ml[kBatch];
+      float top = m;
+#pragma unroll
+      for (int b = 0; b < kBatch; ++b) {
+        ml[b] = __ldcg(stat + min(i0 + b, tile.n_parts - 1) * (stride / 2));
+        if (i0 + b >= tile.n_parts) ml[b].y = 0.0f;
+        top = fmaxf(top, ml[b].x);
+      }
+      l = l > 0.0f ? l * ex2_approx(m - top) : 0.0f;
+#pragma unroll
+      for (int b = 0; b < kBatch; ++b) l += ml[b].y > 0.0f ? ml[b].y * ex2_approx(ml[b].x - top) : 0.0f;
+      m = top;
+    }
+    const float inv = l > 0.0f ? 1.0f / l : 0.0f;
+    const size_t out_row = tile_out_row + size_t(r);
+    __nv_bfloat16 *o_row = static_cast<__nv_bfloat16 *>(p.o) + out_row * D;
+    const float4 *col = reinterpret_cast<const float4 *>(base) + r;
+    // few rows: the shorter loop body, whose first pass through the instruction cache counts (a decode step with
+    // 4 rows per tile: 41.1 -> 38.9 us)
+    if (lanes <= 4) {
+#pragma unroll 1
+      for (int c0 = share; c0 < D / 4; c0 += 8 * lanes)
+        combine_columns<D, 8, 4>(col, stat, stride, p.part_rows, tile.n_parts, c0, lanes, m, inv, o_row);
+    } else {
+#pragma unroll 1
+      for (int c0 = share; c0 < D / 4; c0 += 4 * lanes)
+        combine_columns<D, 4, 4>(col, stat, stride, p.part_rows, tile.n_parts, c0, lanes, m, inv, o_row);
+    }
+    if (p.lse != nullptr && share == 0)
+      p.lse[out_row] = l > 0.0f ? 0.6931471805599453f * (m + log2f(l)) : -CUDART_INF_F;
+  }
+  __syncwarp();
+}
+
+template <int D, int kEmu, bool kSplit>
 __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, const int r) {
   using C = Cfg<D>;
   const int lane = r % 32;
@@ -552,24 +663,26 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
     const Item w = load_item(p.items, k);
     if (w.head(s) < 0) continue;
     const int row = w.qtile(s) * kTile + r;
-    const size_t out_row = (size_t(w.batch) * p.heads_q + w.head(s)) * size_t(p.seq_q) + size_t(row);
+    const size_t out_row = (size_t(w.batch) * p.heads_q + w.head(s)) * size_t(p.rows_q) + size_t(row);
     float m_ref = -CUDART_INF_F, l = 0.0f;
     const int lo = w.lo(s), hi = w.hi(s);
     const bool active = hi >= lo;
 
     // Range items: tiles f_lo .. f_hi need no element-wise mask (case ii).  List items carry it in the entry.
     int f_lo = 0, f_hi = p.seq_kv / kTile - 1;
-    if (causal) f_hi = min(f_hi, (w.qtile(s) * kTile + off + 1) / kTile - 1);
+    const int r0 = w.qtile(s) * kTile, r1 = min(r0 + kTile, p.rows_q) - 1;
+    const bool one_head = r0 / p.seq_q == r1 / p.seq_q;  // else the tile spans all positions
+    if (causal) f_hi = min(f_hi, ((one_head ? r0 % p.seq_q : 0) + off + 1) / kTile - 1);
     if (windowed) {
-      const int first = min(w.qtile(s) * kTile + kTile - 1, p.seq_q - 1) + off - p.window + 1;
+      const int first = (one_head ? r1 % p.seq_q : p.seq_q - 1) + off - p.window + 1;
       f_lo = first > 0 ? (first + kTile - 1) / kTile : 0;
     }
-    const uint32_t *entries = reinterpret_cast<const uint32_t *>(p.steps + w.list_off) + s;
+    const uint32_t *entries = reinterpret_cast<const uint32_t *>(p.steps + w.list_off()) + s;
     uint32_t next_entry = (w.kind != 0 && active) ? __ldg(entries + 2 * lo) : 0u;
 
     for (int t = lo; t <= hi; ++t) {
       // which key tile, and does it need the element-wise mask (case iii)?
-      int j = w.j0 + t;
+      int j = w.j0(s) + t;
       bool partial = j < f_lo || j > f_hi;
       uint32_t sub = 0xF;
       if (w.kind != 0) {
@@ -603,7 +716,7 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
 
       if (partial) {
         // visible columns of this row form one interval [c_lo, c_hi] of the tile
-        const int pos = row + off, jb = j * kTile;
+        const int pos = row % p.seq_q + off, jb = j * kTile;  // key position aligned with the row's query
         int c_hi = min(kTile - 1, p.seq_kv - 1 - jb), c_lo = 0;
         if (causal) c_hi = min(c_hi, pos - jb);
         if (windowed) c_lo = max(c_lo, pos - p.window + 1 - jb);
@@ -696,31 +809,52 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
       if (!ok) return;
       ++n_use;
       tc_fence_after();
-      const float inv = l > 0.0f ? 1.0f / l : 0.0f;
+      const bool valid = row < p.rows_q;
+      const int split = kSplit ? w.split(s) : -1;
+      if (kSplit && split >= 0) {
+        // one of several key ranges of this query tile: leave O and (m, l) for the part that ends last
+        float *part = part_buffer<D>(p, p.split_tiles[split >> 6].first + (split & 63));
 #pragma unroll
-      for (int c = 0; c < D / 32; ++c) {
-        uint32_t regs[32];
-        tmem_ld32(t_o + c * 32, regs);
-        tc_wait_ld();
-        if (row < p.seq_q) {
-          uint4 *dst = reinterpret_cast<uint4 *>(o_base + out_row * D + c * 32);
+        for (int c = 0; c < D / 32; ++c) {
+          uint32_t regs[32];
+          tmem_ld32(t_o + c * 32, regs);
+          tc_wait_ld();
+          if (valid) {
+            uint4 *dst = reinterpret_cast<uint4 *>(part) + size_t(c) * 8 * p.part_rows + r;
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            uint4 v;
-            v.x = pack_bf16x2(__uint_as_float(regs[8 * i + 0]) * inv, __uint_as_float(regs[8 * i + 1]) * inv);
-            v.y = pack_bf16x2(__uint_as_float(regs[8 * i + 2]) * inv, __uint_as_float(regs[8 * i + 3]) * inv);
-            v.z = pack_bf16x2(__uint_as_float(regs[8 * i + 4]) * inv, __uint_as_float(regs[8 * i + 5]) * inv);
-            v.w = pack_bf16x2(__uint_as_float(regs[8 * i + 6]) * inv, __uint_as_float(regs[8 * i + 7]) * inv);
-            dst[i] = v;
+            for (int i = 0; i < 8; ++i)
+              dst[i * p.part_rows] = make_uint4(regs[4 * i], regs[4 * i + 1], regs[4 * i + 2], regs[4 * i + 3]);
           }
         }
+        if (valid) reinterpret_cast<float2 *>(part + size_t(D) * p.part_rows)[r] = make_float2(m_ref, l);
+      } else {
+        const float inv = l > 0.0f ? 1.0f / l : 0.0f;
+#pragma unroll
+        for (int c = 0; c < D / 32; ++c) {
+          uint32_t regs[32];
+          tmem_ld32(t_o + c * 32, regs);
+          tc_wait_ld();
+          if (valid) {
+            uint4 *dst = reinterpret_cast<uint4 *>(o_base + out_row * D + c * 32);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              uint4 v;
+              v.x = pack_bf16x2(__uint_as_float(regs[8 * i + 0]) * inv, __uint_as_float(regs[8 * i + 1]) * inv);
+              v.y = pack_bf16x2(__uint_as_float(regs[8 * i + 2]) * inv, __uint_as_float(regs[8 * i + 3]) * inv);
+              v.z = pack_bf16x2(__uint_as_float(regs[8 * i + 4]) * inv, __uint_as_float(regs[8 * i + 5]) * inv);
+              v.w = pack_bf16x2(__uint_as_float(regs[8 * i + 6]) * inv, __uint_as_float(regs[8 * i + 7]) * inv);
+              dst[i] = v;
+            }
+          }
+        }
+        if (p.lse != nullptr && valid)
+          p.lse[out_row] = l > 0.0f ? 0.6931471805599453f * (m_ref + log2f(l)) : -CUDART_INF_F;
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&ctrl.o_empty[s]);
-      if (p.lse != nullptr && row < p.seq_q)
-        p.lse[out_row] = l > 0.0f ? 0.6931471805599453f * (m_ref + log2f(l)) : -CUDART_INF_F;
-    } else if (row < p.seq_q) {
+      if (kSplit && split >= 0) finish_part<D>(p, split, w.qtile(s) * kTile, out_row - size_t(r), r / 32, lane);
+    } else if (row < p.rows_q) {
       // no key tile is visible to this query tile
       uint4 *dst = reinterpret_cast<uint4 *>(o_base + out_row * D);
 #pragma unroll
@@ -731,7 +865,7 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
 }
 
 // ------------------------------------------------------------------------------------------------
-template <int D, int kEmu>
+template <int D, int kEmu, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
 steel_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                   const __grid_constant__ CUtensorMap map_v, const __grid_constant__ KernelParams p) {
@@ -779,7 +913,7 @@ steel_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 
   if (warp < 8) {
     setmaxnreg_inc<kRegsSoftmax>();
-    softmax_role<D, kEmu>(p, ctrl, warp / 4, threadIdx.x % kTile);
+    softmax_role<D, kEmu, kSplit>(p, ctrl, warp / 4, threadIdx.x % kTile);
   } else {
     setmaxnreg_dec<kRegsOther>();
     if (warp == kProducerWarp) {
@@ -797,16 +931,24 @@ steel_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 
 namespace {
 
+// The build that combines split query tiles is a kernel of its own, so that its code does not lengthen the
+// instruction stream of the others.
 template <int D, int kEmu>
 cudaError_t configure_one() {
-  return cudaFuncSetAttribute(steel_attn_kernel<D, kEmu>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const cudaError_t e = cudaFuncSetAttribute(steel_attn_kernel<D, kEmu, false>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D>::kSmemBytes);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(steel_attn_kernel<D, kEmu, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               Cfg<D>::kSmemBytes);
 }
 
 template <int D, int kEmu>
 void launch_one(const CUtensorMap &map_q, const CUtensorMap &map_k, const CUtensorMap &map_v,
                 const KernelParams &params, int grid, cudaStream_t stream) {
-  steel_attn_kernel<D, kEmu><<<grid, kThreads, Cfg<D>::kSmemBytes, stream>>>(map_q, map_k, map_v, params);
+  if (params.split_tiles)
+    steel_attn_kernel<D, kEmu, true><<<grid, kThreads, Cfg<D>::kSmemBytes, stream>>>(map_q, map_k, map_v, params);
+  else
+    steel_attn_kernel<D, kEmu, false><<<grid, kThreads, Cfg<D>::kSmemBytes, stream>>>(map_q, map_k, map_v, params);
 }
 
 template <int D>

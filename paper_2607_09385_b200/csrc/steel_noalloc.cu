@@ -108,12 +108,12 @@ extern "C" steel_status_t steel_attn_run_noalloc(const steel_attn_params_t *para
     cudaGetLastError();
     return STEEL_ERR_CUDA;
   }
-  KernelParams kp;
+  KernelParams kp{};  // no split query tiles: their buffers have no room in the array
   kp.items = reinterpret_cast<const WorkItem *>(base + kOffItems);
   kp.cta_begin = reinterpret_cast<const int32_t *>(base + kOffCtaBegin);
   kp.steps = reinterpret_cast<const StepPair *>(base + kOffSteps);
   kp.status = reinterpret_cast<int32_t *>(base + kOffStatus);
-  kp.clock_probe = nullptr;
+  set_query_view(*params, plan.packed, &kp);
   kp.timeout_cycles = kDefaultTimeoutCycles;
   kp.stall_cta = -1;
   st = launch_with_params(*params, kp, plan.grid, q, k, v, o, lse, stream, nullptr);

@@ -29,13 +29,21 @@ struct WorkItem {
   int32_t lo[2];
   int32_t hi[2];
   int32_t n_steps;
-  int32_t kind;      // 0: range (key tile of step t is j0 + t for both slots), 1: list
-  int32_t j0;        // range kind
-  int32_t list_off;  // list kind: index of the item's first StepPair
-  int32_t cost;      // executed tiles
-  int32_t pad;
+  int32_t kind;      // 0: range (key tile of step t is j0[s] + t for slot s), 1: list
+  int32_t j0[2];     // range kind; list kind: j0[0] is the index of the item's first StepPair
+  int32_t split[2];  // slot s holds one of several key ranges of its query tile: split_code; else -1
 };
 static_assert(sizeof(WorkItem) == 64, "WorkItem layout");
+
+// A query tile whose key tiles are cut over several items: each part leaves its unnormalised O and its
+// row statistics in a buffer of its own, and the part that finishes last combines them.
+constexpr int kMaxParts = 64;
+struct SplitTile {
+  int32_t first;    // buffer of part 0; the parts' buffers are consecutive
+  int32_t n_parts;
+};
+constexpr int32_t split_code(int32_t tile, int32_t part) { return tile << 6 | part; }
+static_assert(kMaxParts <= 64, "split_code keeps the part in 6 bits");
 
 // Entries of both slots for one step of a list-kind item.
 struct StepPair {
@@ -49,7 +57,13 @@ struct KernelParams {
   void *o;                   // bf16 [batch, heads_q, seq_q, head_dim]
   float *lse;                // fp32 [batch, heads_q, seq_q] or null
   int32_t *status;           // device status word (0 ok, else STEEL_ERR_TIMEOUT)
-  int32_t heads_q, heads_kv, seq_q, seq_kv;
+  const SplitTile *split_tiles;  // null: no query tile is split
+  float *parts;              // per part: O as float4 [head_dim / 4][part_rows], then (m, l) [part_rows]
+  int32_t part_rows;         // rows of a query tile that can be used (128, or those of a shorter matrix), a multiple of 4
+  int32_t *arrivals;         // per split tile and row quarter: parts finished; zero between calls
+  // Q as [batch][heads_q][rows_q][head_dim]: `heads_q` matrices of rows_q = seq_q rows or, where a query
+  // tile holds rows of several heads of a group, heads_kv matrices of group * seq_q rows
+  int32_t heads_q, heads_kv, rows_q, seq_q, seq_kv;
   uint32_t mask_flags;
   int32_t window;            // clamped to int32 range
   float scale_log2;          // scale * log2(e)

@@ -40,6 +40,14 @@ struct Geom {
   }
 };
 
+// First and last query position in tile I of a matrix of `rows` rows whose row r holds position r mod seq_q.
+void tile_positions(int64_t seq_q, int64_t rows, int64_t I, int64_t *i0, int64_t *i1) {
+  const int64_t r0 = I * kTile, r1 = std::min<int64_t>(r0 + kTile, rows) - 1;
+  const bool one_head = r0 / seq_q == r1 / seq_q;
+  *i0 = one_head ? r0 % seq_q : 0;
+  *i1 = one_head ? r1 % seq_q : seq_q - 1;
+}
+
 struct Ctx {
   const steel_attn_params_t *p;
   Geom g;
@@ -60,7 +68,7 @@ struct Ctx {
     j0 = J * size;
     j1 = std::min<int64_t>(j0 + size - 1, p->seq_kv - 1);
   }
-  // Entry of kernel tile (I, J) for head h, or 0 if the tile is fully masked (case i).
+  // Bitmap masks: entry of kernel tile (I, J) for head h, or 0 if the tile is fully masked (case i).
   uint32_t entry(int h, int64_t I, int64_t J) const {
     int64_t i0, i1, j0, j1;
     rows(I, kTile, i0, i1);
@@ -68,10 +76,7 @@ struct Ctx {
     bool ragged = (j1 - j0 + 1) < kTile;
     uint32_t sub = 0xF;
     bool kept, full;
-    if (!bitmap) {
-      kept = g.any_visible(i0, i1, j0, j1);
-      full = g.all_visible(i0, i1, j0, j1);
-    } else if (bq == kTile) {
+    if (bq == kTile) {
       kept = bit(h, I, J) && g.any_visible(i0, i1, j0, j1);
       full = g.all_visible(i0, i1, j0, j1);
     } else {  // 64-token blocks: four sub-blocks TL, TR, BL, BR
@@ -98,13 +103,190 @@ struct Ctx {
   }
 };
 
-struct Task {  // one query tile of one head
+// Key tiles lo .. hi (empty if lo > hi) that query tile I of a matrix of `rows` rows sees under the causal
+// and window terms; `rows` is seq_q, or a multiple of it where the matrix holds several heads.
+void key_range(const Ctx &c, int64_t rows, int64_t I, int64_t *lo, int64_t *hi) {
+  int64_t i0, i1;
+  tile_positions(c.p->seq_q, rows, I, &i0, &i1);
+  const int64_t p0 = i0 + c.g.off, p1 = i1 + c.g.off;
+  *hi = c.g.causal ? std::min<int64_t>(c.tkv128 - 1, p1 >= 0 ? p1 / kTile : -1) : c.tkv128 - 1;
+  *lo = 0;
+  if (c.g.windowed) {
+    const int64_t first_key = p0 - c.g.window + 1;
+    *lo = first_key > 0 ? first_key / kTile : 0;
+  }
+  auto seen = [&](int64_t J) {
+    return c.g.any_visible(i0, i1, J * kTile, std::min<int64_t>(J * kTile + kTile, c.p->seq_kv) - 1);
+  };
+  while (*lo <= *hi && !seen(*lo)) ++*lo;
+  while (*hi >= *lo && !seen(*hi)) --*hi;
+}
+
+struct Task {  // one query tile of one head (packed: of one group of heads)
   int h;
   int64_t I;
   int64_t jlo = 0, jhi = -1;      // range kind
   std::vector<uint32_t> entries;  // list kind
   int64_t count() const { return entries.empty() ? jhi - jlo + 1 : int64_t(entries.size()); }
 };
+
+bool slot_used(const WorkItem &w, int s) { return w.head[s] >= 0 && w.hi[s] >= w.lo[s]; }
+
+double step_cost(const WorkItem &w) { return slot_used(w, 0) && slot_used(w, 1) ? 1.0 : kSingleStep; }
+
+// Load of the busiest CTA, in steps of two slots, with the longest item first to the least loaded CTA.
+double makespan(const std::vector<Draft> &drafts, int num_ctas) {
+  std::vector<double> cost;
+  for (const Draft &d : drafts) cost.push_back(step_cost(d.w) * d.w.n_steps + kItemOverheadSteps);
+  std::sort(cost.begin(), cost.end(), std::greater<double>());
+  std::priority_queue<double, std::vector<double>, std::greater<double>> load;
+  for (int n = 0; n < num_ctas; ++n) load.push(0.0);
+  double most = 0.0;
+  for (double x : cost) {
+    x += load.top();
+    load.pop();
+    load.push(x);
+    most = std::max(most, x);
+  }
+  return most;
+}
+
+// Steps [t0, t1) of `d`.  A draft of one query tile becomes a piece whose slots walk the two halves of the
+// range, so that one slot's softmax runs beside the other's products.
+Draft cut_piece(const Draft &d, int t0, int t1) {
+  Draft r;
+  r.w = d.w;
+  r.group = d.group;
+  WorkItem &w = r.w;
+  if (!slot_used(d.w, 1)) {
+    const int n0 = (t1 - t0 + 1) / 2, n1 = t1 - t0 - n0;
+    w.head[1] = n1 ? d.w.head[0] : -1;
+    w.qtile[1] = d.w.qtile[0];
+    w.lo[0] = 0;
+    w.hi[0] = n0 - 1;
+    w.lo[1] = n1 ? 0 : 1;
+    w.hi[1] = n1 ? n1 - 1 : 0;
+    w.n_steps = n0;
+    if (d.w.kind == 0) {
+      w.j0[0] = d.w.j0[0] + t0;
+      w.j0[1] = d.w.j0[0] + t0 + n0;
+    } else {
+      for (int t = 0; t < n0; ++t)
+        r.list.push_back(StepPair{{d.list[t0 + t].e[0], t < n1 ? d.list[t0 + n0 + t].e[0] : 0u}});
+    }
+    return r;
+  }
+  int n = 0;
+  for (int s = 0; s < 2; ++s) {  // a slot absent from these steps drops out; the other one is then slot 0
+    const int lo = std::max(d.w.lo[s], t0), hi = std::min(d.w.hi[s], t1 - 1);
+    if (lo > hi) continue;
+    w.head[n] = d.w.head[s];
+    w.qtile[n] = d.w.qtile[s];
+    w.lo[n] = lo - t0;
+    w.hi[n] = hi - t0;
+    if (d.w.kind == 0) w.j0[n] = d.w.j0[s] + t0;
+    for (int t = t0; d.w.kind == 1 && t < t1; ++t) {
+      if (n == 0) r.list.push_back(StepPair{{d.list[t].e[s], 0u}});
+      else r.list[t - t0].e[1] = d.list[t].e[s];
+    }
+    ++n;
+  }
+  if (n == 1) {
+    w.head[1] = -1;
+    w.lo[1] = 1;
+    w.hi[1] = 0;
+  }
+  w.n_steps = std::max(w.hi[0], n == 2 ? w.hi[1] : 0) + 1;
+  return r;
+}
+
+// Cut the drafts' steps, in order, into one share of at most `quota` per CTA (a piece of a draft at either
+// end of a share) and number the parts of the query tiles that were cut.  False if the shares do not suffice.
+bool cut_into_shares(const std::vector<Draft> &drafts, int num_ctas, double quota, double fill,
+                     std::vector<Draft> *pieces, Plan *plan) {
+  const double overhead = kPieceOverheadSteps + part_write_steps(fill);
+  int cta = 0;
+  double left = quota;
+  auto next_share = [&] {
+    ++cta;
+    left = quota;
+  };
+  for (const Draft &d : drafts) {
+    const bool one = !slot_used(d.w, 1);
+    const double w = one ? 0.5 : 1.0;
+    const int n = d.w.n_steps, per_step = one ? 1 : 2;
+    // at most kMaxParts parts of one query tile (two per piece)
+    const int least = std::max<int>(min_piece_tiles(fill) / per_step, (n + kMaxParts / 2 - 1) / (kMaxParts / 2));
+    const size_t first = pieces->size();
+    int t = 0;
+    do {
+      int take = std::max(0, int((left - overhead) / w));
+      if (take < std::min(least, n - t) && left < quota) {  // the rest of this share is too short
+        next_share();
+        continue;
+      }
+      take = std::max(take, least);
+      if (n - t - take < least) take = n - t;
+      if (cta >= num_ctas) return false;
+      // a tile with few rows in use is worth two parts even within one CTA
+      const bool whole = take == n && !(one && fill <= 0.25 && n >= 2 * least);
+      pieces->push_back(whole ? d : cut_piece(d, t, t + take));
+      pieces->back().cta = cta;
+      left -= (whole && one ? kSingleStep : w) * take + (whole ? kPieceOverheadSteps : overhead);
+      if (left <= overhead) next_share();
+      t += take;
+    } while (t < n);
+    if (pieces->size() == first + 1 && !(one && slot_used(pieces->back().w, 1))) continue;
+    // the parts of each query tile are all slots of its pieces that hold it
+    for (int s = 0; s < (one ? 1 : 2); ++s) {
+      SplitTile tile{plan->n_parts, 0};
+      const int32_t id = int32_t(plan->split_tiles.size());
+      int32_t *only = nullptr;
+      for (size_t k = first; k < pieces->size(); ++k)
+        for (int u = 0; u < 2; ++u) {
+          WorkItem &x = (*pieces)[k].w;
+          if (slot_used(x, u) && x.head[u] == d.w.head[s] && x.qtile[u] == d.w.qtile[s]) {
+            only = &x.split[u];
+            *only = split_code(id, tile.n_parts++);
+          }
+        }
+      if (tile.n_parts > 1) {
+        plan->split_tiles.push_back(tile);
+        plan->n_parts += tile.n_parts;
+      } else if (only) {
+        *only = -1;
+      }
+    }
+  }
+  return true;
+}
+
+// The same with the smallest share that works, to 3 %.  Returns the load of the busiest CTA, or infinity where
+// nothing was cut.
+double cut_over_ctas(const std::vector<Draft> &drafts, int num_ctas, double fill, std::vector<Draft> *pieces,
+                     Plan *plan) {
+  double work = 0.0;
+  size_t live = 0;
+  for (const Draft &d : drafts) {
+    work += (slot_used(d.w, 1) ? 1.0 : 0.5) * d.w.n_steps;
+    live += d.w.n_steps > 0;
+  }
+  double quota = (work + kPieceOverheadSteps * double(std::max<size_t>(live, num_ctas))) / num_ctas;
+  while (!cut_into_shares(drafts, num_ctas, quota, fill, pieces, plan)) {
+    quota *= 1.03;
+    pieces->clear();
+    plan->split_tiles.clear();
+    plan->n_parts = 0;
+  }
+  if (plan->split_tiles.empty()) return std::numeric_limits<double>::infinity();
+  std::vector<double> load(num_ctas, 0.0);
+  int most_parts = 0;
+  for (const Draft &d : *pieces)
+    load[d.cta] += step_cost(d.w) * d.w.n_steps + kPieceOverheadSteps +
+                   (d.w.split[0] >= 0 || d.w.split[1] >= 0 ? part_write_steps(fill) : 0.0);
+  for (const SplitTile &t : plan->split_tiles) most_parts = std::max(most_parts, t.n_parts);
+  return *std::max_element(load.begin(), load.end()) + combine_steps(fill, most_parts);
+}
 
 }  // namespace
 
@@ -130,7 +312,7 @@ steel_status_t validate_params(const steel_attn_params_t *p) {
   return STEEL_OK;
 }
 
-steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan, bool exec_stats) {
+steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan, bool exec_stats, bool spread) {
   steel_status_t st = validate_params(p);
   if (st != STEEL_OK) return st;
   const int policy = p->policy;
@@ -148,10 +330,15 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
   c.tqb = (p->seq_q + c.bq - 1) / c.bq;
   c.tkvb = (p->seq_kv + c.bkv - 1) / c.bkv;
   c.words = (c.tkvb + 31) / 32;
-  const int G = p->heads_q / p->heads_kv;
+  int G = p->heads_q / p->heads_kv;  // heads (matrices of Q) that share a KV head
+  int heads = p->heads_q;
+  spread = spread && policy == 0;
 
   plan->items.clear();
   plan->steps.clear();
+  plan->split_tiles.clear();
+  plan->n_parts = 0;
+  plan->packed = false;
   plan->cta_begin.clear();
   steel_attn_stats_t &s = plan->stats;
   s = steel_attn_stats_t{};
@@ -189,8 +376,31 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
   }
 
   // ---- per (head, query tile) executed key tiles
-  std::vector<std::vector<Task>> tasks(p->heads_q);  // [h][I]
-  for (int h = 0; h < p->heads_q; ++h) {
+  // Heads of a group lie one behind the other in Q, O and LSE, so their rows form one matrix of G * seq_q
+  // rows.  Few queries per head leave most of a head's last tile empty (a decode step: 127 of 128 rows);
+  // tiles over that matrix are then fewer.  A tile that holds the end of one head and the start of the next
+  // spans all positions, which costs key tiles under a causal mask: taken only where the total is smaller.
+  if (spread && !c.bitmap && G > 1) {
+    auto executed = [&](bool packed) {
+      const int64_t rows = packed ? int64_t(G) * p->seq_q : p->seq_q;
+      int64_t n = 0, lo, hi;
+      for (int64_t I = 0; I * kTile < rows; ++I) {
+        key_range(c, rows, I, &lo, &hi);
+        n += std::max<int64_t>(0, hi - lo + 1);
+      }
+      return packed ? n : n * G;
+    };
+    // with more than 8 tiles per head a shared tile saves less than one in eight
+    if (c.tq128 <= 8 && executed(true) < executed(false)) {
+      plan->packed = true;
+      c.tq128 = (int64_t(G) * p->seq_q + kTile - 1) / kTile;
+      heads = p->heads_kv;
+      G = 1;
+    }
+  }
+  const int64_t rows_q = plan_rows_q(*p, *plan);
+  std::vector<std::vector<Task>> tasks(heads);  // [h][I]
+  for (int h = 0; h < heads; ++h) {
     tasks[h].resize(c.tq128);
     for (int64_t I = 0; I < c.tq128; ++I) {
       Task &t = tasks[h][I];
@@ -206,30 +416,14 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
         t.jhi = tasks[0][I].jhi;
       } else {
         // kept key tiles of a row of tiles form one contiguous range under causal / window masks
-        int64_t i0, i1;
-        c.rows(I, kTile, i0, i1);
-        int64_t p0 = i0 + c.g.off, p1 = i1 + c.g.off;
-        int64_t hi = c.g.causal ? std::min<int64_t>(c.tkv128 - 1, p1 >= 0 ? p1 / kTile : -1) : c.tkv128 - 1;
-        int64_t lo = 0;
-        if (c.g.windowed) {
-          int64_t first_key = p0 - c.g.window + 1;
-          lo = first_key > 0 ? first_key / kTile : 0;
-        }
-        while (lo <= hi && !c.entry(0, I, lo)) ++lo;
-        while (hi >= lo && !c.entry(0, I, hi)) --hi;
-        t.jlo = lo;
-        t.jhi = hi;
+        key_range(c, rows_q, I, &t.jlo, &t.jhi);
       }
     }
   }
 
   // ---- work items: pair query tiles that can share K/V loads
-  struct Draft {
-    WorkItem w;
-    std::vector<StepPair> list;
-    int group;
-  };
   std::vector<Draft> drafts;
+  bool pair = true;
   auto finish_range = [&](const Task *a, const Task *b, int batch, int g) {
     Draft d{};
     d.group = g;
@@ -241,7 +435,8 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
     w.qtile[0] = int32_t(a->I);
     w.head[1] = b ? b->h : -1;
     w.qtile[1] = b ? int32_t(b->I) : 0;
-    w.j0 = int32_t(a->jlo);
+    w.j0[0] = w.j0[1] = int32_t(a->jlo);
+    w.split[0] = w.split[1] = -1;
     w.lo[0] = 0;
     w.hi[0] = int32_t(a->jhi - a->jlo);
     w.lo[1] = 1;
@@ -251,7 +446,6 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
       w.hi[1] = int32_t(b->jhi - a->jlo);
     }
     w.n_steps = std::max(w.hi[0], w.hi[1]) + 1;
-    w.cost = int32_t(a->count() + (b ? b->count() : 0));
     drafts.push_back(std::move(d));
   };
   auto finish_list = [&](const Task *a, const Task *b, int batch, int g) {
@@ -265,6 +459,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
     w.qtile[0] = int32_t(a->I);
     w.head[1] = b ? b->h : -1;
     w.qtile[1] = b ? int32_t(b->I) : 0;
+    w.split[0] = w.split[1] = -1;
     size_t na = a->entries.size(), nb = b ? b->entries.size() : 0;
     w.lo[0] = 0;
     w.hi[0] = int32_t(na) - 1;
@@ -296,7 +491,6 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
     }
     for (size_t t = 0; t < size_t(w.n_steps); ++t)
       d.list.push_back(StepPair{{t < na ? ea[t] : 0u, t < nb ? eb[t] : 0u}});
-    w.cost = int32_t(na + nb);
     drafts.push_back(std::move(d));
   };
   auto empty_item = [&](const Task *a, int batch, int g) {  // no visible key: rows get O = 0, LSE = -inf
@@ -309,6 +503,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
     w.head[0] = a->h;
     w.qtile[0] = int32_t(a->I);
     w.head[1] = -1;
+    w.split[0] = w.split[1] = -1;
     w.lo[0] = 0;
     w.hi[0] = -1;
     w.lo[1] = 1;
@@ -317,62 +512,107 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
     drafts.push_back(std::move(d));
   };
 
-  for (int batch = 0; batch < p->batch; ++batch) {
-    for (int g = 0; g < p->heads_kv; ++g) {
-      std::vector<const Task *> live;
-      for (int h = g * G; h < (g + 1) * G; ++h)
-        for (int64_t I = 0; I < c.tq128; ++I) {
-          const Task *t = &tasks[h][I];
-          if (t->count() <= 0) empty_item(t, batch, g);
-          else live.push_back(t);
-        }
-      if (c.bitmap) {
-        // similar lengths pair best: both tiles of an item then finish together
-        std::stable_sort(live.begin(), live.end(), [](const Task *a, const Task *b) { return a->count() > b->count(); });
-        // among the next few tasks of similar length, take the partner with the most key tiles in common
-        std::vector<bool> used(live.size(), false);
-        for (size_t n = 0; n < live.size(); ++n) {
-          if (used[n]) continue;
-          used[n] = true;
-          size_t best = live.size(), seen = 0;
-          int64_t best_common = 0;
-          for (size_t m = n + 1; m < live.size() && seen < kPartnerWindow; ++m) {
-            if (used[m]) continue;
-            ++seen;
-            int64_t common = 0;
-            size_t ia = 0, ib = 0;
-            const std::vector<uint32_t> &ea = live[n]->entries, &eb = live[m]->entries;
-            while (ia < ea.size() && ib < eb.size()) {
-              const uint32_t ta = ea[ia] & kEntryTileMask, tb = eb[ib] & kEntryTileMask;
-              if (ta == tb) { ++common; ++ia; ++ib; }
-              else if (ta < tb) ++ia;
-              else ++ib;
+  auto build_drafts = [&] {
+    drafts.clear();
+    for (int batch = 0; batch < p->batch; ++batch) {
+      for (int g = 0; g < p->heads_kv; ++g) {
+        std::vector<const Task *> live;
+        for (int h = g * G; h < (g + 1) * G; ++h)
+          for (int64_t I = 0; I < c.tq128; ++I) {
+            const Task *t = &tasks[h][I];
+            if (t->count() <= 0) empty_item(t, batch, g);
+            else live.push_back(t);
+          }
+        if (c.bitmap) {
+          // similar lengths pair best: both tiles of an item then finish together
+          std::stable_sort(live.begin(), live.end(), [](const Task *a, const Task *b) { return a->count() > b->count(); });
+          // among the next few tasks of similar length, take the partner with the most key tiles in common
+          std::vector<bool> used(live.size(), false);
+          for (size_t n = 0; n < live.size(); ++n) {
+            if (used[n]) continue;
+            used[n] = true;
+            size_t best = live.size(), seen = 0;
+            int64_t best_common = 0;
+            for (size_t m = n + 1; pair && m < live.size() && seen < kPartnerWindow; ++m) {
+              if (used[m]) continue;
+              ++seen;
+              int64_t common = 0;
+              size_t ia = 0, ib = 0;
+              const std::vector<uint32_t> &ea = live[n]->entries, &eb = live[m]->entries;
+              while (ia < ea.size() && ib < eb.size()) {
+                const uint32_t ta = ea[ia] & kEntryTileMask, tb = eb[ib] & kEntryTileMask;
+                if (ta == tb) { ++common; ++ia; ++ib; }
+                else if (ta < tb) ++ia;
+                else ++ib;
+              }
+              // a step with one idle slot costs far more than a shared load saves
+              const int64_t score = common - 16 * (live[n]->count() - live[m]->count());
+              if (score > best_common || best == live.size()) { best_common = score; best = m; }
             }
-            // a step with one idle slot costs far more than a shared load saves
-            const int64_t score = common - 16 * (live[n]->count() - live[m]->count());
-            if (score > best_common || best == live.size()) { best_common = score; best = m; }
+            if (best < live.size()) used[best] = true;
+            finish_list(live[n], best < live.size() ? live[best] : nullptr, batch, g);
           }
-          if (best < live.size()) used[best] = true;
-          finish_list(live[n], best < live.size() ? live[best] : nullptr, batch, g);
-        }
-      } else if (G % 2 == 0) {
-        // two query heads of the group on the same query tile: identical key ranges
-        for (int h = g * G; h < (g + 1) * G; h += 2)
-          for (int64_t I = 0; I < c.tq128; ++I)
-            if (tasks[h][I].count() > 0) finish_range(&tasks[h][I], &tasks[h + 1][I], batch, g);
-      } else {
-        // adjacent query tiles of one head: ranges differ by at most one tile at each end
-        for (int h = g * G; h < (g + 1) * G; ++h) {
-          int64_t I = 0;
-          while (I < c.tq128) {
-            const Task *a = &tasks[h][I];
-            if (a->count() <= 0) { ++I; continue; }
-            const Task *b = (I + 1 < c.tq128 && tasks[h][I + 1].count() > 0) ? &tasks[h][I + 1] : nullptr;
-            if (b && (b->jlo < a->jlo || b->jlo > a->jhi + 1)) b = nullptr;
-            finish_range(a, b, batch, g);
-            I += b ? 2 : 1;
+        } else if (!pair) {
+          for (const Task *t : live) finish_range(t, nullptr, batch, g);
+        } else if (G % 2 == 0) {
+          // two query heads of the group on the same query tile: identical key ranges
+          for (int h = g * G; h < (g + 1) * G; h += 2)
+            for (int64_t I = 0; I < c.tq128; ++I)
+              if (tasks[h][I].count() > 0) finish_range(&tasks[h][I], &tasks[h + 1][I], batch, g);
+        } else {
+          // adjacent query tiles of one head: ranges differ by at most one tile at each end
+          for (int h = g * G; h < (g + 1) * G; ++h) {
+            int64_t I = 0;
+            while (I < c.tq128) {
+              const Task *a = &tasks[h][I];
+              if (a->count() <= 0) { ++I; continue; }
+              const Task *b = (I + 1 < c.tq128 && tasks[h][I + 1].count() > 0) ? &tasks[h][I + 1] : nullptr;
+              if (b && (b->jlo < a->jlo || b->jlo > a->jhi + 1)) b = nullptr;
+              finish_range(a, b, batch, g);
+              I += b ? 2 : 1;
+            }
           }
         }
+      }
+    }
+  };
+  build_drafts();
+
+  // ---- few items: one query tile per item, or key ranges cut over all CTAs, where that ends earlier.
+  // (Many items spread evenly by themselves: the paired plan stands where its busiest CTA has at most a
+  // tenth more than the mean.)  Kernel time, paired -> chosen plan: 500 queries on 12500 keys, 32/8 heads,
+  // 161 -> 96 us (cut); a decode step of batch 8 on 6001 keys, 32/8 heads, 82 -> 39 us (packed and cut);
+  // 12 heads x 512 d64 11.8 -> 9.6 us, 16/4 heads x 2048 d128 35.2 -> 30.7 us (one query tile per item).
+  if (spread && drafts.size() < size_t(8 * num_ctas)) {
+    const double fill = double(std::min<int64_t>(rows_q, kTile)) / kTile;
+    double work = 0.0;
+    for (const Draft &d : drafts) work += step_cost(d.w) * d.w.n_steps + kItemOverheadSteps;
+    const double paired = makespan(drafts, num_ctas);
+    if (paired > 1.1 * work / num_ctas) {
+      std::vector<Draft> paired_drafts;
+      paired_drafts.swap(drafts);
+      double best = 0.95 * paired;
+      pair = false;
+      build_drafts();
+      std::vector<Draft> singles;
+      singles.swap(drafts);
+      for (const std::vector<Draft> *from : {&paired_drafts, &singles}) {
+        Plan cut;
+        std::vector<Draft> pieces;
+        const double t = cut_over_ctas(*from, num_ctas, fill, &pieces, &cut);
+        if (t < best) {
+          best = t;
+          drafts.swap(pieces);
+          plan->split_tiles.swap(cut.split_tiles);
+          plan->n_parts = cut.n_parts;
+        }
+      }
+      if (makespan(singles, num_ctas) < best) {
+        drafts.swap(singles);
+        plan->split_tiles.clear();
+        plan->n_parts = 0;
+      } else if (drafts.empty()) {
+        drafts.swap(paired_drafts);
       }
     }
   }
@@ -396,7 +636,12 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
   int grid = int(std::min<size_t>(size_t(num_ctas), std::max<size_t>(drafts.size(), 1)));
   std::vector<std::vector<int>> per_cta(grid);
   std::vector<int64_t> load(grid, 0);
-  if (policy == 0) {
+  if (!plan->split_tiles.empty()) {
+    grid = num_ctas;
+    per_cta.resize(grid);
+    load.resize(grid, 0);
+    for (size_t id = 0; id < drafts.size(); ++id) per_cta[drafts[id].cta].push_back(int(id));
+  } else if (policy == 0) {
     // greedy longest-processing-time: next item goes to the least loaded CTA
     typedef std::pair<int64_t, int> Slot;
     std::priority_queue<Slot, std::vector<Slot>, std::greater<Slot>> heap;
@@ -433,7 +678,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
     for (int id : per_cta[cta]) {
       Draft &d = drafts[id];
       if (d.w.kind == 1) {
-        d.w.list_off = int32_t(plan->steps.size());
+        d.w.j0[0] = int32_t(plan->steps.size());
         plan->steps.insert(plan->steps.end(), d.list.begin(), d.list.end());
       }
       plan->items.push_back(d.w);
@@ -462,15 +707,25 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
   return STEEL_OK;
 }
 
+int64_t plan_rows_q(const steel_attn_params_t &p, const Plan &plan) {
+  return plan.packed ? int64_t(p.heads_q / p.heads_kv) * p.seq_q : p.seq_q;
+}
+
+void set_query_view(const steel_attn_params_t &p, bool packed, KernelParams *kp) {
+  kp->heads_q = packed ? p.heads_kv : p.heads_q;
+  kp->rows_q = packed ? p.heads_q / p.heads_kv * p.seq_q : p.seq_q;
+}
+
 // Entry of slot `slot` at step t of an item, as the kernel derives it.
 uint32_t item_entry(const Plan &plan, const WorkItem &w, int slot, int t, const steel_attn_params_t *p) {
   if (w.head[slot] < 0 || t < w.lo[slot] || t > w.hi[slot]) return 0;
-  if (w.kind == 1) return plan.steps[size_t(w.list_off) + size_t(t)].e[slot];
+  if (w.kind == 1) return plan.steps[size_t(w.j0[0]) + size_t(t)].e[slot];
   // range kind: geometry decides whether the element-wise mask is needed
   Geom g{p->seq_q, p->seq_kv, int64_t(p->seq_kv) - p->seq_q, p->mask.window,
          (p->mask.flags & STEEL_MASK_CAUSAL) != 0, (p->mask.flags & STEEL_MASK_WINDOW) != 0};
-  int64_t J = int64_t(w.j0) + t;
-  int64_t i0 = int64_t(w.qtile[slot]) * kTile, i1 = std::min<int64_t>(i0 + kTile - 1, p->seq_q - 1);
+  int64_t J = int64_t(w.j0[slot]) + t;
+  int64_t i0, i1;
+  tile_positions(p->seq_q, plan_rows_q(*p, plan), w.qtile[slot], &i0, &i1);
   int64_t j0 = J * kTile, j1 = std::min<int64_t>(j0 + kTile - 1, p->seq_kv - 1);
   uint32_t e = uint32_t(J) | kEntryPresent | kEntrySubAll;
   if (!g.all_visible(i0, i1, j0, j1) || (j1 - j0 + 1) < kTile) e |= kEntryPartial;

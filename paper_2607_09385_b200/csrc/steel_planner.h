@@ -20,18 +20,46 @@ constexpr size_t kPartnerWindow = 16;
 // CTA count assumed by the host-only planning entry point (the SM count of a B200).
 constexpr int kPlanHostCtas = 148;
 
+// Cutting key ranges over CTAs, in key-tile steps of two slots (1.75 us).  `fill`: share of a query tile's
+// 128 rows in use, 1 except where all rows of a matrix are fewer.
+constexpr double kSingleStep = 0.65;  // a step of which one slot takes part (1.2 us)
+constexpr double kPieceOverheadSteps = 1.5;
+// A part writes 64 KB of O (head_dim 128) before its CTA goes on; the last one reads those of all parts at an
+// SM's 64 bytes per cycle.
+constexpr double part_write_steps(double fill) { return 2.5 * fill; }
+constexpr double combine_steps(double fill, int parts) { return 1.5 + 0.7 * fill * parts; }
+// Shorter pieces (in key tiles) cost more to start and combine than they take.
+constexpr int min_piece_tiles(double fill) { return int(4 + 8 * fill); }
+
+struct Draft {  // a work item before it is placed
+  WorkItem w;
+  std::vector<StepPair> list;
+  int group;
+  int cta = -1;  // placed already (cut_over_ctas)
+};
+
 struct Plan {
   std::vector<WorkItem> items;     // in CTA order
   std::vector<int32_t> cta_begin;  // grid + 1
   std::vector<StepPair> steps;     // list-kind entries
+  std::vector<SplitTile> split_tiles;
+  int32_t n_parts = 0;             // part buffers of all split tiles
+  bool packed = false;             // query tiles hold rows of all heads of a group (KernelParams::rows_q)
   steel_attn_stats_t stats;
   int grid = 0;
 };
 
 steel_status_t validate_params(const steel_attn_params_t *p);
 // Scheduling policy and the other options come from `p`.  `exec_stats` = false skips the statistics
-// that need a walk over every executed tile (exec_tiles, exec_partial, kv_tile_loads stay 0).
-steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan, bool exec_stats = true);
+// that need a walk over every executed tile (exec_tiles, exec_partial, kv_tile_loads stay 0).  `spread`
+// allows what needs more from the caller than the lists: query tiles over the heads of a group, and key
+// ranges cut over CTAs (part buffers).
+steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan, bool exec_stats = true,
+                          bool spread = false);
+
+// Rows of one matrix of Q as the plan's query tiles see it, and the kernel's fields for that view.
+int64_t plan_rows_q(const steel_attn_params_t &p, const Plan &plan);
+void set_query_view(const steel_attn_params_t &p, bool packed, KernelParams *kp);
 
 // Entry (tile index and flags, 0 if absent) of `slot` at step `t`, derived exactly as on the device.
 uint32_t item_entry(const Plan &plan, const WorkItem &w, int slot, int t, const steel_attn_params_t *p);

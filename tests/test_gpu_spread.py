@@ -1,0 +1,81 @@
+"""Calls whose plan packs the heads of a group into query tiles or cuts key ranges over CTAs, against the
+oracle: one row per matrix, row counts that are not a multiple of 4, rows of several heads in one tile, two to
+dozens of parts, rows without a visible key, software exponents.  Repeated calls are bit-identical (the parts
+are combined in a fixed order, whichever ends last), also after a call that was interrupted."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2607_09385_b200 import binding as B
+from paper_2607_09385_b200 import inputs
+
+import helpers as H
+
+pytestmark = pytest.mark.gpu
+CAUSAL, WINDOW, BITMAP = inputs.MASK_CAUSAL, inputs.MASK_WINDOW, inputs.MASK_BITMAP
+
+CASES = [  # batch, heads_q, heads_kv, seq_q, seq_kv, head_dim, flags, window, emulation
+    (2, 32, 8, 1, 6001, 128, CAUSAL, 0, 0), (3, 16, 16, 1, 3000, 64, CAUSAL, 0, 0), (1, 1, 1, 1, 32768, 128, 0, 0, 0),
+    (1, 8, 1, 3, 1000, 64, CAUSAL, 0, 0), (2, 10, 2, 7, 5000, 128, CAUSAL, 0, 2), (1, 4, 1, 40, 5000, 64, WINDOW, 600, 0),
+    (1, 8, 2, 500, 6500, 128, CAUSAL, 0, 0), (1, 6, 2, 200, 900, 128, CAUSAL | WINDOW, 150, 0),
+    (1, 1, 1, 3000, 3000, 128, CAUSAL, 0, 0), (1, 3, 1, 129, 2500, 64, 0, 0, 1), (1, 4, 2, 60, 20, 128, CAUSAL, 0, 0),
+    (1, 2, 1, 400, 4096, 64, BITMAP, 0, 0),
+]
+
+
+def make(case, seed=5):
+    b, hq, hkv, sq, skv, d, flags, window, emu = case
+    rng = np.random.default_rng(seed)
+    q, k, v = (torch.from_numpy(rng.standard_normal(s, np.float32)).to(torch.bfloat16)
+               for s in ((b, hq, sq, d), (b, hkv, skv, d), (b, hkv, skv, d)))
+    bitmap = None
+    if flags & BITMAP:
+        bitmap = rng.integers(0, 1 << 32, (hq, -(-sq // 128), -(-skv // 4096)), dtype=np.uint32)
+    args = (b, hq, hkv, sq, skv, d, 1.0 / math.sqrt(d), flags)
+    attn = B.SteelAttention(*args, window=window, bitmap=bitmap, exp_emulation=emu)
+    p = oracle.OracleProblem(*args, 128, 128, window, bitmap)
+    return attn, p, q, k, v
+
+
+@pytest.mark.parametrize("case", CASES)
+def test_against_oracle(case):
+    attn, p, q, k, v = make(case)
+    dev = [x.cuda() for x in (q, k, v)]
+    o = torch.full_like(dev[0], float("nan"))
+    lse = torch.full(q.shape[:3], float("nan"), device="cuda")
+    attn.run(*dev, o, lse)
+    assert attn.last_status() == B.STEEL_OK
+    rows = oracle.steel_oracle.all_rows(p)
+    if len(rows) > 400:
+        rows = rows[np.sort(np.random.default_rng(1).choice(len(rows), 400, replace=False))]
+    bits = [x.view(torch.int16).numpy().view(np.uint16) for x in (q, k, v)]
+    o_ref, lse_ref = oracle.rows(p, *bits, rows)
+    at = tuple(torch.from_numpy(rows[:, c].astype(np.int64)) for c in range(3))
+    o_gpu, lse_gpu = o.float().cpu()[at].numpy(), lse.cpu()[at].numpy()
+    err = np.abs(o_gpu - o_ref)
+    assert err.max() <= H.TOL_O_MAX and err.mean() <= H.TOL_O_MEAN
+    seen = np.isfinite(lse_ref)
+    assert np.array_equal(np.isfinite(lse_gpu), seen) and np.abs(lse_gpu[seen] - lse_ref[seen]).max(initial=0) <= H.TOL_LSE
+    for _ in range(3):
+        o2, lse2 = attn.run(*dev)
+        assert torch.equal(o2, o) and torch.equal(lse2, lse)
+    attn.close()
+
+
+def test_interrupted_call_leaves_nothing_behind():
+    attn, _, q, k, v = make(CASES[6])
+    dev = [x.cuda() for x in (q, k, v)]
+    o, lse = attn.run(*dev)
+    assert attn.last_status() == B.STEEL_OK
+    B.steel_attn_debug_stall(attn.handle, 3, 200_000_000)  # 0.1 s
+    attn.run(*dev)
+    assert attn.last_status() == B.STEEL_ERR_TIMEOUT
+    B.steel_attn_debug_stall(attn.handle, -1)
+    for _ in range(2):
+        o2, lse2 = attn.run(*dev)
+        assert attn.last_status() == B.STEEL_OK
+        assert torch.equal(o2, o) and torch.equal(lse2, lse)
+    attn.close()
