@@ -112,7 +112,10 @@ typedef struct {
  * CUDA device.  On success *out receives the handle; on failure *out is NULL.
  * STEEL_ERR_UNSUPPORTED: head_dim not in {64, 128}; block sizes other than 64 or 128 or
  * block_q != block_kv; more than 2^24 key tiles; batch * heads * seq beyond 2^31 rows.  Allocates device memory;
- * synchronises the device once.
+ * synchronises the device once.  Where the problem has few query tiles, the plan may let a tile hold rows of
+ * several heads of a group and cut a tile's keys over several CTAs; the handle then also owns buffers for the
+ * parts' results (a part of one tile: up to 128 x (head_dim + 2) floats), and the work-list statistics below count
+ * such tiles.  steel_attn_plan_host reports the plan without either.
  */
 steel_status_t steel_attn_create(const steel_attn_params_t *params, steel_attn_t **out);
 
@@ -197,7 +200,7 @@ steel_status_t steel_attn_run_noalloc(const steel_attn_params_t *params, const v
 /*
  * The same operation for tensors in HOST memory (the end-to-end path of Eq. 1 / Algorithm 1:
  * operands start and results end on the host).  A host-side object owns device staging buffers for
- * Q, K, V, O and LSE, three internal streams and one plan per chunk.  The problem is cut into at
+ * Q, K, V, O and LSE, internal streams and one plan per chunk.  The problem is cut into at
  * most `max_chunks` chunks that are independent attention problems with contiguous tensors: groups
  * of batch elements when batch > 1, groups of KV heads (with their query heads and their slice of
  * the bitmap) when batch == 1; the number used is the largest divisor of batch (of heads_kv) not

@@ -120,9 +120,9 @@ steel_status_t launch_with_params(const steel_attn_params_t &p, KernelParams kp,
 
 }  // namespace steel
 
-extern "C" {
+namespace steel {
 
-steel_status_t steel_attn_create(const steel_attn_params_t *params, steel_attn_t **out) {
+steel_status_t create_attention(const steel_attn_params_t *params, Spread most, steel_attn_t **out) {
   if (!out) return STEEL_ERR_INVALID_ARG;
   *out = nullptr;
   steel_status_t st = validate_params(params);
@@ -139,9 +139,9 @@ steel_status_t steel_attn_create(const steel_attn_params_t *params, steel_attn_t
   steel_attn *h = new (std::nothrow) steel_attn();
   if (!h) return STEEL_ERR_ALLOC;
   Plan plan;
-  for (bool spread : {true, false}) {
+  for (Spread spread : {most, Spread::kTiles}) {  // the second only without memory for the first's part buffers
     try {
-      st = build_plan(params, prop.multiProcessorCount, &plan, /*exec_stats=*/true, spread);
+      st = build_plan(params, prop.multiProcessorCount, &plan, /*stats=*/true, spread);
     } catch (const std::bad_alloc &) {
       st = STEEL_ERR_ALLOC;
     }
@@ -199,6 +199,14 @@ steel_status_t steel_attn_create(const steel_attn_params_t *params, steel_attn_t
   }
   *out = h;
   return STEEL_OK;
+}
+
+}  // namespace steel
+
+extern "C" {
+
+steel_status_t steel_attn_create(const steel_attn_params_t *params, steel_attn_t **out) {
+  return create_attention(params, Spread::kCut, out);
 }
 
 steel_status_t steel_attn_run(steel_attn_t *h, const void *q, const void *k, const void *v, void *o, float *lse,

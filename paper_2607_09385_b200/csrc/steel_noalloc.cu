@@ -9,6 +9,7 @@
 // until the process exits.  Inputs and outputs are still the caller's.
 #include <cuda_runtime.h>
 
+#include <cstring>
 #include <mutex>
 #include <new>
 
@@ -23,11 +24,12 @@ namespace {
 constexpr size_t kMaxItems = 16384;   // work items (64 bytes each)
 constexpr size_t kMaxCtas = 1024;     // persistent CTAs (+1 range entry)
 constexpr size_t kMaxSteps = 131072;  // explicit step-list entries of bitmap masks (8 bytes each)
-constexpr size_t kOffStatus = 0;
-constexpr size_t kOffItems = 256;
-constexpr size_t kOffCtaBegin = kOffItems + kMaxItems * sizeof(WorkItem);
-constexpr size_t kOffSteps = (kOffCtaBegin + (kMaxCtas + 1) * sizeof(int32_t) + 255) / 256 * 256;
-constexpr size_t kScratchBytes = kOffSteps + kMaxSteps * sizeof(StepPair);  // about 2.0 MiB
+// The call's lists are packed one behind the other, so that one copy brings them: status word, per-CTA
+// ranges, items, steps.
+constexpr size_t kOffCtaBegin = 256;
+constexpr size_t round16(size_t n) { return (n + 15) / 16 * 16; }
+constexpr size_t kScratchBytes = kOffCtaBegin + round16((kMaxCtas + 1) * sizeof(int32_t)) +
+                                 kMaxItems * sizeof(WorkItem) + kMaxSteps * sizeof(StepPair);  // about 2.0 MiB
 
 // In host code this name is only a handle for the symbol, never a device address: the address the
 // kernel needs comes from cudaGetSymbolAddress below.
@@ -82,47 +84,51 @@ extern "C" steel_status_t steel_attn_run_noalloc(const steel_attn_params_t *para
     return st;
   }
 
-  Plan plan;  // host memory only
+  // Host memory only.  One query tile per item can need more list entries than pairs: where the fixed array
+  // has no room for it, the paired plan is taken.  What fits in neither way is refused, not truncated.
+  Plan plan;
+  bool fits = false;
+  std::vector<unsigned char> lists;
+  size_t off_items = 0, off_steps = 0;
   try {
-    st = build_plan(params, sm_count, &plan, /*exec_stats=*/false);
+    for (Spread spread : {Spread::kTiles, Spread::kNone}) {
+      st = build_plan(params, sm_count, &plan, /*stats=*/false, spread);
+      if (st != STEEL_OK) return st;
+      fits = plan.items.size() <= kMaxItems && plan.steps.size() <= kMaxSteps && plan.cta_begin.size() <= kMaxCtas + 1;
+      if (fits) break;
+    }
+    if (!fits) return STEEL_ERR_UNSUPPORTED;
+    off_items = kOffCtaBegin + round16(plan.cta_begin.size() * sizeof(int32_t));
+    off_steps = off_items + plan.items.size() * sizeof(WorkItem);
+    lists.resize(off_steps + plan.steps.size() * sizeof(StepPair));
   } catch (const std::bad_alloc &) {
     return STEEL_ERR_ALLOC;
   }
-  if (st != STEEL_OK) return st;
-  // the fixed array bounds the problem: refuse, rather than truncate, anything larger
-  if (plan.items.size() > kMaxItems || plan.steps.size() > kMaxSteps || plan.cta_begin.size() > kMaxCtas + 1)
-    return STEEL_ERR_UNSUPPORTED;
+  std::memcpy(lists.data() + kOffCtaBegin, plan.cta_begin.data(), plan.cta_begin.size() * sizeof(int32_t));
+  if (!plan.items.empty()) std::memcpy(lists.data() + off_items, plan.items.data(), off_steps - off_items);
+  if (!plan.steps.empty()) std::memcpy(lists.data() + off_steps, plan.steps.data(), lists.size() - off_steps);
 
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  // The array still holds the previous call's lists and status word: overwrite the lists, clear the word.
-  bool ok = cudaMemsetAsync(base + kOffStatus, 0, sizeof(int32_t), stream) == cudaSuccess &&
-            (plan.items.empty() || cudaMemcpyAsync(base + kOffItems, plan.items.data(),
-                                                   plan.items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice,
-                                                   stream) == cudaSuccess) &&
-            cudaMemcpyAsync(base + kOffCtaBegin, plan.cta_begin.data(), plan.cta_begin.size() * sizeof(int32_t),
-                            cudaMemcpyHostToDevice, stream) == cudaSuccess &&
-            (plan.steps.empty() || cudaMemcpyAsync(base + kOffSteps, plan.steps.data(),
-                                                   plan.steps.size() * sizeof(StepPair), cudaMemcpyHostToDevice,
-                                                   stream) == cudaSuccess);
-  if (!ok) {
+  // The array still holds the previous call's lists and status word: overwrite both (the word with 0).
+  if (cudaMemcpyAsync(base, lists.data(), lists.size(), cudaMemcpyHostToDevice, stream) != cudaSuccess) {
     cudaGetLastError();
     return STEEL_ERR_CUDA;
   }
   KernelParams kp{};  // no split query tiles: their buffers have no room in the array
-  kp.items = reinterpret_cast<const WorkItem *>(base + kOffItems);
+  kp.items = reinterpret_cast<const WorkItem *>(base + off_items);
   kp.cta_begin = reinterpret_cast<const int32_t *>(base + kOffCtaBegin);
-  kp.steps = reinterpret_cast<const StepPair *>(base + kOffSteps);
-  kp.status = reinterpret_cast<int32_t *>(base + kOffStatus);
+  kp.steps = reinterpret_cast<const StepPair *>(base + off_steps);
+  kp.status = reinterpret_cast<int32_t *>(base);
   set_query_view(*params, plan.packed, &kp);
   kp.timeout_cycles = kDefaultTimeoutCycles;
   kp.stall_cta = -1;
   st = launch_with_params(*params, kp, plan.grid, q, k, v, o, lse, stream, nullptr);
   if (st != STEEL_OK) return st;
-  // Blocking by design: the host lists above must outlive the copies, and the status word has to
-  // be read before the next call clears it.
+  // Blocking by design: the host lists above must outlive the copy, and the status word has to be read
+  // before the next call clears it.  The read on the same stream waits for the kernel.
   int32_t word = 0;
-  if (cudaStreamSynchronize(stream) != cudaSuccess ||
-      cudaMemcpy(&word, base + kOffStatus, sizeof word, cudaMemcpyDeviceToHost) != cudaSuccess) {
+  if (cudaMemcpyAsync(&word, base, sizeof word, cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+      cudaStreamSynchronize(stream) != cudaSuccess) {
     cudaGetLastError();
     return STEEL_ERR_CUDA;
   }

@@ -68,38 +68,68 @@ struct Ctx {
     j0 = J * size;
     j1 = std::min<int64_t>(j0 + size - 1, p->seq_kv - 1);
   }
-  // Bitmap masks: entry of kernel tile (I, J) for head h, or 0 if the tile is fully masked (case i).
-  uint32_t entry(int h, int64_t I, int64_t J) const {
-    int64_t i0, i1, j0, j1;
+  // First and last tile of `size` keys that queries i0 .. i1 see, and that they see whole, under the causal
+  // and window terms (each set is a range; empty if first > last).
+  void seen_range(int64_t i0, int64_t i1, int64_t size, int64_t tiles, int64_t *first, int64_t *last) const {
+    const int64_t top = g.causal ? i1 + g.off : kInf, bottom = g.windowed ? i0 + g.off - g.window + 1 : 0;
+    *last = top < 0 ? -1 : std::min(tiles - 1, top / size);
+    *first = bottom > 0 ? bottom / size : 0;
+  }
+  void whole_range(int64_t i0, int64_t i1, int64_t size, int64_t *first, int64_t *last) const {
+    const int64_t top = g.causal ? i0 + g.off : kInf, bottom = g.windowed ? i1 + g.off - g.window + 1 : 0;
+    *last = top < 0 ? -1 : (std::min<int64_t>(top, p->seq_kv - 1) + 1) / size - 1;
+    if (top >= p->seq_kv - 1) *last = (p->seq_kv - 1) / size;  // a ragged last tile is seen whole
+    *first = bottom > 0 ? (bottom + size - 1) / size : 0;
+  }
+  // Bits first .. last of the word that holds bits 32 w .. 32 w + 31.
+  static uint32_t range_bits(int64_t w, int64_t first, int64_t last) {
+    const int64_t a = std::max<int64_t>(first - 32 * w, 0), b = std::min<int64_t>(last - 32 * w, 31);
+    return a > b ? 0u : (0xFFFFFFFFu >> (31 - (b - a))) << a;
+  }
+
+  // Bitmap masks: the entries of query tile I of head h, fully masked tiles (case i) left out.  Word by word:
+  // one tile at a time took most of the planning (8 heads x 4096 tokens, 64-token blocks: 528 us in all, now 55).
+  void entries(int h, int64_t I, std::vector<uint32_t> *out) const {
+    int64_t i0, i1, whole_lo, whole_hi;
     rows(I, kTile, i0, i1);
-    keys(J, kTile, j0, j1);
-    bool ragged = (j1 - j0 + 1) < kTile;
-    uint32_t sub = 0xF;
-    bool kept, full;
-    if (bq == kTile) {
-      kept = bit(h, I, J) && g.any_visible(i0, i1, j0, j1);
-      full = g.all_visible(i0, i1, j0, j1);
-    } else {  // 64-token blocks: four sub-blocks TL, TR, BL, BR
-      sub = 0;
-      kept = false;
-      full = g.all_visible(i0, i1, j0, j1);
-      for (int a = 0; a < 2; ++a)
-        for (int b = 0; b < 2; ++b) {
-          int64_t si0 = i0 + 64 * a, sj0 = j0 + 64 * b;
-          if (si0 > i1 || sj0 > j1) continue;  // outside the problem
-          int64_t si1 = std::min(si0 + 63, i1), sj1 = std::min(sj0 + 63, j1);
-          if (bit(h, 2 * I + a, 2 * J + b)) {
-            sub |= 1u << (2 * a + b);
-            kept = kept || g.any_visible(si0, si1, sj0, sj1);
-          } else {
-            full = false;
-          }
-        }
+    whole_range(i0, i1, kTile, &whole_lo, &whole_hi);
+    const bool ragged = p->seq_kv % kTile != 0;
+    const int per = int(kTile / bq);  // blocks of a tile in each direction: 1 or 2
+    const uint32_t *row[2] = {nullptr, nullptr};
+    int64_t lo[2] = {0, 0}, hi[2] = {-1, -1};
+    for (int a = 0; a < per && per * I + a < tqb; ++a) {
+      row[a] = p->mask.bitmap + (int64_t(h) * tqb + per * I + a) * words;
+      int64_t r0, r1;
+      rows(per * I + a, bq, r0, r1);
+      seen_range(r0, r1, bq, tkvb, &lo[a], &hi[a]);
     }
-    if (!kept) return 0;
-    uint32_t e = uint32_t(J) | kEntryPresent | (sub << kEntrySubShift);
-    if (!full || ragged) e |= kEntryPartial;
-    return e;
+    const int64_t w_first = (per == 1 ? lo[0] : std::min(lo[0], row[1] ? lo[1] : lo[0])) / 32;
+    const int64_t w_last = std::max(hi[0], hi[1]) / 32;
+    if (std::max(hi[0], hi[1]) < 0) return;
+    for (int64_t w = w_first; w <= w_last; ++w) {
+      const uint32_t inside = range_bits(w, 0, tkvb - 1);
+      uint32_t set[2] = {0u, 0u}, kept = 0u;
+      for (int a = 0; a < per; ++a)
+        if (row[a]) {
+          set[a] = row[a][w] & inside;
+          kept |= set[a] & range_bits(w, lo[a], hi[a]);
+        }
+      if (per == 2) kept = (kept | kept >> 1) & 0x55555555u;
+      for (; kept; kept &= kept - 1) {
+        const int bit0 = __builtin_ctz(kept);
+        const int64_t J = (32 * w + bit0) / per;
+        uint32_t sub = 0xF;
+        bool full = J >= whole_lo && J <= whole_hi;
+        if (per == 2) {  // sub-blocks TL, TR, BL, BR; those outside the problem do not make a tile partial
+          const uint32_t a = (set[0] >> bit0) & 3u, b = (set[1] >> bit0) & 3u, in = (inside >> bit0) & 3u;
+          sub = a | b << 2;
+          full = full && a == in && (!row[1] || b == in);
+        }
+        uint32_t e = uint32_t(J) | kEntryPresent | (sub << kEntrySubShift);
+        if (!full || (ragged && J == tkv128 - 1)) e |= kEntryPartial;
+        out->push_back(e);
+      }
+    }
   }
 };
 
@@ -312,7 +342,7 @@ steel_status_t validate_params(const steel_attn_params_t *p) {
   return STEEL_OK;
 }
 
-steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan, bool exec_stats, bool spread) {
+steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan, bool stats, Spread spread) {
   steel_status_t st = validate_params(p);
   if (st != STEEL_OK) return st;
   const int policy = p->policy;
@@ -332,7 +362,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
   c.words = (c.tkvb + 31) / 32;
   int G = p->heads_q / p->heads_kv;  // heads (matrices of Q) that share a KV head
   int heads = p->heads_q;
-  spread = spread && policy == 0;
+  if (policy != 0) spread = Spread::kNone;
 
   plan->items.clear();
   plan->steps.clear();
@@ -344,7 +374,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
   s = steel_attn_stats_t{};
 
   // ---- statistics at the descriptor's block granularity (what "kept tiles" means to a caller)
-  {
+  if (stats) {
     int64_t kept = 0, partial = 0;
     double pairs = 0.0;
     for (int h = 0; h < p->heads_q; ++h) {
@@ -380,7 +410,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
   // rows.  Few queries per head leave most of a head's last tile empty (a decode step: 127 of 128 rows);
   // tiles over that matrix are then fewer.  A tile that holds the end of one head and the start of the next
   // spans all positions, which costs key tiles under a causal mask: taken only where the total is smaller.
-  if (spread && !c.bitmap && G > 1) {
+  if (spread != Spread::kNone && !c.bitmap && G > 1) {
     auto executed = [&](bool packed) {
       const int64_t rows = packed ? int64_t(G) * p->seq_q : p->seq_q;
       int64_t n = 0, lo, hi;
@@ -400,6 +430,9 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
   }
   const int64_t rows_q = plan_rows_q(*p, *plan);
   std::vector<std::vector<Task>> tasks(heads);  // [h][I]
+  const size_t key_words = size_t(c.tkv128 + 63) / 64;
+  std::vector<uint64_t> keys;  // bitmap masks: the key tiles of each task as bits
+  if (c.bitmap) keys.assign(size_t(heads) * size_t(c.tq128) * key_words, 0);
   for (int h = 0; h < heads; ++h) {
     tasks[h].resize(c.tq128);
     for (int64_t I = 0; I < c.tq128; ++I) {
@@ -407,9 +440,11 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
       t.h = h;
       t.I = I;
       if (c.bitmap) {
-        for (int64_t J = 0; J < c.tkv128; ++J) {
-          uint32_t e = c.entry(h, I, J);
-          if (e) t.entries.push_back(e);
+        t.entries.reserve(size_t(c.tkv128));
+        c.entries(h, I, &t.entries);
+        for (uint32_t e : t.entries) {
+          const uint32_t J = e & kEntryTileMask;
+          keys[size_t(h * c.tq128 + I) * key_words + J / 64] |= uint64_t(1) << (J % 64);
         }
       } else if (h > 0) {
         t.jlo = tasks[0][I].jlo;
@@ -448,6 +483,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
     w.n_steps = std::max(w.hi[0], w.hi[1]) + 1;
     drafts.push_back(std::move(d));
   };
+  std::vector<uint32_t> ea, eb, rest_a, rest_b;  // of finish_list
   auto finish_list = [&](const Task *a, const Task *b, int batch, int g) {
     Draft d{};
     d.group = g;
@@ -468,9 +504,11 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
     w.n_steps = int32_t(std::max(na, nb));
     // Key tiles may be visited in any order (the online softmax does not care), so the tiles both
     // query tiles want come first, in the same steps: each of those steps needs one K/V load, not two.
-    std::vector<uint32_t> ea, eb;
+    ea.clear();
+    eb.clear();
     if (b) {
-      std::vector<uint32_t> rest_a, rest_b;
+      rest_a.clear();
+      rest_b.clear();
       size_t ia = 0, ib = 0;
       while (ia < na || ib < nb) {
         const uint32_t ta = ia < na ? (a->entries[ia] & kEntryTileMask) : 0xFFFFFFFFu;
@@ -489,6 +527,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
     } else {
       ea = a->entries;
     }
+    d.list.reserve(size_t(w.n_steps));
     for (size_t t = 0; t < size_t(w.n_steps); ++t)
       d.list.push_back(StepPair{{t < na ? ea[t] : 0u, t < nb ? eb[t] : 0u}});
     drafts.push_back(std::move(d));
@@ -537,14 +576,9 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
               if (used[m]) continue;
               ++seen;
               int64_t common = 0;
-              size_t ia = 0, ib = 0;
-              const std::vector<uint32_t> &ea = live[n]->entries, &eb = live[m]->entries;
-              while (ia < ea.size() && ib < eb.size()) {
-                const uint32_t ta = ea[ia] & kEntryTileMask, tb = eb[ib] & kEntryTileMask;
-                if (ta == tb) { ++common; ++ia; ++ib; }
-                else if (ta < tb) ++ia;
-                else ++ib;
-              }
+              const uint64_t *ka = &keys[size_t(live[n]->h * c.tq128 + live[n]->I) * key_words],
+                             *kb = &keys[size_t(live[m]->h * c.tq128 + live[m]->I) * key_words];
+              for (size_t w = 0; w < key_words; ++w) common += __builtin_popcountll(ka[w] & kb[w]);
               // a step with one idle slot costs far more than a shared load saves
               const int64_t score = common - 16 * (live[n]->count() - live[m]->count());
               if (score > best_common || best == live.size()) { best_common = score; best = m; }
@@ -583,7 +617,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
   // tenth more than the mean.)  Kernel time, paired -> chosen plan: 500 queries on 12500 keys, 32/8 heads,
   // 161 -> 96 us (cut); a decode step of batch 8 on 6001 keys, 32/8 heads, 82 -> 39 us (packed and cut);
   // 12 heads x 512 d64 11.8 -> 9.6 us, 16/4 heads x 2048 d128 35.2 -> 30.7 us (one query tile per item).
-  if (spread && drafts.size() < size_t(8 * num_ctas)) {
+  if (spread != Spread::kNone && drafts.size() < size_t(8 * num_ctas)) {
     const double fill = double(std::min<int64_t>(rows_q, kTile)) / kTile;
     double work = 0.0;
     for (const Draft &d : drafts) work += step_cost(d.w) * d.w.n_steps + kItemOverheadSteps;
@@ -597,6 +631,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
       std::vector<Draft> singles;
       singles.swap(drafts);
       for (const std::vector<Draft> *from : {&paired_drafts, &singles}) {
+        if (spread != Spread::kCut) break;
         Plan cut;
         std::vector<Draft> pieces;
         const double t = cut_over_ctas(*from, num_ctas, fill, &pieces, &cut);
@@ -698,7 +733,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
     s.max_cta_steps = std::max(s.max_cta_steps, st_sum);
   }
   // the walk visits every executed tile (millions on long sequences): only for callers that read these
-  if (exec_stats) walk_plan(*plan, [&](int, const WorkItem &, int, int, uint32_t entry, bool shared) {
+  if (stats) walk_plan(*plan, [&](int, const WorkItem &, int, int, uint32_t entry, bool shared) {
     ++s.exec_tiles;
     s.exec_partial += (entry & kEntryPartial) != 0;
     s.kv_tile_loads += shared ? 0 : 1;

@@ -50,12 +50,19 @@ struct Plan {
 };
 
 steel_status_t validate_params(const steel_attn_params_t *p);
-// Scheduling policy and the other options come from `p`.  `exec_stats` = false skips the statistics
-// that need a walk over every executed tile (exec_tiles, exec_partial, kv_tile_loads stay 0).  `spread`
-// allows what needs more from the caller than the lists: query tiles over the heads of a group, and key
-// ranges cut over CTAs (part buffers).
-steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan, bool exec_stats = true,
-                          bool spread = false);
+// What a plan may do beyond pairing query tiles (policy 0 only; build_plan takes what ends earliest).
+enum class Spread {
+  kNone,
+  kTiles,  // query tiles over the heads of a group, one query tile per item
+  kCut,    // also key ranges cut over CTAs, which needs part buffers
+};
+// Scheduling policy and the other options come from `p`.  Without `stats` the plan's statistics stay 0 (they
+// take a walk over every block and every executed tile).
+steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan, bool stats = true,
+                          Spread spread = Spread::kNone);
+
+// steel_attn_create with a limit on what the plan may do (implemented in steel_attn.cu).
+steel_status_t create_attention(const steel_attn_params_t *params, Spread most, steel_attn_t **out);
 
 // Rows of one matrix of Q as the plan's query tiles see it, and the kernel's fields for that view.
 int64_t plan_rows_q(const steel_attn_params_t &p, const Plan &plan);

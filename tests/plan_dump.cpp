@@ -21,7 +21,7 @@ int main(int argc, char **argv) {
   p.mask.window = std::atoi(argv[8]);
   p.mask.bitmap = bitmap.empty() ? nullptr : bitmap.data();
   steel::Plan plan;
-  if (steel::build_plan(&p, std::atoi(argv[1]), &plan, true, true) != STEEL_OK) return 3;
+  if (steel::build_plan(&p, std::atoi(argv[1]), &plan, true, steel::Spread::kCut) != STEEL_OK) return 3;
   std::printf("plan %d %d %d %d\n", plan.grid, int(plan.packed), plan.n_parts, int(plan.items.size()));
   for (const steel::SplitTile &t : plan.split_tiles) std::printf("split %d %d\n", t.first, t.n_parts);
   for (size_t c = 0; c + 1 < plan.cta_begin.size(); ++c)
