@@ -227,6 +227,7 @@ steel_status_t steel_attn_run(steel_attn_t *h, const void *q, const void *k, con
   kp.part_rows = h->part_rows;
   kp.arrivals = h->d_arrivals;
   set_query_view(h->params, h->packed, &kp);
+  kp.overlap_launch = h->stats.max_cta_steps <= kOverlapSteps;
   kp.clock_probe = h->d_clock_probe;
   kp.timeout_cycles = h->timeout_cycles;
   kp.stall_cta = h->stall_cta;

@@ -907,6 +907,10 @@ steel_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     tmem_alloc(&ctrl.tmem_base, 512);
     tmem_relinquish();
   }
+  // From here on the next launch on the stream may set itself up on SMs that this one leaves; this launch in
+  // turn touches global memory only after the one before it has completed.
+  grid_launch_dependents();
+  grid_dependency_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -945,10 +949,20 @@ cudaError_t configure_one() {
 template <int D, int kEmu>
 void launch_one(const CUtensorMap &map_q, const CUtensorMap &map_k, const CUtensorMap &map_v,
                 const KernelParams &params, int grid, cudaStream_t stream) {
+  cudaLaunchConfig_t config = {};
+  config.gridDim = dim3(grid);
+  config.blockDim = dim3(kThreads);
+  config.dynamicSmemBytes = Cfg<D>::kSmemBytes;
+  config.stream = stream;
+  cudaLaunchAttribute overlap;
+  overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  overlap.val.programmaticStreamSerializationAllowed = 1;
+  config.attrs = &overlap;
+  config.numAttrs = params.overlap_launch ? 1 : 0;
   if (params.split_tiles)
-    steel_attn_kernel<D, kEmu, true><<<grid, kThreads, Cfg<D>::kSmemBytes, stream>>>(map_q, map_k, map_v, params);
+    cudaLaunchKernelEx(&config, steel_attn_kernel<D, kEmu, true>, map_q, map_k, map_v, params);
   else
-    steel_attn_kernel<D, kEmu, false><<<grid, kThreads, Cfg<D>::kSmemBytes, stream>>>(map_q, map_k, map_v, params);
+    cudaLaunchKernelEx(&config, steel_attn_kernel<D, kEmu, false>, map_q, map_k, map_v, params);
 }
 
 template <int D>

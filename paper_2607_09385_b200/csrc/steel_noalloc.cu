@@ -120,6 +120,7 @@ extern "C" steel_status_t steel_attn_run_noalloc(const steel_attn_params_t *para
   kp.steps = reinterpret_cast<const StepPair *>(base + off_steps);
   kp.status = reinterpret_cast<int32_t *>(base);
   set_query_view(*params, plan.packed, &kp);
+  kp.overlap_launch = plan.stats.max_cta_steps <= kOverlapSteps;
   kp.timeout_cycles = kDefaultTimeoutCycles;
   kp.stall_cta = -1;
   st = launch_with_params(*params, kp, plan.grid, q, k, v, o, lse, stream, nullptr);

@@ -69,6 +69,7 @@ struct KernelParams {
   float scale_log2;          // scale * log2(e)
   long long *clock_probe;    // measurement hook: CTA 0 stores {SM cycles, nanoseconds} of its run here, else null
   long long timeout_cycles;  // bound of every device-side wait
+  bool overlap_launch;       // host side: start beside the end of the launch before it on the stream
   int32_t stall_cta;         // test hook: this CTA's producer withholds its commands (-1: none)
 };
 
