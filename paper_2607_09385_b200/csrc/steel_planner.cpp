@@ -156,7 +156,16 @@ struct Task {  // one query tile of one head (packed: of one group of heads)
   int h;
   int64_t I;
   int64_t jlo = 0, jhi = -1;      // range kind
-  std::vector<uint32_t> entries;  // list kind
+  // list kind: the task's stretch of one array for all tasks (a heap block each took longer than the rest)
+  struct Entries {
+    const uint32_t *first = nullptr;
+    size_t n = 0, at = 0;  // `at`: offset in the array, while that grows
+    size_t size() const { return n; }
+    bool empty() const { return n == 0; }
+    uint32_t operator[](size_t i) const { return first[i]; }
+    const uint32_t *begin() const { return first; }
+    const uint32_t *end() const { return first + n; }
+  } entries;
   int64_t count() const { return entries.empty() ? jhi - jlo + 1 : int64_t(entries.size()); }
 };
 
@@ -165,9 +174,7 @@ bool slot_used(const WorkItem &w, int s) { return w.head[s] >= 0 && w.hi[s] >= w
 double step_cost(const WorkItem &w) { return slot_used(w, 0) && slot_used(w, 1) ? 1.0 : kSingleStep; }
 
 // Load of the busiest CTA, in steps of two slots, with the longest item first to the least loaded CTA.
-double makespan(const std::vector<Draft> &drafts, int num_ctas) {
-  std::vector<double> cost;
-  for (const Draft &d : drafts) cost.push_back(step_cost(d.w) * d.w.n_steps + kItemOverheadSteps);
+double makespan(std::vector<double> cost, int num_ctas) {
   std::sort(cost.begin(), cost.end(), std::greater<double>());
   std::priority_queue<double, std::vector<double>, std::greater<double>> load;
   for (int n = 0; n < num_ctas; ++n) load.push(0.0);
@@ -179,6 +186,13 @@ double makespan(const std::vector<Draft> &drafts, int num_ctas) {
     most = std::max(most, x);
   }
   return most;
+}
+
+double makespan(const std::vector<Draft> &drafts, int num_ctas) {
+  std::vector<double> cost;
+  cost.reserve(drafts.size());
+  for (const Draft &d : drafts) cost.push_back(step_cost(d.w) * d.w.n_steps + kItemOverheadSteps);
+  return makespan(std::move(cost), num_ctas);
 }
 
 // Steps [t0, t1) of `d`.  A draft of one query tile becomes a piece whose slots walk the two halves of the
@@ -431,6 +445,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
   const int64_t rows_q = plan_rows_q(*p, *plan);
   std::vector<std::vector<Task>> tasks(heads);  // [h][I]
   const size_t key_words = size_t(c.tkv128 + 63) / 64;
+  std::vector<uint32_t> entries;
   std::vector<uint64_t> keys;  // bitmap masks: the key tiles of each task as bits
   if (c.bitmap) keys.assign(size_t(heads) * size_t(c.tq128) * key_words, 0);
   for (int h = 0; h < heads; ++h) {
@@ -440,10 +455,11 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
       t.h = h;
       t.I = I;
       if (c.bitmap) {
-        t.entries.reserve(size_t(c.tkv128));
-        c.entries(h, I, &t.entries);
-        for (uint32_t e : t.entries) {
-          const uint32_t J = e & kEntryTileMask;
+        t.entries.at = entries.size();
+        c.entries(h, I, &entries);
+        t.entries.n = entries.size() - t.entries.at;
+        for (size_t n = t.entries.at; n < entries.size(); ++n) {
+          const uint32_t J = entries[n] & kEntryTileMask;
           keys[size_t(h * c.tq128 + I) * key_words + J / 64] |= uint64_t(1) << (J % 64);
         }
       } else if (h > 0) {
@@ -455,6 +471,9 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
       }
     }
   }
+
+  for (std::vector<Task> &row : tasks)
+    for (Task &t : row) t.entries.first = entries.data() + t.entries.at;
 
   // ---- work items: pair query tiles that can share K/V loads
   std::vector<Draft> drafts;
@@ -525,7 +544,10 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
       ea.insert(ea.end(), rest_a.begin(), rest_a.end());
       eb.insert(eb.end(), rest_b.begin(), rest_b.end());
     } else {
-      ea = a->entries;
+      d.list.reserve(na);
+      for (uint32_t e : a->entries) d.list.push_back(StepPair{{e, 0u}});
+      drafts.push_back(std::move(d));
+      return;
     }
     d.list.reserve(size_t(w.n_steps));
     for (size_t t = 0; t < size_t(w.n_steps); ++t)
@@ -564,27 +586,37 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
           }
         if (c.bitmap) {
           // similar lengths pair best: both tiles of an item then finish together
-          std::stable_sort(live.begin(), live.end(), [](const Task *a, const Task *b) { return a->count() > b->count(); });
+          struct Length {
+            int64_t n;
+            const uint64_t *keys;
+            const Task *task;
+          };
+          std::vector<Length> by_length;
+          by_length.reserve(live.size());
+          for (const Task *t : live)
+            by_length.push_back({t->count(), &keys[size_t(t->h * c.tq128 + t->I) * key_words], t});
+          if (pair)
+            std::stable_sort(by_length.begin(), by_length.end(), [](const Length &a, const Length &b) { return a.n > b.n; });
           // among the next few tasks of similar length, take the partner with the most key tiles in common
-          std::vector<bool> used(live.size(), false);
+          std::vector<char> used(live.size(), 0);
           for (size_t n = 0; n < live.size(); ++n) {
             if (used[n]) continue;
-            used[n] = true;
+            used[n] = 1;
+            const Length &a = by_length[n];
             size_t best = live.size(), seen = 0;
             int64_t best_common = 0;
             for (size_t m = n + 1; pair && m < live.size() && seen < kPartnerWindow; ++m) {
               if (used[m]) continue;
               ++seen;
+              const Length &b = by_length[m];
               int64_t common = 0;
-              const uint64_t *ka = &keys[size_t(live[n]->h * c.tq128 + live[n]->I) * key_words],
-                             *kb = &keys[size_t(live[m]->h * c.tq128 + live[m]->I) * key_words];
-              for (size_t w = 0; w < key_words; ++w) common += __builtin_popcountll(ka[w] & kb[w]);
+              for (size_t w = 0; w < key_words; ++w) common += __builtin_popcountll(a.keys[w] & b.keys[w]);
               // a step with one idle slot costs far more than a shared load saves
-              const int64_t score = common - 16 * (live[n]->count() - live[m]->count());
+              const int64_t score = common - 16 * (a.n - b.n);
               if (score > best_common || best == live.size()) { best_common = score; best = m; }
             }
-            if (best < live.size()) used[best] = true;
-            finish_list(live[n], best < live.size() ? live[best] : nullptr, batch, g);
+            if (best < live.size()) used[best] = 1;
+            finish_list(a.task, best < live.size() ? by_length[best].task : nullptr, batch, g);
           }
         } else if (!pair) {
           for (const Task *t : live) finish_range(t, nullptr, batch, g);
@@ -610,6 +642,32 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
       }
     }
   };
+  // Bitmap masks: the search for partners takes most of the planning, so where no key range may be cut the
+  // choice between pairs and single tiles is made on the lengths alone (partners are of similar length).
+  bool chosen = false;
+  if (spread == Spread::kTiles && c.bitmap && int64_t(p->batch) * heads * c.tq128 < 8 * num_ctas) {
+    std::vector<double> paired, single;
+    double work = 0.0;
+    std::vector<int64_t> count;
+    for (int g = 0; g < p->heads_kv; ++g) {
+      count.clear();
+      for (int h = g * G; h < (g + 1) * G; ++h)
+        for (const Task &t : tasks[h])
+          if (t.count() > 0) count.push_back(t.count());
+      std::sort(count.begin(), count.end(), std::greater<int64_t>());
+      for (int batch = 0; batch < p->batch; ++batch)
+        for (size_t n = 0; n < count.size(); ++n) {
+          single.push_back(kSingleStep * double(count[n]) + kItemOverheadSteps);
+          if (n % 2) continue;
+          paired.push_back((n + 1 < count.size() ? 1.0 : kSingleStep) * double(count[n]) + kItemOverheadSteps);
+          work += paired.back();
+        }
+    }
+    const double load = makespan(std::move(paired), num_ctas);
+    chosen = true;
+    pair = !(load > 1.1 * work / num_ctas && makespan(std::move(single), num_ctas) < 0.95 * load);
+  }
+  drafts.reserve(size_t(p->batch) * size_t(heads) * size_t(c.tq128));
   build_drafts();
 
   // ---- few items: one query tile per item, or key ranges cut over all CTAs, where that ends earlier.
@@ -617,7 +675,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
   // tenth more than the mean.)  Kernel time, paired -> chosen plan: 500 queries on 12500 keys, 32/8 heads,
   // 161 -> 96 us (cut); a decode step of batch 8 on 6001 keys, 32/8 heads, 82 -> 39 us (packed and cut);
   // 12 heads x 512 d64 11.8 -> 9.6 us, 16/4 heads x 2048 d128 35.2 -> 30.7 us (one query tile per item).
-  if (spread != Spread::kNone && drafts.size() < size_t(8 * num_ctas)) {
+  if (spread != Spread::kNone && !chosen && drafts.size() < size_t(8 * num_ctas)) {
     const double fill = double(std::min<int64_t>(rows_q, kTile)) / kTile;
     double work = 0.0;
     for (const Draft &d : drafts) work += step_cost(d.w) * d.w.n_steps + kItemOverheadSteps;
@@ -659,12 +717,21 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
   if (policy == 0) {
     const double kv_bytes_per_head = 2.0 * double(p->seq_kv) * p->head_dim * 2.0;
     int heads_per_wave = int(std::max(1.0, std::floor(double(kL2WaveBytes) / kv_bytes_per_head)));
-    auto wave_of = [&](const Draft &d) { return (int64_t(d.w.batch) * p->heads_kv + d.group) / heads_per_wave; };
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-      int64_t wa = wave_of(drafts[a]), wb = wave_of(drafts[b]);
-      if (wa != wb) return wa < wb;
-      return drafts[a].w.n_steps > drafts[b].w.n_steps;
+    struct Key {
+      int64_t wave;
+      int32_t n_steps, id;
+    };
+    std::vector<Key> keys(drafts.size());
+    for (size_t n = 0; n < keys.size(); ++n) {
+      const Draft &d = drafts[n];
+      keys[n] = Key{(int64_t(d.w.batch) * p->heads_kv + d.group) / heads_per_wave, d.w.n_steps, int32_t(n)};
+    }
+    std::sort(keys.begin(), keys.end(), [](const Key &a, const Key &b) {
+      if (a.wave != b.wave) return a.wave < b.wave;
+      if (a.n_steps != b.n_steps) return a.n_steps > b.n_steps;
+      return a.id < b.id;
     });
+    for (size_t n = 0; n < keys.size(); ++n) order[n] = keys[n].id;
   }
 
   // ---- assignment to persistent CTAs
@@ -707,6 +774,10 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
     }
   }
 
+  size_t n_steps = 0;
+  for (const Draft &d : drafts) n_steps += d.list.size();
+  plan->steps.reserve(n_steps);
+  plan->items.reserve(drafts.size());
   plan->grid = grid;
   plan->cta_begin.push_back(0);
   for (int cta = 0; cta < grid; ++cta) {
