@@ -547,11 +547,12 @@ __device__ __forceinline__ float *part_buffer(const KernelParams &p, int n) {
 }
 
 // Columns c0, c0 + step, ... of one row (in units of four columns): kCols of them from kBatch parts at a time.
+// Returns sum_i w_i l_i.
 template <int D, int kCols, int kBatch>
-__device__ __forceinline__ void combine_columns(const float4 *col, const float2 *stat, size_t stride, int part_rows,
-                                                int n_parts, int c0, int step, float m, float inv,
-                                                __nv_bfloat16 *o_row) {
+__device__ __forceinline__ float combine_columns(const float4 *col, const float2 *stat, size_t stride, int part_rows,
+                                                 int n_parts, int c0, int step, float m, __nv_bfloat16 *o_row) {
   float4 acc[kCols] = {};
+  float l = 0.0f;
 #pragma unroll 1
   for (int i0 = 0; i0 < n_parts; i0 += kBatch) {
     float2 ml[kBatch];
@@ -567,6 +568,7 @@ __device__ __forceinline__ void combine_columns(const float4 *col, const float2 
 #pragma unroll
     for (int b = 0; b < kBatch; ++b) {
       const float w = (ml[b].y > 0.0f && i0 + b < n_parts) ? ex2_approx(ml[b].x - m) : 0.0f;
+      l = fmaf(w, ml[b].y, l);
 #pragma unroll
       for (int k = 0; k < kCols; ++k) {
         acc[k].x = fmaf(w, v[b][k].x, acc[k].x);
@@ -576,11 +578,13 @@ __device__ __forceinline__ void combine_columns(const float4 *col, const float2 
       }
     }
   }
+  const float inv = l > 0.0f ? 1.0f / l : 0.0f;
 #pragma unroll
   for (int k = 0; k < kCols; ++k)
     if (c0 + k * step < D / 4)
       *reinterpret_cast<uint2 *>(o_row + (c0 + k * step) * 4) =
           make_uint2(pack_bf16x2(acc[k].x * inv, acc[k].y * inv), pack_bf16x2(acc[k].z * inv, acc[k].w * inv));
+  return l;
 }
 
 template <int D>
@@ -599,30 +603,25 @@ __device__ __forceinline__ void finish_part(const KernelParams &p, int split, in
   if (lane == 0) *counter = 0;  // for the next call
   // `lanes` lanes share a row: lane = row + rows * share
   const int rows = used > 16 ? 32 : used > 8 ? 16 : used > 4 ? 8 : used > 2 ? 4 : used > 1 ? 2 : 1, lanes = 32 / rows;
-  const int row = lane & (rows - 1), share = lane / rows;
-  if (row < used) {
-    const int r = warp * 32 + row;
-    const size_t stride = size_t(p.part_rows) * (D + 2);
-    const float *base = part_buffer<D>(p, tile.first);
-    const float2 *stat = reinterpret_cast<const float2 *>(base + size_t(D) * p.part_rows) + r;
-    constexpr int kBatch = 4;
-    float m = -CUDART_INF_F, l = 0.0f;
+  const int share = lane / rows;
+  const bool valid = (lane & (rows - 1)) < used;
+  const int r = warp * 32 + min(lane & (rows - 1), used - 1);
+  const size_t stride = size_t(p.part_rows) * (D + 2);
+  const float *base = part_buffer<D>(p, tile.first);
+  const float2 *stat = reinterpret_cast<const float2 *>(base + size_t(D) * p.part_rows) + r;
+  // max m: each lane of a row over its share of the parts, then over the lanes
+  float m = -CUDART_INF_F;
 #pragma unroll 1
-    for (int i0 = 0; i0 < tile.n_parts; i0 += kBatch) {
-      float2 ml[kBatch];
-      float top = m;
+  for (int i0 = share; i0 < tile.n_parts; i0 += 4 * lanes) {
+    float top[4];
 #pragma unroll
-      for (int b = 0; b < kBatch; ++b) {
-        ml[b] = __ldcg(stat + min(i0 + b, tile.n_parts - 1) * (stride / 2));
-        if (i0 + b >= tile.n_parts) ml[b].y = 0.0f;
-        top = fmaxf(top, ml[b].x);
-      }
-      l = l > 0.0f ? l * ex2_approx(m - top) : 0.0f;
-#pragma unroll
-      for (int b = 0; b < kBatch; ++b) l += ml[b].y > 0.0f ? ml[b].y * ex2_approx(ml[b].x - top) : 0.0f;
-      m = top;
-    }
-    const float inv = l > 0.0f ? 1.0f / l : 0.0f;
+    for (int b = 0; b < 4; ++b) top[b] = __ldcg(stat + min(i0 + b * lanes, tile.n_parts - 1) * (stride / 2)).x;
+    m = fmax3(fmax3(m, top[0], top[1]), top[2], top[3]);
+  }
+#pragma unroll 1
+  for (int step = rows; step < 32; step *= 2) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, step));
+  if (valid) {
+    float l = 0.0f;
     const size_t out_row = tile_out_row + size_t(r);
     __nv_bfloat16 *o_row = static_cast<__nv_bfloat16 *>(p.o) + out_row * D;
     const float4 *col = reinterpret_cast<const float4 *>(base) + r;
@@ -631,11 +630,11 @@ __device__ __forceinline__ void finish_part(const KernelParams &p, int split, in
     if (lanes <= 4) {
 #pragma unroll 1
       for (int c0 = share; c0 < D / 4; c0 += 8 * lanes)
-        combine_columns<D, 8, 4>(col, stat, stride, p.part_rows, tile.n_parts, c0, lanes, m, inv, o_row);
+        l = combine_columns<D, 8, 4>(col, stat, stride, p.part_rows, tile.n_parts, c0, lanes, m, o_row);
     } else {
 #pragma unroll 1
       for (int c0 = share; c0 < D / 4; c0 += 4 * lanes)
-        combine_columns<D, 4, 4>(col, stat, stride, p.part_rows, tile.n_parts, c0, lanes, m, inv, o_row);
+        l = combine_columns<D, 4, 4>(col, stat, stride, p.part_rows, tile.n_parts, c0, lanes, m, o_row);
     }
     if (p.lse != nullptr && share == 0)
       p.lse[out_row] = l > 0.0f ? 0.6931471805599453f * (m + log2f(l)) : -CUDART_INF_F;
