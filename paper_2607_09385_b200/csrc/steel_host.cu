@@ -15,9 +15,13 @@
 #include "../../include/steel_attn.h"
 #include "steel_planner.h"
 
-// Host -> device copies go to these streams in turn: a copy's start-up (about 5 us) then overlaps the one before
-// it (32 heads x 4096, 8 chunks: 2.29 -> 2.24 ms).
-constexpr int kInStreams = 3;
+// Host -> device copies of large chunks go to kInStreams streams in turn, so that a copy's start-up (about 5 us)
+// overlaps the one before it; a chunk's copies wait for those of kInLag chunks earlier, so that the chunks still
+// arrive in order.  One stream -> three: 32 heads x 4096 2.28 -> 2.24 ms, 32/8 heads x 4096 1.55 -> 1.40 ms; but
+// 32/4 heads x 8192 1.28 -> 1.42 ms (with a Q so much larger than K and V the streams drift apart), and below
+// kInBytes per chunk the extra events cost more than the overlap saves (0.36 -> 0.38 ms): one stream there.
+constexpr int kInStreams = 3, kInLag = 2;
+constexpr size_t kInBytes = size_t(4) << 20, kInMostQ = 4;  // Q of at most kInMostQ times K
 
 struct steel_attn_host {
   steel_attn_params_t params{};
@@ -183,15 +187,20 @@ extern "C" steel_status_t steel_attn_host_run(steel_attn_host_t *h, const void *
   }
   // everything below starts after the work already queued on the caller's stream
   STEEL_HOST_CHECK(cudaEventRecord(h->ev_begin, user));
-  for (cudaStream_t s : h->s_in) STEEL_HOST_CHECK(cudaStreamWaitEvent(s, h->ev_begin, 0));
-  int copies = 0;  // host -> device copies go to the streams in turn
-  auto next_in = [&] { return h->s_in[copies++ % kInStreams]; };
+  const bool many = h->q_chunk_bytes + 2 * h->kv_chunk_bytes >= kInBytes && h->q_chunk_bytes <= kInMostQ * h->kv_chunk_bytes;
+  const int n_in = many ? kInStreams : 1;
+  int copies = 0;
+  for (int n = 0; n < n_in; ++n) STEEL_HOST_CHECK(cudaStreamWaitEvent(h->s_in[n], h->ev_begin, 0));
+  auto next_in = [&] { return h->s_in[copies++ % n_in]; };
   for (int c = 0; c < h->n_chunks; ++c) {
     const size_t qo = c * h->q_chunk_bytes, ko = c * h->kv_chunk_bytes, lo = c * h->lse_chunk_bytes;
+    for (int n = 0; n_in > 1 && c >= kInLag && n < n_in; ++n)
+      for (int k = 0; k < n_in; ++k)
+        STEEL_HOST_CHECK(cudaStreamWaitEvent(h->s_in[n], h->ev_in[(c - kInLag) * kInStreams + k], 0));
     STEEL_HOST_CHECK(cudaMemcpyAsync(h->dq + qo, hq + qo, h->q_chunk_bytes, cudaMemcpyHostToDevice, next_in()));
     STEEL_HOST_CHECK(cudaMemcpyAsync(h->dk + ko, hk + ko, h->kv_chunk_bytes, cudaMemcpyHostToDevice, next_in()));
     STEEL_HOST_CHECK(cudaMemcpyAsync(h->dv + ko, hv + ko, h->kv_chunk_bytes, cudaMemcpyHostToDevice, next_in()));
-    for (int n = 0; n < kInStreams; ++n) {
+    for (int n = 0; n < n_in; ++n) {
       STEEL_HOST_CHECK(cudaEventRecord(h->ev_in[c * kInStreams + n], h->s_in[n]));
       STEEL_HOST_CHECK(cudaStreamWaitEvent(h->s_run, h->ev_in[c * kInStreams + n], 0));
     }
