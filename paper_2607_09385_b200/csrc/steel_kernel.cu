@@ -568,7 +568,9 @@ __device__ __forceinline__ float combine_columns(const float4 *col, const float2
     }
 #pragma unroll
     for (int b = 0; b < kBatch; ++b) {
-      const float w = (ml[b].y > 0.0f && i0 + b < n_parts) ? ex2_approx(ml[b].x - m) : 0.0f;
+      // beyond the last part: not weight 0, because an infinite O would make a NaN of it
+      if (i0 + b >= n_parts) break;
+      const float w = ml[b].y > 0.0f ? ex2_approx(ml[b].x - m) : 0.0f;
       l = fmaf(w, ml[b].y, l);
 #pragma unroll
       for (int k = 0; k < kCols; ++k) {

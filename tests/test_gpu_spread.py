@@ -79,3 +79,28 @@ def test_interrupted_call_leaves_nothing_behind():
         assert attn.last_status() == B.STEEL_OK
         assert torch.equal(o2, o) and torch.equal(lse2, lse)
     attn.close()
+
+
+@pytest.mark.parametrize("case", [CASES[0], CASES[1], CASES[6]])  # 18, 6 and 8 parts per tile: batches of 4 and a rest
+@pytest.mark.parametrize("what", ["v", "q", "k"])
+def test_infinite_and_nan_operands_as_in_an_uncut_plan(case, what):
+    """One infinite value of V, one row of NaN in Q or in K: infinities and NaN of O and LSE do not depend on
+    the plan (policy 1 never packs or cuts)."""
+    attn, _, q, k, v = make(case)
+    b, hq, hkv, sq, skv, d, flags, window, emu = case
+    if what == "v":
+        v[0, 0, skv - sq, 3] = math.inf  # every query sees this key
+    elif what == "q":
+        q[0, 0, sq // 2] = math.nan
+    else:
+        k[0, 0, skv // 2] = math.nan
+    dev = [x.cuda() for x in (q, k, v)]
+    uncut = B.SteelAttention(b, hq, hkv, sq, skv, d, 1.0 / math.sqrt(d), flags, policy=1)
+    (o, lse), (o_ref, lse_ref) = attn.run(*dev), uncut.run(*dev)
+    assert attn.last_status() == B.STEEL_OK and uncut.last_status() == B.STEEL_OK
+    for x, y in ((o, o_ref), (lse, lse_ref)):
+        assert torch.equal(x.isnan(), y.isnan()) and torch.equal(x.isposinf(), y.isposinf())
+        assert torch.equal(x.isneginf(), y.isneginf())
+    assert o.isposinf().any() if what == "v" else o.isnan().any()
+    attn.close()
+    uncut.close()
