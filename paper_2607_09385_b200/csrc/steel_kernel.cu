@@ -560,16 +560,16 @@ __device__ __forceinline__ float combine_columns(const float4 *col, const float2
     float4 v[kBatch][kCols];
 #pragma unroll
     for (int b = 0; b < kBatch; ++b) {
-      const int i = min(i0 + b, n_parts - 1);
-      ml[b] = __ldcg(stat + i * (stride / 2));
+      // beyond the last part zeros, not another part with weight 0: where its O is infinite, that is a NaN
+      const bool in = i0 + b < n_parts;
+      ml[b] = in ? __ldcg(stat + (i0 + b) * (stride / 2)) : make_float2(0.0f, 0.0f);
 #pragma unroll
       for (int k = 0; k < kCols; ++k)
-        v[b][k] = __ldcg(col + i * (stride / 4) + size_t(min(c0 + k * step, D / 4 - 1)) * part_rows);
+        v[b][k] = in ? __ldcg(col + (i0 + b) * (stride / 4) + size_t(min(c0 + k * step, D / 4 - 1)) * part_rows)
+                     : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
 #pragma unroll
     for (int b = 0; b < kBatch; ++b) {
-      // beyond the last part: not weight 0, because an infinite O would make a NaN of it
-      if (i0 + b >= n_parts) break;
       const float w = ml[b].y > 0.0f ? ex2_approx(ml[b].x - m) : 0.0f;
       l = fmaf(w, ml[b].y, l);
 #pragma unroll
