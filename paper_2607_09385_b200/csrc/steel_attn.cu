@@ -241,10 +241,7 @@ steel_status_t steel_attn_last_status(steel_attn_t *h, void *cuda_stream) {
   if (cudaStreamSynchronize(stream) != cudaSuccess ||
       cudaMemcpy(&word, h->d_status, sizeof word, cudaMemcpyDeviceToHost) != cudaSuccess)
     return STEEL_ERR_CUDA;
-  // an interrupted call can leave some parts counted
-  if (word != 0 && (cudaMemset(h->d_status, 0, sizeof(int32_t)) != cudaSuccess ||
-                    (h->d_arrivals && cudaMemset(h->d_arrivals, 0, h->arrivals_bytes) != cudaSuccess)))
-    return STEEL_ERR_CUDA;
+  if (word != 0 && cudaMemset(h->d_status, 0, sizeof(int32_t)) != cudaSuccess) return STEEL_ERR_CUDA;
   return word == 0 ? STEEL_OK : STEEL_ERR_TIMEOUT;
 }
 

@@ -590,20 +590,39 @@ __device__ __forceinline__ float combine_columns(const float4 *col, const float2
   return l;
 }
 
-template <int D>
-__device__ __forceinline__ void finish_part(const KernelParams &p, int split, int tile_row0, size_t tile_out_row,
-                                            int warp, int lane) {
-  const int used = min(32, p.rows_q - tile_row0 - warp * 32);
-  if (used <= 0) return;
-  const SplitTile tile = p.split_tiles[split >> 6];
+// Count one part of a split tile as ended for this warp's 32 rows.  True for the warp that ends last, which sets
+// the counter back for the next launch.  Rows beyond the matrix are not counted (`used` <= 0).
+__device__ __forceinline__ bool count_part(const KernelParams &p, int split, int n_parts, int used, int warp, int lane) {
+  if (used <= 0) return false;
   int32_t *counter = p.arrivals + (split >> 6) * 4 + warp;
   __syncwarp();
   int before = 0;
   if (lane == 0) before = atomic_add_acq_rel(counter, 1);
   before = __shfl_sync(0xffffffffu, before, 0);
   __syncwarp();
-  if (before != tile.n_parts - 1) return;
-  if (lane == 0) *counter = 0;  // for the next call
+  if (before != n_parts - 1) return false;
+  if (lane == 0) *counter = 0;
+  return true;
+}
+
+// A warp that leaves on an expired wait counts the parts of its items from k on all the same: every launch then
+// counts every part once, and the counters are back at 0 for the next launch without any help from the host.
+// (What is combined in this launch is undefined, as its status says.)
+__device__ __noinline__ void count_abandoned_parts(const KernelParams &p, int k, int s, int warp, int lane) {
+  for (const int k_end = p.cta_begin[blockIdx.x + 1]; k < k_end; ++k) {
+    const Item w = load_item(p.items, k);
+    if (!w.active(s) || w.split(s) < 0) continue;
+    count_part(p, w.split(s), p.split_tiles[w.split(s) >> 6].n_parts, p.rows_q - w.qtile(s) * kTile - warp * 32, warp,
+               lane);
+  }
+}
+
+template <int D>
+__device__ __forceinline__ void finish_part(const KernelParams &p, int split, int tile_row0, size_t tile_out_row,
+                                            int warp, int lane) {
+  const int used = min(32, p.rows_q - tile_row0 - warp * 32);
+  const SplitTile tile = p.split_tiles[split >> 6];
+  if (!count_part(p, split, tile.n_parts, used, warp, lane)) return;
   // `lanes` lanes share a row: lane = row + rows * share
   const int rows = used > 16 ? 32 : used > 8 ? 16 : used > 4 ? 8 : used > 2 ? 4 : used > 1 ? 2 : 1, lanes = 32 / rows;
   const int share = lane / rows;
@@ -645,8 +664,9 @@ __device__ __forceinline__ void finish_part(const KernelParams &p, int split, in
   __syncwarp();
 }
 
+// Returns -1, or the item in which a wait expired.
 template <int D, int kEmu, bool kSplit, bool kList>
-__device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, const int r) {
+__device__ int softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, const int r) {
   using C = Cfg<D>;
   const int lane = r % 32;
   const uint32_t lane_base = uint32_t((r / 32) * 32) << 16;
@@ -699,7 +719,7 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
       {
         ok = warp_wait(&ctrl.s_full[s], n_sp & 1u, ctrl, p.status, lane);
       }
-      if (!ok) return;
+      if (!ok) return k;
       tc_fence_after();
 
       float x[kTile];
@@ -758,7 +778,7 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
         const bool need = ms > m_ref + kRescaleThreshold;
         if (__any_sync(0xffffffffu, need)) {
           // PV(s, t - 1) accumulates into O: it must have finished
-          if (!warp_wait(&ctrl.p_free[s], (n_sp - 1u) & 1u, ctrl, p.status, lane)) return;
+          if (!warp_wait(&ctrl.p_free[s], (n_sp - 1u) & 1u, ctrl, p.status, lane)) return k;
           tc_fence_after();
           const float v = need ? ex2_approx(m_ref - ms) : 1.0f;
           l *= v;
@@ -789,7 +809,7 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
           // head_dim 64 does all the same: its barrier is complete (or in its initial phase), and the loop is
           // faster without the test (32 heads x 8192 362 -> 355 us; at head_dim 128, 32/8 heads x 16384, slower:
           // 1622 -> 1638 us).
-          if (!warp_wait(&ctrl.p_free[s], (n_sp - 1u) & 1u, ctrl, p.status, lane)) return;
+          if (!warp_wait(&ctrl.p_free[s], (n_sp - 1u) & 1u, ctrl, p.status, lane)) return k;
           tc_fence_after();
         }
         tmem_st32(t_p + half * 32, packed);
@@ -811,7 +831,7 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
       {
         ok = warp_wait(&ctrl.o_full[s], n_use & 1u, ctrl, p.status, lane);
       }
-      if (!ok) return;
+      if (!ok) return k;
       ++n_use;
       tc_fence_after();
       const bool valid = row < p.rows_q;
@@ -867,6 +887,7 @@ __device__ void softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, con
       if (p.lse != nullptr) p.lse[out_row] = -CUDART_INF_F;
     }
   }
+  return -1;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -922,7 +943,8 @@ steel_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 
   if (warp < 8) {
     setmaxnreg_inc<kRegsSoftmax>();
-    softmax_role<D, kEmu, kSplit, kList>(p, ctrl, warp / 4, threadIdx.x % kTile);
+    const int left = softmax_role<D, kEmu, kSplit, kList>(p, ctrl, warp / 4, threadIdx.x % kTile);
+    if (kSplit && left >= 0) count_abandoned_parts(p, left, warp / 4, warp % 4, lane);
   } else {
     setmaxnreg_dec<kRegsOther>();
     if (warp == kProducerWarp) {

@@ -60,7 +60,7 @@ struct KernelParams {
   const SplitTile *split_tiles;  // null: no query tile is split
   float *parts;              // per part: O as float4 [head_dim / 4][part_rows], then (m, l) [part_rows]
   int32_t part_rows;         // rows of a query tile that can be used (128, or those of a shorter matrix), a multiple of 4
-  int32_t *arrivals;         // per split tile and row quarter: parts finished; zero between calls
+  int32_t *arrivals;         // per split tile and row quarter: parts finished; zero between launches
   // Q as [batch][heads_q][rows_q][head_dim]: `heads_q` matrices of rows_q = seq_q rows or, where a query
   // tile holds rows of several heads of a group, heads_kv matrices of group * seq_q rows
   int32_t heads_q, heads_kv, rows_q, seq_q, seq_kv;

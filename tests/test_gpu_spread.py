@@ -104,3 +104,25 @@ def test_infinite_and_nan_operands_as_in_an_uncut_plan(case, what):
     assert o.isposinf().any() if what == "v" else o.isnan().any()
     attn.close()
     uncut.close()
+
+
+@pytest.mark.parametrize("case", [CASES[0], CASES[6]])
+def test_calls_after_an_interrupted_one_need_no_repair(case):
+    """A call whose waits expire, others queued behind it before anyone asks for the status: those are right."""
+    attn, _, q, k, v = make(case)
+    dev = [x.cuda() for x in (q, k, v)]
+    o, lse = attn.run(*dev)
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream):
+        for cta in (3, 0):
+            B.steel_attn_debug_stall(attn.handle, cta, 200_000_000)  # 0.1 s
+            attn.run(*dev)
+            B.steel_attn_debug_stall(attn.handle, -1)
+            later = [attn.run(*dev) for _ in range(3)]
+            assert attn.last_status() == B.STEEL_ERR_TIMEOUT
+            later += [attn.run(*dev) for _ in range(2)]
+            assert attn.last_status() == B.STEEL_OK
+            for o2, lse2 in later:
+                assert torch.equal(o2, o) and torch.equal(lse2, lse)
+    attn.close()
