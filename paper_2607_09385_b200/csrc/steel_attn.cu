@@ -237,11 +237,15 @@ steel_status_t steel_attn_run(steel_attn_t *h, const void *q, const void *k, con
 steel_status_t steel_attn_last_status(steel_attn_t *h, void *cuda_stream) {
   if (!h) return STEEL_ERR_INVALID_ARG;
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+  // Read and clear on `stream` alone, and wait for both: on the default stream they would wait for work that is not
+  // the handle's, and a clear that nothing orders before the handle's next run could take that run's status away.
   int32_t word = 0;
-  if (cudaStreamSynchronize(stream) != cudaSuccess ||
-      cudaMemcpy(&word, h->d_status, sizeof word, cudaMemcpyDeviceToHost) != cudaSuccess)
+  if (cudaMemcpyAsync(&word, h->d_status, sizeof word, cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+      cudaStreamSynchronize(stream) != cudaSuccess)
     return STEEL_ERR_CUDA;
-  if (word != 0 && cudaMemset(h->d_status, 0, sizeof(int32_t)) != cudaSuccess) return STEEL_ERR_CUDA;
+  if (word != 0 && (cudaMemsetAsync(h->d_status, 0, sizeof(int32_t), stream) != cudaSuccess ||
+                    cudaStreamSynchronize(stream) != cudaSuccess))
+    return STEEL_ERR_CUDA;
   return word == 0 ? STEEL_OK : STEEL_ERR_TIMEOUT;
 }
 

@@ -35,3 +35,26 @@ def test_wait_expiry_sets_status_and_context_stays_usable():
     with pytest.raises(binding.SteelError):
         binding.steel_attn_debug_stall(attn.handle, 10_000, 0)     # no such CTA
     attn.close()
+
+
+def test_status_is_read_and_cleared_on_its_own_stream():
+    """last_status on a side stream neither waits for nor is ordered with work on the default stream."""
+    w = inputs.Workload("stall_side", 1, 4, 2, 1024, 128, 128, inputs.MASK_CAUSAL)
+    data = inputs.make_inputs(w, seed=92)
+    attn = H.make_attention(w)
+    q, k, v = (H.to_device(data[x]) for x in "qkv")
+    o = torch.empty_like(q)
+    torch.cuda.synchronize()
+    side, busy = torch.cuda.Stream(), torch.cuda.Event()
+    for stalled in (True, False, True):
+        binding.steel_attn_debug_stall(attn.handle, 0 if stalled else -1, 50_000_000)
+        torch.cuda._sleep(2_000_000_000)                   # about a second of the default stream
+        busy.record()
+        with torch.cuda.stream(side):
+            attn.run(q, k, v, o, want_lse=False)
+            status = attn.last_status()
+        assert not busy.query()
+        assert status == (binding.STEEL_ERR_TIMEOUT if stalled else binding.STEEL_OK)
+        torch.cuda.synchronize()
+    binding.steel_attn_debug_stall(attn.handle, -1)
+    attn.close()
