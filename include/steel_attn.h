@@ -31,8 +31,9 @@
  * Ownership and threading: every tensor pointer is a DEVICE pointer owned by the caller,
  * 16-byte aligned, and must stay valid until the stream has executed the call.  The bitmap
  * is a HOST pointer read only during steel_attn_create.  A handle owns its device work lists
- * and status word; it is bound to the device that was current at create time and must
- * not be used by two streams at once.  All functions return a status code; nothing throws,
+ * and status word; it is bound to the device that was current at create time.  Its runs may be
+ * queued on several streams and captured into graphs (see steel_attn_run); calls on one handle
+ * from several host threads must be serialised by the caller.  All functions return a status code; nothing throws,
  * aborts or traps.  There is no CPU fallback: without a usable CUDA device the run fails.
  */
 #ifndef STEEL_ATTN_H_
@@ -122,10 +123,18 @@ steel_status_t steel_attn_create(const steel_attn_params_t *params, steel_attn_t
 /*
  * Enqueue one attention call (Eq. 1, computed as Algorithm 1 over the handle's work lists) on `cuda_stream` (a cudaStream_t cast to void*; NULL = default
  * stream).  q, k, v, o: device bf16 tensors in the layouts above; lse: device float32 or
- * NULL.  Asynchronous: no allocation, no host synchronisation.  One persistent kernel is
+ * NULL.  Asynchronous: no host synchronisation, no allocation except as below.  One persistent kernel is
  * launched; device-side waits are bounded and, if one expires, the kernel stops and the
  * error is reported by steel_attn_last_status.  STEEL_ERR_INVALID_ARG also if the current device
  * is not the one the handle was created on.
+ *
+ * Runs of one handle may overlap.  Where the plan cuts key ranges, launches that could overlap use
+ * different part buffers: those made by create serve the first stream; the first run on another stream
+ * allocates one more set, and an event keeps the runs of all streams but the first apart; each stream of
+ * a capture gets a set at its first captured run (up to 30 sets and 64 MiB per handle, kept until destroy;
+ * beyond that, or without memory, a run takes the plan without cuts: slower, and equal within rounding).
+ * The captured launches keep using the handle's memory, and two executable graphs made from ONE capture
+ * share its set, so those two must not be replayed at the same time.
  */
 steel_status_t steel_attn_run(steel_attn_t *handle, const void *q, const void *k, const void *v,
                               void *o, float *lse, void *cuda_stream);

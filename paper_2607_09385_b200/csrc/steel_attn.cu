@@ -5,7 +5,9 @@
 #include <algorithm>
 #include <cstring>
 #include <limits>
+#include <mutex>
 #include <new>
+#include <vector>
 
 #include "../../include/steel_attn.h"
 #include "steel_kernel.h"
@@ -15,21 +17,45 @@ using namespace steel;
 
 static_assert(sizeof(steel_mask_desc_t) == 32 && sizeof(steel_attn_params_t) == 72, "public struct layout");
 
+// Cut plans: the parts of a launch are left in buffers and counted in counters.  Launches that may overlap must
+// not share them, so a handle has several sets: one for the stream that it was first run on; one for all its other
+// streams, whose launches an event keeps apart; and one for each sequence of captured launches (one stream in one
+// capture), because a graph replays them at any time beside anything else.  A launch for which there is no set
+// runs the plan without cuts, which leaves nothing on the device.
+constexpr int kHomeSet = 0, kRoamingSet = 1, kFirstCapturedSet = 2, kMaxPartSets = 32;
+constexpr size_t kCapturedPartBytes = size_t(64) << 20;  // part buffers of all captured sequences of a handle
+
+struct PartSet {
+  float *parts = nullptr;
+  unsigned long long stream = 0, capture = 0;  // who uses it: a stream's id, or its handle and the capture's id
+  bool used = false;
+};
+
+struct DeviceLists {  // a plan's lists in device memory
+  WorkItem *items = nullptr;
+  int32_t *cta_begin = nullptr;
+  StepPair *steps = nullptr;
+  int grid = 0;
+  bool overlap_launch = false;
+};
+
 struct steel_attn {
   steel_attn_params_t params;
   steel_attn_stats_t stats;
   int device = -1;
-  int grid = 0;
-  WorkItem *d_items = nullptr;
-  int32_t *d_cta_begin = nullptr;
-  StepPair *d_steps = nullptr;
+  unsigned char *d_lists = nullptr;  // one allocation: everything below except the part buffers
+  DeviceLists plan, whole;           // `whole`: the plan without cuts, where `plan` cuts key ranges
   int32_t *d_status = nullptr;
   SplitTile *d_split_tiles = nullptr;  // null: no query tile is split
-  int32_t *d_arrivals = nullptr;
-  size_t arrivals_bytes = 0;
-  float *d_parts = nullptr;
+  int32_t *d_arrivals = nullptr;       // counters of kMaxPartSets sets, n_split * 4 each
+  size_t n_split = 0;
+  size_t part_bytes = 0;
   int32_t part_rows = 0;
   bool packed = false;
+  std::mutex parts_lock;  // held from the choice of a set to the end of the launch's record
+  PartSet sets[kMaxPartSets];
+  int n_sets = kFirstCapturedSet;
+  cudaEvent_t roaming_done = nullptr;  // after the last launch with the roaming set
   long long *d_clock_probe = nullptr;
   long long timeout_cycles = kDefaultTimeoutCycles;
   int32_t stall_cta = -1;
@@ -73,13 +99,98 @@ bool make_map(CUtensorMap *map, const void *base, int head_dim, int64_t rows, in
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 void free_device(steel_attn *h) {
-  if (h->d_items) cudaFree(h->d_items);
-  if (h->d_cta_begin) cudaFree(h->d_cta_begin);
-  if (h->d_steps) cudaFree(h->d_steps);
-  if (h->d_status) cudaFree(h->d_status);
-  if (h->d_split_tiles) cudaFree(h->d_split_tiles);
-  if (h->d_arrivals) cudaFree(h->d_arrivals);
-  if (h->d_parts) cudaFree(h->d_parts);
+  if (h->d_lists) cudaFree(h->d_lists);
+  for (PartSet &set : h->sets)
+    if (set.parts) cudaFree(set.parts);
+  if (h->roaming_done) cudaEventDestroy(h->roaming_done);
+}
+
+constexpr size_t round16(size_t n) { return (n + 15) / 16 * 16; }
+
+// Append a plan's lists to `image`; `lists` receives offsets, which place_lists makes addresses.
+void append_lists(const Plan &plan, std::vector<unsigned char> *image, DeviceLists *lists) {
+  auto put = [image](const void *data, size_t bytes) {
+    const size_t at = image->size();
+    image->resize(at + round16(bytes));
+    if (bytes) std::memcpy(image->data() + at, data, bytes);
+    return at;
+  };
+  lists->cta_begin = reinterpret_cast<int32_t *>(put(plan.cta_begin.data(), plan.cta_begin.size() * sizeof(int32_t)));
+  lists->items = reinterpret_cast<WorkItem *>(put(plan.items.data(), plan.items.size() * sizeof(WorkItem)));
+  lists->steps = reinterpret_cast<StepPair *>(put(plan.steps.data(), plan.steps.size() * sizeof(StepPair)));
+  lists->grid = plan.grid;
+  lists->overlap_launch = plan.stats.max_cta_steps <= kOverlapSteps;
+}
+
+template <class T>
+void place(T **offset, unsigned char *base) {
+  *offset = reinterpret_cast<T *>(base + reinterpret_cast<uintptr_t>(*offset));
+}
+void place_lists(DeviceLists *lists, unsigned char *base) {
+  place(&lists->cta_begin, base);
+  place(&lists->items, base);
+  place(&lists->steps, base);
+}
+
+// cudaMalloc that is also possible while a stream is captured (the allocation is not part of the capture).
+bool allocate_parts(steel_attn *h, PartSet *set) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
+  const bool ok = cudaMalloc(&set->parts, h->part_bytes) == cudaSuccess;
+  if (!ok) {
+    cudaGetLastError();
+    set->parts = nullptr;
+  }
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return ok;
+}
+
+// The set for a launch on `stream`, or -1: none is left, or nothing can be said about the stream.
+int take_part_set(steel_attn *h, cudaStream_t stream) {
+  unsigned long long id = 0, capture = 0;
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamGetCaptureInfo(stream, &status, &capture) != cudaSuccess) {
+    cudaGetLastError();
+    return -1;
+  }
+  if (status == cudaStreamCaptureStatusNone) {
+    // ids, not handles: the handle of a destroyed stream, whose work may still run, can come back.  (Asking for
+    // the id of a stream that is being captured would end the capture.)
+    if (cudaStreamGetId(stream, &id) != cudaSuccess) {
+      cudaGetLastError();
+      return -1;
+    }
+    PartSet &home = h->sets[kHomeSet], &roaming = h->sets[kRoamingSet];
+    if (!home.used) {
+      home.used = true;
+      home.stream = id;
+    }
+    if (home.stream == id) return kHomeSet;
+    if (!h->roaming_done && cudaEventCreateWithFlags(&h->roaming_done, cudaEventDisableTiming) != cudaSuccess) {
+      cudaGetLastError();
+      h->roaming_done = nullptr;
+      return -1;
+    }
+    if (!roaming.parts && !allocate_parts(h, &roaming)) return -1;
+    if (roaming.used && roaming.stream != id && cudaStreamWaitEvent(stream, h->roaming_done, 0) != cudaSuccess) {
+      cudaGetLastError();
+      return -1;
+    }
+    roaming.used = true;
+    roaming.stream = id;
+    return kRoamingSet;
+  }
+  if (status != cudaStreamCaptureStatusActive) return -1;
+  id = reinterpret_cast<uintptr_t>(stream);  // within one capture the handle says enough
+  for (int n = kFirstCapturedSet; n < h->n_sets; ++n)
+    if (h->sets[n].capture == capture && h->sets[n].stream == id) return n;
+  const size_t captured = size_t(h->n_sets - kFirstCapturedSet) * h->part_bytes;
+  if (h->n_sets == kMaxPartSets || captured + h->part_bytes > kCapturedPartBytes) return -1;
+  PartSet &set = h->sets[h->n_sets];
+  if (!allocate_parts(h, &set)) return -1;
+  set.stream = id;
+  set.capture = capture;
+  return h->n_sets++;
 }
 
 }  // namespace
@@ -138,60 +249,60 @@ steel_status_t create_attention(const steel_attn_params_t *params, Spread most, 
 
   steel_attn *h = new (std::nothrow) steel_attn();
   if (!h) return STEEL_ERR_ALLOC;
-  Plan plan;
-  for (Spread spread : {most, Spread::kTiles}) {  // the second only without memory for the first's part buffers
-    try {
-      st = build_plan(params, prop.multiProcessorCount, &plan, /*stats=*/true, spread);
-    } catch (const std::bad_alloc &) {
-      st = STEEL_ERR_ALLOC;
+  Plan plan, whole;
+  std::vector<unsigned char> image;
+  try {
+    for (Spread spread : {most, Spread::kTiles}) {  // the second only without memory for the first's part buffers
+      whole = Plan();
+      st = build_plan(params, prop.multiProcessorCount, &plan, /*stats=*/true, spread, &whole);
+      if (st != STEEL_OK) {
+        delete h;
+        return st;
+      }
+      if (plan.split_tiles.empty()) break;
+      // part buffers; without memory for them the key ranges stay whole.  Rows in multiples of four: every
+      // part's buffer then starts on a 16-byte boundary.
+      h->part_rows = int32_t(std::min<int64_t>((plan_rows_q(*params, plan) + 3) / 4 * 4, kTile));
+      h->part_bytes = size_t(plan.n_parts) * size_t(h->part_rows) * size_t(params->head_dim + 2) * sizeof(float);
+      if (allocate_parts(h, &h->sets[kHomeSet])) break;
     }
-    if (st != STEEL_OK) {
-      delete h;
-      return st;
-    }
-    if (plan.split_tiles.empty()) break;
-    // part buffers; without memory for them the key ranges stay whole.  Rows in multiples of four: every
-    // part's buffer then starts on a 16-byte boundary.
-    h->part_rows = int32_t(std::min<int64_t>((plan_rows_q(*params, plan) + 3) / 4 * 4, kTile));
-    const size_t part_bytes = size_t(plan.n_parts) * size_t(h->part_rows) * size_t(params->head_dim + 2) * sizeof(float);
-    if (cudaMalloc(&h->d_parts, part_bytes) == cudaSuccess) break;
-    cudaGetLastError();
-    h->d_parts = nullptr;
+    // one image of status word, counters (both zero) and lists
+    h->n_split = plan.split_tiles.size();
+    const size_t at_arrivals = 256;
+    image.resize(at_arrivals + round16(h->n_split * 4 * sizeof(int32_t) * kMaxPartSets));
+    h->d_split_tiles = reinterpret_cast<SplitTile *>(image.size());
+    image.resize(image.size() + round16(h->n_split * sizeof(SplitTile)));
+    if (h->n_split)
+      std::memcpy(image.data() + reinterpret_cast<uintptr_t>(h->d_split_tiles), plan.split_tiles.data(),
+                  h->n_split * sizeof(SplitTile));
+    append_lists(plan, &image, &h->plan);
+    if (h->n_split) append_lists(whole, &image, &h->whole);
+    h->d_arrivals = reinterpret_cast<int32_t *>(at_arrivals);
+  } catch (const std::bad_alloc &) {
+    free_device(h);
+    delete h;
+    return STEEL_ERR_ALLOC;
   }
   h->params = *params;
   h->params.mask.bitmap = nullptr;  // the caller's bitmap is not referenced after create
   h->stats = plan.stats;
   h->device = device;
-  h->grid = plan.grid;
   h->packed = plan.packed;
-  const size_t n_split = plan.split_tiles.size();
-  h->arrivals_bytes = n_split * 4 * sizeof(int32_t);
-
-  const size_t n_items = plan.items.size() ? plan.items.size() : 1, n_steps = plan.steps.size() ? plan.steps.size() : 1;
-  bool ok = cudaMalloc(&h->d_items, n_items * sizeof(WorkItem)) == cudaSuccess &&
-            cudaMalloc(&h->d_cta_begin, plan.cta_begin.size() * sizeof(int32_t)) == cudaSuccess &&
-            cudaMalloc(&h->d_steps, n_steps * sizeof(StepPair)) == cudaSuccess &&
-            cudaMalloc(&h->d_status, sizeof(int32_t)) == cudaSuccess &&
-            (n_split == 0 || (cudaMalloc(&h->d_split_tiles, n_split * sizeof(SplitTile)) == cudaSuccess &&
-                              cudaMalloc(&h->d_arrivals, h->arrivals_bytes) == cudaSuccess));
-  if (!ok) {
+  if (cudaMalloc(&h->d_lists, image.size()) != cudaSuccess) {
     cudaGetLastError();
+    h->d_lists = nullptr;
     free_device(h);
     delete h;
     return STEEL_ERR_ALLOC;
   }
-  ok = (plan.items.empty() || cudaMemcpy(h->d_items, plan.items.data(), plan.items.size() * sizeof(WorkItem),
-                                         cudaMemcpyHostToDevice) == cudaSuccess) &&
-       cudaMemcpy(h->d_cta_begin, plan.cta_begin.data(), plan.cta_begin.size() * sizeof(int32_t),
-                  cudaMemcpyHostToDevice) == cudaSuccess &&
-       (plan.steps.empty() || cudaMemcpy(h->d_steps, plan.steps.data(), plan.steps.size() * sizeof(StepPair),
-                                         cudaMemcpyHostToDevice) == cudaSuccess) &&
-       (n_split == 0 || (cudaMemcpy(h->d_split_tiles, plan.split_tiles.data(), n_split * sizeof(SplitTile),
-                                    cudaMemcpyHostToDevice) == cudaSuccess &&
-                         cudaMemset(h->d_arrivals, 0, h->arrivals_bytes) == cudaSuccess)) &&
-       cudaMemset(h->d_status, 0, sizeof(int32_t)) == cudaSuccess && configure_kernels() == cudaSuccess &&
-       cudaDeviceSynchronize() == cudaSuccess;
-  if (!ok || !encode_fn()) {
+  h->d_status = reinterpret_cast<int32_t *>(h->d_lists);
+  place(&h->d_arrivals, h->d_lists);
+  place(&h->d_split_tiles, h->d_lists);
+  if (h->n_split == 0) h->d_split_tiles = nullptr;
+  place_lists(&h->plan, h->d_lists);
+  place_lists(&h->whole, h->d_lists);
+  if (cudaMemcpy(h->d_lists, image.data(), image.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+      configure_kernels() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess || !encode_fn()) {
     cudaGetLastError();
     free_device(h);
     delete h;
@@ -217,21 +328,35 @@ steel_status_t steel_attn_run(steel_attn_t *h, const void *q, const void *k, con
   int device = -1;
   if (cudaGetDevice(&device) != cudaSuccess) return STEEL_ERR_CUDA;
   if (device != h->device) return STEEL_ERR_INVALID_ARG;  // the work lists live on the create-time device
+  cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   KernelParams kp{};
-  kp.items = h->d_items;
-  kp.cta_begin = h->d_cta_begin;
-  kp.steps = h->d_steps;
   kp.status = h->d_status;
-  kp.split_tiles = h->d_split_tiles;
-  kp.parts = h->d_parts;
-  kp.part_rows = h->part_rows;
-  kp.arrivals = h->d_arrivals;
   set_query_view(h->params, h->packed, &kp);
-  kp.overlap_launch = h->stats.max_cta_steps <= kOverlapSteps;
   kp.clock_probe = h->d_clock_probe;
   kp.timeout_cycles = h->timeout_cycles;
   kp.stall_cta = h->stall_cta;
-  return launch_with_params(h->params, kp, h->grid, q, k, v, o, lse, static_cast<cudaStream_t>(cuda_stream), &h->maps);
+  auto launch = [&](const DeviceLists &lists) {
+    kp.items = lists.items;
+    kp.cta_begin = lists.cta_begin;
+    kp.steps = lists.steps;
+    kp.overlap_launch = lists.overlap_launch;
+    return launch_with_params(h->params, kp, lists.grid, q, k, v, o, lse, stream, &h->maps);
+  };
+  if (!h->d_split_tiles) return launch(h->plan);
+  std::lock_guard<std::mutex> lock(h->parts_lock);
+  const int set = take_part_set(h, stream);
+  if (set < 0) return launch(h->whole);
+  kp.split_tiles = h->d_split_tiles;
+  kp.parts = h->sets[set].parts;
+  kp.part_rows = h->part_rows;
+  kp.arrivals = h->d_arrivals + size_t(set) * h->n_split * 4;
+  const steel_status_t st = launch(h->plan);
+  if (set == kRoamingSet && cudaEventRecord(h->roaming_done, stream) != cudaSuccess) {
+    cudaGetLastError();
+    cudaStreamSynchronize(stream);  // in place of the event
+    return STEEL_ERR_CUDA;
+  }
+  return st;
 }
 
 steel_status_t steel_attn_last_status(steel_attn_t *h, void *cuda_stream) {
@@ -301,7 +426,7 @@ steel_status_t steel_attn_debug_clock_probe(steel_attn_t *h, int64_t *device_pai
 }
 
 steel_status_t steel_attn_debug_stall(steel_attn_t *h, int32_t cta, int64_t timeout_cycles) {
-  if (!h || cta >= h->grid) return STEEL_ERR_INVALID_ARG;
+  if (!h || cta >= h->plan.grid) return STEEL_ERR_INVALID_ARG;
   h->stall_cta = cta < 0 ? -1 : cta;
   h->timeout_cycles = timeout_cycles > 0 ? timeout_cycles : kDefaultTimeoutCycles;
   return STEEL_OK;

@@ -332,6 +332,107 @@ double cut_over_ctas(const std::vector<Draft> &drafts, int num_ctas, double fill
   return *std::max_element(load.begin(), load.end()) + combine_steps(fill, most_parts);
 }
 
+// Order the drafts, assign them to CTAs and write the plan's lists and the statistics of its items.
+steel_status_t place_items(const steel_attn_params_t &p, int num_ctas, std::vector<Draft> &drafts, Plan *plan) {
+  // ---- order: waves of KV heads whose K and V fit comfortably in L2, longest item first inside
+  // a wave (policy 0); natural order (policy 1)
+  std::vector<int> order(drafts.size());
+  for (size_t n = 0; n < order.size(); ++n) order[n] = int(n);
+  const int policy = p.policy;
+  if (policy == 0) {
+    const double kv_bytes_per_head = 2.0 * double(p.seq_kv) * p.head_dim * 2.0;
+    int heads_per_wave = int(std::max(1.0, std::floor(double(kL2WaveBytes) / kv_bytes_per_head)));
+    struct Key {
+      int64_t wave;
+      int32_t n_steps, id;
+    };
+    std::vector<Key> keys(drafts.size());
+    for (size_t n = 0; n < keys.size(); ++n) {
+      const Draft &d = drafts[n];
+      keys[n] = Key{(int64_t(d.w.batch) * p.heads_kv + d.group) / heads_per_wave, d.w.n_steps, int32_t(n)};
+    }
+    std::sort(keys.begin(), keys.end(), [](const Key &a, const Key &b) {
+      if (a.wave != b.wave) return a.wave < b.wave;
+      if (a.n_steps != b.n_steps) return a.n_steps > b.n_steps;
+      return a.id < b.id;
+    });
+    for (size_t n = 0; n < keys.size(); ++n) order[n] = keys[n].id;
+  }
+
+  // ---- assignment to persistent CTAs
+  int grid = int(std::min<size_t>(size_t(num_ctas), std::max<size_t>(drafts.size(), 1)));
+  std::vector<std::vector<int>> per_cta(grid);
+  std::vector<int64_t> load(grid, 0);
+  if (!plan->split_tiles.empty()) {
+    grid = num_ctas;
+    per_cta.resize(grid);
+    load.resize(grid, 0);
+    for (size_t id = 0; id < drafts.size(); ++id) per_cta[drafts[id].cta].push_back(int(id));
+  } else if (policy == 0) {
+    // greedy longest-processing-time: next item goes to the least loaded CTA
+    typedef std::pair<int64_t, int> Slot;
+    std::priority_queue<Slot, std::vector<Slot>, std::greater<Slot>> heap;
+    for (int cta = 0; cta < grid; ++cta) heap.push(Slot(0, cta));
+    for (int id : order) {
+      Slot sl = heap.top();
+      heap.pop();
+      per_cta[sl.second].push_back(id);
+      sl.first += drafts[id].w.n_steps + kItemOverheadSteps;
+      load[sl.second] = sl.first;
+      heap.push(sl);
+    }
+  } else if (policy == 1) {
+    // uniform placement: contiguous chunks of the natural order
+    size_t n = order.size();
+    for (size_t k = 0; k < n; ++k) {
+      int cta = int(k * size_t(grid) / std::max<size_t>(n, 1));
+      per_cta[cta].push_back(order[k]);
+      load[cta] += drafts[order[k]].w.n_steps + kItemOverheadSteps;
+    }
+  } else {
+    // interleaved placement: consecutive items of the natural order go to consecutive CTAs, so
+    // that CTAs working side by side hold query tiles of similar sparsity
+    for (size_t k = 0; k < order.size(); ++k) {
+      int cta = int(k % size_t(grid));
+      per_cta[cta].push_back(order[k]);
+      load[cta] += drafts[order[k]].w.n_steps + kItemOverheadSteps;
+    }
+  }
+
+  size_t n_steps = 0;
+  for (const Draft &d : drafts) n_steps += d.list.size();
+  plan->steps.reserve(n_steps);
+  plan->items.reserve(drafts.size());
+  plan->grid = grid;
+  plan->cta_begin.push_back(0);
+  for (int cta = 0; cta < grid; ++cta) {
+    for (int id : per_cta[cta]) {
+      Draft &d = drafts[id];
+      if (d.w.kind == 1) {
+        d.w.j0[0] = int32_t(plan->steps.size());
+        plan->steps.insert(plan->steps.end(), d.list.begin(), d.list.end());
+      }
+      plan->items.push_back(d.w);
+    }
+    plan->cta_begin.push_back(int32_t(plan->items.size()));
+  }
+  if (plan->steps.size() >= (size_t(1) << 31)) return STEEL_ERR_UNSUPPORTED;
+
+  // ---- statistics of the executed plan
+  steel_attn_stats_t &s = plan->stats;
+  s.work_items = int64_t(plan->items.size());
+  s.grid = grid;
+  s.list_entries = int64_t(plan->steps.size());
+  s.max_cta_steps = 0;
+  for (int cta = 0; cta < grid; ++cta) {
+    int64_t st_sum = 0;
+    for (int id : per_cta[cta]) st_sum += drafts[id].w.n_steps;
+    s.max_cta_steps = std::max(s.max_cta_steps, st_sum);
+  }
+  for (const WorkItem &w : plan->items) s.steps += w.n_steps;
+  return STEEL_OK;
+}
+
 }  // namespace
 
 steel_status_t validate_params(const steel_attn_params_t *p) {
@@ -356,7 +457,8 @@ steel_status_t validate_params(const steel_attn_params_t *p) {
   return STEEL_OK;
 }
 
-steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan, bool stats, Spread spread) {
+steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan, bool stats, Spread spread,
+                          Plan *whole) {
   steel_status_t st = validate_params(p);
   if (st != STEEL_OK) return st;
   const int policy = p->policy;
@@ -476,7 +578,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
     for (Task &t : row) t.entries.first = entries.data() + t.entries.at;
 
   // ---- work items: pair query tiles that can share K/V loads
-  std::vector<Draft> drafts;
+  std::vector<Draft> drafts, uncut;  // `uncut`: for `whole`
   bool pair = true;
   auto finish_range = [&](const Task *a, const Task *b, int batch, int g) {
     Draft d{};
@@ -700,116 +802,31 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
           plan->n_parts = cut.n_parts;
         }
       }
-      if (makespan(singles, num_ctas) < best) {
+      const double single = makespan(singles, num_ctas);
+      if (single < best) {
         drafts.swap(singles);
         plan->split_tiles.clear();
         plan->n_parts = 0;
       } else if (drafts.empty()) {
         drafts.swap(paired_drafts);
+      } else {
+        uncut.swap(single < 0.95 * paired ? singles : paired_drafts);
       }
     }
   }
 
-  // ---- order: waves of KV heads whose K and V fit comfortably in L2, longest item first inside
-  // a wave (policy 0); natural order (policy 1)
-  std::vector<int> order(drafts.size());
-  for (size_t n = 0; n < order.size(); ++n) order[n] = int(n);
-  if (policy == 0) {
-    const double kv_bytes_per_head = 2.0 * double(p->seq_kv) * p->head_dim * 2.0;
-    int heads_per_wave = int(std::max(1.0, std::floor(double(kL2WaveBytes) / kv_bytes_per_head)));
-    struct Key {
-      int64_t wave;
-      int32_t n_steps, id;
-    };
-    std::vector<Key> keys(drafts.size());
-    for (size_t n = 0; n < keys.size(); ++n) {
-      const Draft &d = drafts[n];
-      keys[n] = Key{(int64_t(d.w.batch) * p->heads_kv + d.group) / heads_per_wave, d.w.n_steps, int32_t(n)};
-    }
-    std::sort(keys.begin(), keys.end(), [](const Key &a, const Key &b) {
-      if (a.wave != b.wave) return a.wave < b.wave;
-      if (a.n_steps != b.n_steps) return a.n_steps > b.n_steps;
-      return a.id < b.id;
-    });
-    for (size_t n = 0; n < keys.size(); ++n) order[n] = keys[n].id;
+  st = place_items(*p, num_ctas, drafts, plan);
+  if (st == STEEL_OK && whole && !plan->split_tiles.empty()) {
+    whole->packed = plan->packed;
+    st = place_items(*p, num_ctas, uncut, whole);
   }
-
-  // ---- assignment to persistent CTAs
-  int grid = int(std::min<size_t>(size_t(num_ctas), std::max<size_t>(drafts.size(), 1)));
-  std::vector<std::vector<int>> per_cta(grid);
-  std::vector<int64_t> load(grid, 0);
-  if (!plan->split_tiles.empty()) {
-    grid = num_ctas;
-    per_cta.resize(grid);
-    load.resize(grid, 0);
-    for (size_t id = 0; id < drafts.size(); ++id) per_cta[drafts[id].cta].push_back(int(id));
-  } else if (policy == 0) {
-    // greedy longest-processing-time: next item goes to the least loaded CTA
-    typedef std::pair<int64_t, int> Slot;
-    std::priority_queue<Slot, std::vector<Slot>, std::greater<Slot>> heap;
-    for (int cta = 0; cta < grid; ++cta) heap.push(Slot(0, cta));
-    for (int id : order) {
-      Slot sl = heap.top();
-      heap.pop();
-      per_cta[sl.second].push_back(id);
-      sl.first += drafts[id].w.n_steps + kItemOverheadSteps;
-      load[sl.second] = sl.first;
-      heap.push(sl);
-    }
-  } else if (policy == 1) {
-    // uniform placement: contiguous chunks of the natural order
-    size_t n = order.size();
-    for (size_t k = 0; k < n; ++k) {
-      int cta = int(k * size_t(grid) / std::max<size_t>(n, 1));
-      per_cta[cta].push_back(order[k]);
-      load[cta] += drafts[order[k]].w.n_steps + kItemOverheadSteps;
-    }
-  } else {
-    // interleaved placement: consecutive items of the natural order go to consecutive CTAs, so
-    // that CTAs working side by side hold query tiles of similar sparsity
-    for (size_t k = 0; k < order.size(); ++k) {
-      int cta = int(k % size_t(grid));
-      per_cta[cta].push_back(order[k]);
-      load[cta] += drafts[order[k]].w.n_steps + kItemOverheadSteps;
-    }
-  }
-
-  size_t n_steps = 0;
-  for (const Draft &d : drafts) n_steps += d.list.size();
-  plan->steps.reserve(n_steps);
-  plan->items.reserve(drafts.size());
-  plan->grid = grid;
-  plan->cta_begin.push_back(0);
-  for (int cta = 0; cta < grid; ++cta) {
-    for (int id : per_cta[cta]) {
-      Draft &d = drafts[id];
-      if (d.w.kind == 1) {
-        d.w.j0[0] = int32_t(plan->steps.size());
-        plan->steps.insert(plan->steps.end(), d.list.begin(), d.list.end());
-      }
-      plan->items.push_back(d.w);
-    }
-    plan->cta_begin.push_back(int32_t(plan->items.size()));
-  }
-  if (plan->steps.size() >= (size_t(1) << 31)) return STEEL_ERR_UNSUPPORTED;
-
-  // ---- statistics of the executed plan
-  s.work_items = int64_t(plan->items.size());
-  s.grid = grid;
-  s.list_entries = int64_t(plan->steps.size());
-  s.max_cta_steps = 0;
-  for (int cta = 0; cta < grid; ++cta) {
-    int64_t st_sum = 0;
-    for (int id : per_cta[cta]) st_sum += drafts[id].w.n_steps;
-    s.max_cta_steps = std::max(s.max_cta_steps, st_sum);
-  }
+  if (st != STEEL_OK) return st;
   // the walk visits every executed tile (millions on long sequences): only for callers that read these
   if (stats) walk_plan(*plan, [&](int, const WorkItem &, int, int, uint32_t entry, bool shared) {
     ++s.exec_tiles;
     s.exec_partial += (entry & kEntryPartial) != 0;
     s.kv_tile_loads += shared ? 0 : 1;
   }, p);
-  for (const WorkItem &w : plan->items) s.steps += w.n_steps;
   return STEEL_OK;
 }
 

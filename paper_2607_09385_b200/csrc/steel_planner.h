@@ -57,9 +57,10 @@ enum class Spread {
   kCut,    // also key ranges cut over CTAs, which needs part buffers
 };
 // Scheduling policy and the other options come from `p`.  Without `stats` the plan's statistics stay 0 (they
-// take a walk over every block and every executed tile).
+// take a walk over every block and every executed tile).  Where `plan` cuts key ranges, `whole` (if not null)
+// becomes the plan that would be taken without cuts: items, steps and the statistics of its items.
 steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan, bool stats = true,
-                          Spread spread = Spread::kNone);
+                          Spread spread = Spread::kNone, Plan *whole = nullptr);
 
 // steel_attn_create with a limit on what the plan may do (implemented in steel_attn.cu).
 steel_status_t create_attention(const steel_attn_params_t *params, Spread most, steel_attn_t **out);

@@ -126,3 +126,102 @@ def test_calls_after_an_interrupted_one_need_no_repair(case):
             for o2, lse2 in later:
                 assert torch.equal(o2, o) and torch.equal(lse2, lse)
     attn.close()
+
+
+def several_inputs(case, n):
+    """A handle, n sets of operands on the GPU, and each one's results from runs that nothing overlaps."""
+    attn, _, q, k, v = make(case)
+    sets = [[x.roll(m, -2).contiguous().cuda() for x in (q, k, v)] for m in range(n)]
+    ref = []
+    for dev in sets:
+        ref.append(attn.run(*dev))
+        torch.cuda.synchronize()
+    assert attn.last_status() == B.STEEL_OK
+    return attn, sets, ref
+
+
+def outputs_like(ref, n):
+    return [tuple(torch.full_like(x, float("nan")) for x in ref[m % len(ref)]) for m in range(n)]
+
+
+@pytest.mark.parametrize("case", [CASES[0], CASES[6]])
+def test_one_handle_on_several_streams(case):
+    """Runs of a cut plan queued on four streams at once, beside work that holds part of the GPU."""
+    attn, sets, ref = several_inputs(case, 5)
+    streams = [torch.cuda.current_stream()] + [torch.cuda.Stream() for _ in range(3)]
+    out = outputs_like(ref, 120)
+    other = torch.randn((4096, 4096), device="cuda", dtype=torch.bfloat16)
+    torch.cuda.synchronize()
+    busy = torch.cuda.Stream()
+    with torch.cuda.stream(busy):
+        for _ in range(60):
+            other @ other
+    for n, (o, lse) in enumerate(out):
+        with torch.cuda.stream(streams[n * 7 % 4]):
+            if n < 4:
+                torch.cuda._sleep(1_000_000)
+            attn.run(*sets[n % 5], o, lse)
+    torch.cuda.synchronize()
+    assert attn.last_status() == B.STEEL_OK
+    for n, (o, lse) in enumerate(out):
+        assert torch.equal(o, ref[n % 5][0]) and torch.equal(lse, ref[n % 5][1]), n
+    attn.close()
+
+
+def test_cut_plan_in_graphs_that_overlap():
+    """Two captured graphs, the first with two branches and a join, replayed beside each other and eager runs."""
+    attn, sets, ref = several_inputs(CASES[0], 5)
+    out = outputs_like(ref, 5)
+    side, graphs = torch.cuda.Stream(), [torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()]
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graphs[0]):
+        here = torch.cuda.current_stream()
+        side.wait_stream(here)
+        with torch.cuda.stream(side):
+            attn.run(*sets[0], *out[0])
+        attn.run(*sets[1], *out[1])
+        here.wait_stream(side)
+        attn.run(*sets[2], *out[2])
+    with torch.cuda.graph(graphs[1]):
+        attn.run(*sets[3], *out[3])
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for _ in range(20):
+        for o, lse in out:
+            o.fill_(float("nan"))
+            lse.fill_(float("nan"))
+        for g, stream in zip(graphs, streams):
+            stream.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.stream(stream):
+                g.replay()
+                g.replay()
+        for _ in range(4):
+            attn.run(*sets[4], *out[4])
+        torch.cuda.synchronize()
+        for (o, lse), (o_ref, lse_ref) in zip(out, ref):
+            assert torch.equal(o, o_ref) and torch.equal(lse, lse_ref)
+    assert attn.last_status() == B.STEEL_OK
+    del graphs
+    attn.close()
+
+
+def test_more_captures_than_part_buffers():
+    """Captures beyond the handle's bound run the plan without cuts: the same result within rounding."""
+    attn, sets, ref = several_inputs(CASES[0], 3)
+    out, graphs = outputs_like(ref, 36), []
+    torch.cuda.synchronize()
+    for n in range(36):
+        graphs.append(torch.cuda.CUDAGraph())
+        with torch.cuda.graph(graphs[-1]):
+            attn.run(*sets[n % 3], *out[n])
+    for g in graphs:
+        g.replay()
+    torch.cuda.synchronize()
+    assert attn.last_status() == B.STEEL_OK
+    exact = [torch.equal(o, ref[n % 3][0]) for n, (o, _) in enumerate(out)]
+    assert all(exact[:30])
+    for n, (o, lse) in enumerate(out):
+        err = (o.float() - ref[n % 3][0].float()).abs()
+        assert float(err.max()) <= H.TOL_O_MAX and float(err.mean()) <= H.TOL_O_MEAN
+        assert float((lse - ref[n % 3][1]).abs().max()) <= H.TOL_LSE
+    del graphs
+    attn.close()
