@@ -239,13 +239,15 @@ steel_status_t create_attention(const steel_attn_params_t *params, Spread most, 
   steel_status_t st = validate_params(params);
   if (st != STEEL_OK) return st;
 
-  int device = 0;
-  cudaDeviceProp prop;
-  if (cudaGetDevice(&device) != cudaSuccess || cudaGetDeviceProperties(&prop, device) != cudaSuccess) {
+  // two attributes: all properties take 2.5 ms, most of what creating a handle took
+  int device = 0, major = 0, num_sms = 0;
+  if (cudaGetDevice(&device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
     cudaGetLastError();
     return STEEL_ERR_CUDA;
   }
-  if (prop.major != 10) return STEEL_ERR_CUDA;  // the kernel is built for sm_100a only
+  if (major != 10) return STEEL_ERR_CUDA;  // the kernel is built for sm_100a only
 
   steel_attn *h = new (std::nothrow) steel_attn();
   if (!h) return STEEL_ERR_ALLOC;
@@ -254,7 +256,7 @@ steel_status_t create_attention(const steel_attn_params_t *params, Spread most, 
   try {
     for (Spread spread : {most, Spread::kTiles}) {  // the second only without memory for the first's part buffers
       whole = Plan();
-      st = build_plan(params, prop.multiProcessorCount, &plan, /*stats=*/true, spread, &whole);
+      st = build_plan(params, num_sms, &plan, /*stats=*/true, spread, &whole);
       if (st != STEEL_OK) {
         delete h;
         return st;
@@ -302,7 +304,8 @@ steel_status_t create_attention(const steel_attn_params_t *params, Spread most, 
   place_lists(&h->plan, h->d_lists);
   place_lists(&h->whole, h->d_lists);
   if (cudaMemcpy(h->d_lists, image.data(), image.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-      configure_kernels() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess || !encode_fn()) {
+      configure_kernels(params->head_dim, params->exp_emulation) != cudaSuccess ||
+      cudaDeviceSynchronize() != cudaSuccess || !encode_fn()) {
     cudaGetLastError();
     free_device(h);
     delete h;

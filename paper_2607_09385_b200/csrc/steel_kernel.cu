@@ -1013,16 +1013,21 @@ void launch_dim(int exp_emulation, const CUtensorMap &map_q, const CUtensorMap &
 
 }  // namespace
 
+cudaError_t configure_kernels(int head_dim, int exp_emulation) {
+  const bool wide = head_dim == 128;
+  switch (exp_emulation) {
+    case 1: return wide ? configure_one<128, 1>() : configure_one<64, 1>();
+    case 2: return wide ? configure_one<128, 2>() : configure_one<64, 2>();
+    case 3: return wide ? configure_one<128, 3>() : configure_one<64, 3>();
+    default: return wide ? configure_one<128, 0>() : configure_one<64, 0>();
+  }
+}
+
 cudaError_t configure_kernels() {
   cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess) e = configure_one<128, 0>();
-  if (e == cudaSuccess) e = configure_one<128, 1>();
-  if (e == cudaSuccess) e = configure_one<128, 2>();
-  if (e == cudaSuccess) e = configure_one<128, 3>();
-  if (e == cudaSuccess) e = configure_one<64, 0>();
-  if (e == cudaSuccess) e = configure_one<64, 1>();
-  if (e == cudaSuccess) e = configure_one<64, 2>();
-  if (e == cudaSuccess) e = configure_one<64, 3>();
+  for (int emulation = 0; emulation <= 3; ++emulation)
+    for (int head_dim : {64, 128})
+      if (e == cudaSuccess) e = configure_kernels(head_dim, emulation);
   return e;
 }
 

@@ -8,8 +8,10 @@
 
 namespace steel {
 
-// Opt the kernels in to their dynamic shared-memory size on the current device.
+// Opt kernels in to their dynamic shared-memory size on the current device, which loads them: all builds, or those of
+// one kind of problem.
 cudaError_t configure_kernels();
+cudaError_t configure_kernels(int head_dim, int exp_emulation);
 
 // Enqueue the persistent kernel: `grid` CTAs of 384 threads, one per SM.  `exp_emulation` selects the
 // build with 0, 12.5, 25 or 50 % of the exponentials on the FMA pipe (values 0..3).

@@ -244,10 +244,16 @@ Draft cut_piece(const Draft &d, int t0, int t1) {
   return r;
 }
 
-// Cut the drafts' steps, in order, into one share of at most `quota` per CTA (a piece of a draft at either
-// end of a share) and number the parts of the query tiles that were cut.  False if the shares do not suffice.
-bool cut_into_shares(const std::vector<Draft> &drafts, int num_ctas, double quota, double fill,
-                     std::vector<Draft> *pieces, Plan *plan) {
+// Steps [t0, t1) of a draft, or all of it as it is, for one CTA.
+struct Share {
+  int32_t draft, t0, t1, cta;
+  bool whole;
+};
+
+// Deal the drafts' steps, in order, into one share of at most `quota` per CTA (a piece of a draft at either end
+// of a share).  False if the shares do not suffice.  Only the numbers: the pieces are made once the quota is found
+// (made at every step of the search they took most of the planning: bitmap, 4 heads x 8192, 791 us in all, now 277).
+bool deal_shares(const std::vector<Draft> &drafts, int num_ctas, double quota, double fill, std::vector<Share> *shares) {
   const double overhead = kPieceOverheadSteps + part_write_steps(fill);
   int cta = 0;
   double left = quota;
@@ -255,13 +261,13 @@ bool cut_into_shares(const std::vector<Draft> &drafts, int num_ctas, double quot
     ++cta;
     left = quota;
   };
-  for (const Draft &d : drafts) {
+  for (size_t id = 0; id < drafts.size(); ++id) {
+    const Draft &d = drafts[id];
     const bool one = !slot_used(d.w, 1);
     const double w = one ? 0.5 : 1.0;
     const int n = d.w.n_steps, per_step = one ? 1 : 2;
     // at most kMaxParts parts of one query tile (two per piece)
     const int least = std::max<int>(min_piece_tiles(fill) / per_step, (n + kMaxParts / 2 - 1) / (kMaxParts / 2));
-    const size_t first = pieces->size();
     int t = 0;
     do {
       int take = std::max(0, int((left - overhead) / w));
@@ -274,21 +280,36 @@ bool cut_into_shares(const std::vector<Draft> &drafts, int num_ctas, double quot
       if (cta >= num_ctas) return false;
       // a tile with few rows in use is worth two parts even within one CTA
       const bool whole = take == n && !(one && fill <= 0.25 && n >= 2 * least);
-      pieces->push_back(whole ? d : cut_piece(d, t, t + take));
-      pieces->back().cta = cta;
+      shares->push_back(Share{int32_t(id), t, t + take, cta, whole});
       left -= (whole && one ? kSingleStep : w) * take + (whole ? kPieceOverheadSteps : overhead);
       if (left <= overhead) next_share();
       t += take;
     } while (t < n);
+  }
+  return true;
+}
+
+// The pieces of dealt drafts, and the numbers of the parts of the query tiles that were cut.
+void make_pieces(const std::vector<Draft> &drafts, const std::vector<Share> &shares, std::vector<Draft> *pieces,
+                 Plan *plan) {
+  pieces->reserve(shares.size());
+  for (size_t k = 0; k < shares.size();) {
+    const size_t first = pieces->size();
+    const Draft &d = drafts[shares[k].draft];
+    const bool one = !slot_used(d.w, 1);
+    for (const int32_t id = shares[k].draft; k < shares.size() && shares[k].draft == id; ++k) {
+      pieces->push_back(shares[k].whole ? d : cut_piece(d, shares[k].t0, shares[k].t1));
+      pieces->back().cta = shares[k].cta;
+    }
     if (pieces->size() == first + 1 && !(one && slot_used(pieces->back().w, 1))) continue;
     // the parts of each query tile are all slots of its pieces that hold it
     for (int s = 0; s < (one ? 1 : 2); ++s) {
       SplitTile tile{plan->n_parts, 0};
       const int32_t id = int32_t(plan->split_tiles.size());
       int32_t *only = nullptr;
-      for (size_t k = first; k < pieces->size(); ++k)
+      for (size_t n = first; n < pieces->size(); ++n)
         for (int u = 0; u < 2; ++u) {
-          WorkItem &x = (*pieces)[k].w;
+          WorkItem &x = (*pieces)[n].w;
           if (slot_used(x, u) && x.head[u] == d.w.head[s] && x.qtile[u] == d.w.qtile[s]) {
             only = &x.split[u];
             *only = split_code(id, tile.n_parts++);
@@ -302,11 +323,10 @@ bool cut_into_shares(const std::vector<Draft> &drafts, int num_ctas, double quot
       }
     }
   }
-  return true;
 }
 
-// The same with the smallest share that works, to 3 %.  Returns the load of the busiest CTA, or infinity where
-// nothing was cut.
+// Cut the drafts over the CTAs with the smallest share that works, to 3 %.  Returns the load of the busiest CTA, or
+// infinity where nothing was cut.
 double cut_over_ctas(const std::vector<Draft> &drafts, int num_ctas, double fill, std::vector<Draft> *pieces,
                      Plan *plan) {
   double work = 0.0;
@@ -316,12 +336,12 @@ double cut_over_ctas(const std::vector<Draft> &drafts, int num_ctas, double fill
     live += d.w.n_steps > 0;
   }
   double quota = (work + kPieceOverheadSteps * double(std::max<size_t>(live, num_ctas))) / num_ctas;
-  while (!cut_into_shares(drafts, num_ctas, quota, fill, pieces, plan)) {
+  std::vector<Share> shares;
+  while (!deal_shares(drafts, num_ctas, quota, fill, &shares)) {
     quota *= 1.03;
-    pieces->clear();
-    plan->split_tiles.clear();
-    plan->n_parts = 0;
+    shares.clear();
   }
+  make_pieces(drafts, shares, pieces, plan);
   if (plan->split_tiles.empty()) return std::numeric_limits<double>::infinity();
   std::vector<double> load(num_ctas, 0.0);
   int most_parts = 0;
@@ -330,6 +350,41 @@ double cut_over_ctas(const std::vector<Draft> &drafts, int num_ctas, double fill
                    (d.w.split[0] >= 0 || d.w.split[1] >= 0 ? part_write_steps(fill) : 0.0);
   for (const SplitTile &t : plan->split_tiles) most_parts = std::max(most_parts, t.n_parts);
   return *std::max_element(load.begin(), load.end()) + combine_steps(fill, most_parts);
+}
+
+// Statistics of the executed tiles.  Ranges are counted as such: visiting every tile of them took most of the
+// planning of long sequences (32/8 heads x 131072: 154 ms in all, now 6).
+void count_tiles(const Ctx &c, const Plan &plan, int64_t rows, steel_attn_stats_t *s) {
+  for (const WorkItem &w : plan.items) {
+    if (w.kind == 1) {
+      for (int t = 0; t < w.n_steps; ++t) {
+        const StepPair &pair = plan.steps[size_t(w.j0[0]) + size_t(t)];
+        const bool in0 = pair.e[0] != 0, in1 = pair.e[1] != 0;
+        const bool shared = in0 && in1 && (pair.e[0] & kEntryTileMask) == (pair.e[1] & kEntryTileMask);
+        s->exec_tiles += in0 + in1;
+        s->exec_partial += ((pair.e[0] & kEntryPartial) != 0) + ((pair.e[1] & kEntryPartial) != 0);
+        s->kv_tile_loads += in0 + in1 - shared;
+      }
+      continue;
+    }
+    int64_t tiles = 0, shared = 0;
+    for (int u = 0; u < 2; ++u) {
+      if (!slot_used(w, u)) continue;
+      tiles += w.hi[u] - w.lo[u] + 1;
+      // those seen whole, and not ragged
+      int64_t i0, i1, first, last;
+      tile_positions(c.p->seq_q, rows, w.qtile[u], &i0, &i1);
+      c.whole_range(i0, i1, kTile, &first, &last);
+      if (c.p->seq_kv % kTile) last = std::min(last, c.tkv128 - 2);
+      first = std::max<int64_t>(first, int64_t(w.j0[u]) + w.lo[u]);
+      last = std::min<int64_t>(last, int64_t(w.j0[u]) + w.hi[u]);
+      s->exec_partial += w.hi[u] - w.lo[u] + 1 - std::max<int64_t>(0, last - first + 1);
+    }
+    if (slot_used(w, 0) && slot_used(w, 1) && w.j0[0] == w.j0[1])
+      shared = std::max(0, std::min(w.hi[0], w.hi[1]) - std::max(w.lo[0], w.lo[1]) + 1);
+    s->exec_tiles += tiles;
+    s->kv_tile_loads += tiles - shared;
+  }
 }
 
 // Order the drafts, assign them to CTAs and write the plan's lists and the statistics of its items.
@@ -821,12 +876,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
     st = place_items(*p, num_ctas, uncut, whole);
   }
   if (st != STEEL_OK) return st;
-  // the walk visits every executed tile (millions on long sequences): only for callers that read these
-  if (stats) walk_plan(*plan, [&](int, const WorkItem &, int, int, uint32_t entry, bool shared) {
-    ++s.exec_tiles;
-    s.exec_partial += (entry & kEntryPartial) != 0;
-    s.kv_tile_loads += shared ? 0 : 1;
-  }, p);
+  if (stats) count_tiles(c, *plan, rows_q, &s);
   return STEEL_OK;
 }
 

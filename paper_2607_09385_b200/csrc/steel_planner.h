@@ -35,7 +35,7 @@ struct Draft {  // a work item before it is placed
   WorkItem w;
   std::vector<StepPair> list;
   int group;
-  int cta = -1;  // placed already (cut_over_ctas)
+  int cta = -1;  // placed already (make_pieces)
 };
 
 struct Plan {
@@ -57,7 +57,7 @@ enum class Spread {
   kCut,    // also key ranges cut over CTAs, which needs part buffers
 };
 // Scheduling policy and the other options come from `p`.  Without `stats` the plan's statistics stay 0 (they
-// take a walk over every block and every executed tile).  Where `plan` cuts key ranges, `whole` (if not null)
+// take a walk over every block).  Where `plan` cuts key ranges, `whole` (if not null)
 // becomes the plan that would be taken without cuts: items, steps and the statistics of its items.
 steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan, bool stats = true,
                           Spread spread = Spread::kNone, Plan *whole = nullptr);
