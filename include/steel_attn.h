@@ -209,7 +209,7 @@ steel_status_t steel_attn_run_noalloc(const steel_attn_params_t *params, const v
 /*
  * The same operation for tensors in HOST memory (the end-to-end path of Eq. 1 / Algorithm 1:
  * operands start and results end on the host).  A host-side object owns device staging buffers for
- * Q, K, V, O and LSE, internal streams and one plan per chunk.  The problem is cut into at
+ * Q, K, V, O and LSE, three internal streams and one plan per chunk.  The problem is cut into at
  * most `max_chunks` chunks that are independent attention problems with contiguous tensors: groups
  * of batch elements when batch > 1, groups of KV heads (with their query heads and their slice of
  * the bitmap) when batch == 1; the number used is the largest divisor of batch (of heads_kv) not

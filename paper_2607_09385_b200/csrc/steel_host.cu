@@ -2,11 +2,17 @@
 //
 // The problem is cut into chunks that are independent attention problems with contiguous tensors
 // (groups of batch elements when batch > 1, groups of KV heads with their query heads when
-// batch == 1).  Each chunk goes host -> device on a group of streams, through the attention
-// kernel on another and device -> host on a third, so that the copies of one chunk overlap the kernel of
+// batch == 1).  Each chunk goes host -> device on one stream, through the attention kernel on a
+// second and device -> host on a third, so that the copies of one chunk overlap the kernel of
 // another and both directions of the host link are busy at once.  Every step of the computation
 // runs in the same kernel as steel_attn_run: this file only plans chunks, owns the staging buffers
 // and orders copies and launches with events.
+//
+// One stream brings the operands.  Three in turn, so that a copy's start-up hides behind the one before it, also let
+// a later chunk's copies share the link with an earlier chunk's, which then ends later: us, one stream -> three,
+// head_dim 128, causal, 8 chunks: 32/8 heads x 4096 1 548 -> 1 410, 20/5 heads x 4096 (5 chunks) 1 005 -> 868, but
+// batch 8, 32/8 heads x 2048 4 674 -> 5 036, batch 16, 32/8 x 1024 4 581 -> 4 956, batch 4, 24/8 x 1777 1 841 -> 1 994,
+// batch 2, 32/8 x 4096 2 807 -> 3 129.  The sign follows neither sizes nor the number of chunks, so: one.
 #include <cuda_runtime.h>
 
 #include <new>
@@ -14,14 +20,6 @@
 
 #include "../../include/steel_attn.h"
 #include "steel_planner.h"
-
-// Host -> device copies of large chunks go to kInStreams streams in turn, so that a copy's start-up (about 5 us)
-// overlaps the one before it; a chunk's copies wait for those of kInLag chunks earlier, so that the chunks still
-// arrive in order.  One stream -> three: 32 heads x 4096 2.28 -> 2.24 ms, 32/8 heads x 4096 1.55 -> 1.40 ms; but
-// 32/4 heads x 8192 1.28 -> 1.42 ms (with a Q so much larger than K and V the streams drift apart), and below
-// kInBytes per chunk the extra events cost more than the overlap saves (0.36 -> 0.38 ms): one stream there.
-constexpr int kInStreams = 3, kInLag = 2;
-constexpr size_t kInBytes = size_t(4) << 20, kInMostQ = 4;  // Q of at most kInMostQ times K
 
 struct steel_attn_host {
   steel_attn_params_t params{};
@@ -31,7 +29,7 @@ struct steel_attn_host {
   std::vector<steel_attn_t *> child;  // one per chunk (bitmap masks) or a single shared one
   unsigned char *dq = nullptr, *dk = nullptr, *dv = nullptr, *dout = nullptr;
   float *dlse = nullptr;
-  cudaStream_t s_in[kInStreams] = {}, s_run = nullptr, s_out = nullptr;
+  cudaStream_t s_in = nullptr, s_run = nullptr, s_out = nullptr;
   cudaEvent_t ev_begin = nullptr, ev_end = nullptr;
   std::vector<cudaEvent_t> ev_in, ev_run;
 };
@@ -55,8 +53,7 @@ void release(steel_attn_host *h) {
   for (cudaEvent_t e : h->ev_run) cudaEventDestroy(e);
   if (h->ev_begin) cudaEventDestroy(h->ev_begin);
   if (h->ev_end) cudaEventDestroy(h->ev_end);
-  for (cudaStream_t s : h->s_in)
-    if (s) cudaStreamDestroy(s);
+  if (h->s_in) cudaStreamDestroy(h->s_in);
   if (h->s_run) cudaStreamDestroy(h->s_run);
   if (h->s_out) cudaStreamDestroy(h->s_out);
   cudaFree(h->dq);
@@ -122,8 +119,10 @@ extern "C" steel_status_t steel_attn_host_create(const steel_attn_params_t *para
       p.mask.bitmap = params->mask.bitmap + static_cast<int64_t>(c) * cp.heads_q * words_per_head;
     }
     steel_attn_t *child = nullptr;
-    // A chunk's kernel hides behind the copies, which it slows while it runs: over all SMs the call takes
-    // longer, not shorter (32 heads x 4096, 8 chunks: 2.24 ms with paired query tiles, 2.41 ms spread).
+    // A chunk's kernel hides behind the copies, so what spreading it over all SMs changes is only when the copy back
+    // starts, and the call gets slower or faster with that (8 chunks, head_dim 128, paired query tiles / spread:
+    // 32 heads x 4096 2.29 / 2.42 ms, 12 heads x 6000 dense 1.43 / 1.30 ms, most others within 2 %): paired, and
+    // chunks stay without part buffers.
     st = steel::create_attention(&p, h->n_chunks > 1 ? steel::Spread::kNone : steel::Spread::kCut, &child);
     if (st == STEEL_OK) h->child.push_back(child);
   }
@@ -143,19 +142,15 @@ extern "C" steel_status_t steel_attn_host_create(const steel_attn_params_t *para
     release(h);
     return STEEL_ERR_ALLOC;
   }
-  ok = true;
-  for (cudaStream_t &s : h->s_in) ok = ok && cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess;
-  ok = ok && cudaStreamCreateWithFlags(&h->s_run, cudaStreamNonBlocking) == cudaSuccess &&
+  ok = cudaStreamCreateWithFlags(&h->s_in, cudaStreamNonBlocking) == cudaSuccess &&
+       cudaStreamCreateWithFlags(&h->s_run, cudaStreamNonBlocking) == cudaSuccess &&
        cudaStreamCreateWithFlags(&h->s_out, cudaStreamNonBlocking) == cudaSuccess &&
        cudaEventCreateWithFlags(&h->ev_begin, cudaEventDisableTiming) == cudaSuccess &&
        cudaEventCreateWithFlags(&h->ev_end, cudaEventDisableTiming) == cudaSuccess;
   for (int c = 0; c < h->n_chunks && ok; ++c) {
-    for (int n = 0; n < kInStreams && ok; ++n) {
-      cudaEvent_t a = nullptr;
-      ok = cudaEventCreateWithFlags(&a, cudaEventDisableTiming) == cudaSuccess;
-      if (ok) h->ev_in.push_back(a);
-    }
-    cudaEvent_t b = nullptr;
+    cudaEvent_t a = nullptr, b = nullptr;
+    ok = cudaEventCreateWithFlags(&a, cudaEventDisableTiming) == cudaSuccess;
+    if (ok) h->ev_in.push_back(a);
     ok = ok && cudaEventCreateWithFlags(&b, cudaEventDisableTiming) == cudaSuccess;
     if (ok) h->ev_run.push_back(b);
   }
@@ -187,23 +182,15 @@ extern "C" steel_status_t steel_attn_host_run(steel_attn_host_t *h, const void *
   }
   // everything below starts after the work already queued on the caller's stream
   STEEL_HOST_CHECK(cudaEventRecord(h->ev_begin, user));
-  const bool many = h->q_chunk_bytes + 2 * h->kv_chunk_bytes >= kInBytes && h->q_chunk_bytes <= kInMostQ * h->kv_chunk_bytes;
-  const int n_in = many ? kInStreams : 1;
-  int copies = 0;
-  for (int n = 0; n < n_in; ++n) STEEL_HOST_CHECK(cudaStreamWaitEvent(h->s_in[n], h->ev_begin, 0));
-  auto next_in = [&] { return h->s_in[copies++ % n_in]; };
+  STEEL_HOST_CHECK(cudaStreamWaitEvent(h->s_in, h->ev_begin, 0));
   for (int c = 0; c < h->n_chunks; ++c) {
     const size_t qo = c * h->q_chunk_bytes, ko = c * h->kv_chunk_bytes, lo = c * h->lse_chunk_bytes;
-    for (int n = 0; n_in > 1 && c >= kInLag && n < n_in; ++n)
-      for (int k = 0; k < n_in; ++k)
-        STEEL_HOST_CHECK(cudaStreamWaitEvent(h->s_in[n], h->ev_in[(c - kInLag) * kInStreams + k], 0));
-    STEEL_HOST_CHECK(cudaMemcpyAsync(h->dq + qo, hq + qo, h->q_chunk_bytes, cudaMemcpyHostToDevice, next_in()));
-    STEEL_HOST_CHECK(cudaMemcpyAsync(h->dk + ko, hk + ko, h->kv_chunk_bytes, cudaMemcpyHostToDevice, next_in()));
-    STEEL_HOST_CHECK(cudaMemcpyAsync(h->dv + ko, hv + ko, h->kv_chunk_bytes, cudaMemcpyHostToDevice, next_in()));
-    for (int n = 0; n < n_in; ++n) {
-      STEEL_HOST_CHECK(cudaEventRecord(h->ev_in[c * kInStreams + n], h->s_in[n]));
-      STEEL_HOST_CHECK(cudaStreamWaitEvent(h->s_run, h->ev_in[c * kInStreams + n], 0));
-    }
+    STEEL_HOST_CHECK(cudaMemcpyAsync(h->dq + qo, hq + qo, h->q_chunk_bytes, cudaMemcpyHostToDevice, h->s_in));
+    STEEL_HOST_CHECK(cudaMemcpyAsync(h->dk + ko, hk + ko, h->kv_chunk_bytes, cudaMemcpyHostToDevice, h->s_in));
+    STEEL_HOST_CHECK(cudaMemcpyAsync(h->dv + ko, hv + ko, h->kv_chunk_bytes, cudaMemcpyHostToDevice, h->s_in));
+    STEEL_HOST_CHECK(cudaEventRecord(h->ev_in[c], h->s_in));
+
+    STEEL_HOST_CHECK(cudaStreamWaitEvent(h->s_run, h->ev_in[c], 0));
     steel_attn_t *child = h->child[h->child.size() == 1 ? 0 : c];
     const steel_status_t st =
         steel_attn_run(child, h->dq + qo, h->dk + ko, h->dv + ko, h->dout + qo,
@@ -242,7 +229,7 @@ extern "C" steel_status_t steel_attn_host_destroy(steel_attn_host_t *h) {
   if (!h) return STEEL_OK;
   int prev = 0;
   if (cudaGetDevice(&prev) == cudaSuccess && prev == h->device) {
-    for (cudaStream_t s : h->s_in) cudaStreamSynchronize(s);
+    cudaStreamSynchronize(h->s_in);
     cudaStreamSynchronize(h->s_run);
     cudaStreamSynchronize(h->s_out);
   }
