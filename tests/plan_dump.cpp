@@ -1,14 +1,14 @@
-// Prints the plan that steel_attn_create builds, for tests/test_plan_spread.py.  Host code only.
-// usage: plan_dump ctas batch heads_q heads_kv seq_q seq_kv flags window [bitmap words in hex ...]
+// Prints the plan that steel_attn_create builds, for tests/test_plan_spread.py and tests/test_gpu_spread.py.  Host code
+// only.  usage: plan_dump ctas batch heads_q heads_kv seq_q seq_kv flags window block [bitmap words in hex ...]
 #include <cstdio>
 #include <cstdlib>
 
 #include "../paper_2607_09385_b200/csrc/steel_planner.h"
 
 int main(int argc, char **argv) {
-  if (argc < 9) return 2;
+  if (argc < 10) return 2;
   std::vector<uint32_t> bitmap;
-  for (int n = 9; n < argc; ++n) bitmap.push_back(uint32_t(std::strtoul(argv[n], nullptr, 16)));
+  for (int n = 10; n < argc; ++n) bitmap.push_back(uint32_t(std::strtoul(argv[n], nullptr, 16)));
   steel_attn_params_t p{};
   p.batch = std::atoi(argv[2]);
   p.heads_q = std::atoi(argv[3]);
@@ -19,6 +19,7 @@ int main(int argc, char **argv) {
   p.scale = 1.0f;
   p.mask.flags = uint32_t(std::atoi(argv[7]));
   p.mask.window = std::atoi(argv[8]);
+  p.mask.block_q = p.mask.block_kv = std::atoi(argv[9]);
   p.mask.bitmap = bitmap.empty() ? nullptr : bitmap.data();
   steel::Plan plan;
   if (steel::build_plan(&p, std::atoi(argv[1]), &plan, true, steel::Spread::kCut) != STEEL_OK) return 3;

@@ -150,3 +150,26 @@ def test_host_argument_errors():
     assert lib.steel_attn_host_chunks(None) == 0
     B.steel_attn_host_destroy(h)
     B.steel_attn_host_destroy(None)
+
+
+def test_chunks_of_few_queries_and_many_keys():
+    # Chunks are planned without cut key ranges, the whole problem on the device with them (each chunk alone would be
+    # cut as well): keys are combined in another order, so the results agree within rounding.
+    b, hq, hkv, sq, skv, d = 1, 8, 4, 40, 5000, 128
+    rng = np.random.default_rng(57)
+    q, k, v = (torch.from_numpy(rng.standard_normal(s, np.float32)).to(torch.bfloat16).pin_memory()
+               for s in ((b, hq, sq, d), (b, hkv, skv, d), (b, hkv, skv, d)))
+    args = (b, hq, hkv, sq, skv, d, d ** -0.5, CAUSAL)
+    host, attn = B.SteelAttentionHost(*args, max_chunks=4), B.SteelAttention(*args)
+    assert host.chunks == 4 and attn.stats()["max_cta_steps"] < skv // 128  # cut
+    o, lse = torch.full_like(q, float("nan")).pin_memory(), torch.full((b, hq, sq), float("nan")).pin_memory()
+    for _ in range(2):
+        host.run(q, k, v, o, lse)
+    assert host.last_status() == B.STEEL_OK
+    o_dev, lse_dev = attn.run(q.cuda(), k.cuda(), v.cuda())
+    assert attn.last_status() == B.STEEL_OK
+    err = (o.float() - o_dev.float().cpu()).abs()
+    assert float(err.max()) <= H.TOL_O_MAX and float(err.mean()) <= H.TOL_O_MEAN
+    assert float((lse - lse_dev.cpu()).abs().max()) <= H.TOL_LSE
+    host.close()
+    attn.close()

@@ -1,7 +1,8 @@
 """Calls whose plan packs the heads of a group into query tiles or cuts key ranges over CTAs, against the
 oracle: one row per matrix, row counts that are not a multiple of 4, rows of several heads in one tile, two to
-dozens of parts, rows without a visible key, software exponents.  Repeated calls are bit-identical (the parts
-are combined in a fixed order, whichever ends last), also after a call that was interrupted."""
+64 parts, windows and bitmaps of both block sizes cut into parts, rows without a visible key in a part or at all,
+software exponents.  Each case states what its plan shows.  Repeated calls are bit-identical (the parts are combined
+in a fixed order, whichever ends last), also after a call that was interrupted and beside other runs of the handle."""
 import math
 
 import numpy as np
@@ -24,25 +25,51 @@ CASES = [  # batch, heads_q, heads_kv, seq_q, seq_kv, head_dim, flags, window, e
     (1, 1, 1, 3000, 3000, 128, CAUSAL, 0, 0), (1, 3, 1, 129, 2500, 64, 0, 0, 1), (1, 4, 2, 60, 20, 128, CAUSAL, 0, 0),
     (1, 2, 1, 400, 4096, 64, BITMAP, 0, 0),
 ]
+# what the plan of each shows: packed heads, fewest and most parts of a cut query tile (0, 0: none is cut)
+SHOWN = [(1, 18, 18), (0, 6, 6), (0, 64, 64), (1, 0, 0), (1, 12, 12), (1, 0, 0), (0, 8, 8), (1, 0, 0), (0, 0, 0),
+         (1, 0, 0), (1, 0, 0), (0, 0, 0)]
+
+CUT = [  # the same with the block size of the mask, what its bitmap holds, and what the plan shows
+    (1, 32, 16, 700, 4000, 128, CAUSAL, 0, 0, 128, None, (1, 2, 2)),
+    (8, 16, 16, 1, 2000, 64, CAUSAL, 0, 0, 128, None, (0, 2, 2)),
+    (1, 4, 2, 300, 9000, 64, CAUSAL | WINDOW, 5000, 0, 128, None, (1, 6, 7)),
+    (1, 4, 4, 128, 9000, 128, WINDOW, 6000, 0, 128, None, (0, 8, 8)),
+    (1, 2, 2, 128, 8192, 128, BITMAP, 0, 0, 128, "random", (0, 4, 4)),
+    (1, 2, 2, 128, 8192, 128, BITMAP, 0, 0, 64, "ends", (0, 4, 8)),
+    (1, 2, 2, 128, 8192, 64, BITMAP, 0, 3, 64, "ends", (0, 4, 8)),
+    (1, 4, 2, 300, 6000, 64, BITMAP | CAUSAL, 0, 0, 64, "random", (0, 6, 7)),
+]
 
 
-def make(case, seed=5):
+def block_bitmap(case):
+    """"random": half of the blocks.  "ends", two rows of blocks: the first keeps only early keys, the second only late
+    ones, so that parts hold rows without a visible key; the last head keeps nothing in its second row."""
+    _, hq, _, sq, skv, _, _, _, _, block, kind, _ = case
+    tq, tkv = -(-sq // block), -(-skv // block)
+    bits = np.random.default_rng(2).random((hq, tq, -(-tkv // 32) * 32)) < 0.5
+    if kind == "ends":
+        bits[:] = False
+        bits[:, 0, :48] = True
+        bits[:, 1, tkv - 48:tkv] = True
+        bits[-1, 1] = False
+    weight = np.uint64(1) << np.arange(32, dtype=np.uint64)
+    return (bits.reshape(hq, tq, -1, 32).astype(np.uint64) * weight).sum(3).astype(np.uint32)
+
+
+def make(case, seed=5, block=128, bitmap=None):
     b, hq, hkv, sq, skv, d, flags, window, emu = case
     rng = np.random.default_rng(seed)
     q, k, v = (torch.from_numpy(rng.standard_normal(s, np.float32)).to(torch.bfloat16)
                for s in ((b, hq, sq, d), (b, hkv, skv, d), (b, hkv, skv, d)))
-    bitmap = None
-    if flags & BITMAP:
+    if flags & BITMAP and bitmap is None:
         bitmap = rng.integers(0, 1 << 32, (hq, -(-sq // 128), -(-skv // 4096)), dtype=np.uint32)
     args = (b, hq, hkv, sq, skv, d, 1.0 / math.sqrt(d), flags)
-    attn = B.SteelAttention(*args, window=window, bitmap=bitmap, exp_emulation=emu)
-    p = oracle.OracleProblem(*args, 128, 128, window, bitmap)
+    attn = B.SteelAttention(*args, block=block, window=window, bitmap=bitmap, exp_emulation=emu)
+    p = oracle.OracleProblem(*args, block, block, window, bitmap)
     return attn, p, q, k, v
 
 
-@pytest.mark.parametrize("case", CASES)
-def test_against_oracle(case):
-    attn, p, q, k, v = make(case)
+def compare_with_oracle(attn, p, q, k, v):
     dev = [x.cuda() for x in (q, k, v)]
     o = torch.full_like(dev[0], float("nan"))
     lse = torch.full(q.shape[:3], float("nan"), device="cuda")
@@ -63,6 +90,28 @@ def test_against_oracle(case):
         o2, lse2 = attn.run(*dev)
         assert torch.equal(o2, o) and torch.equal(lse2, lse)
     attn.close()
+
+
+def assert_shown(lines, shown):
+    counts = [int(x.split()[2]) for x in lines if x.startswith("split")] or [0]
+    assert (int(lines[0].split()[2]), min(counts), max(counts)) == shown
+
+
+@pytest.mark.parametrize("case,shown", list(zip(CASES, SHOWN)))
+def test_against_oracle(case, shown, plan_dump):
+    attn, p, q, k, v = make(case)
+    b, hq, hkv, sq, skv, _, flags, window, _ = case
+    words = p.bitmap.ravel() if flags & BITMAP else ()
+    assert_shown(plan_dump(148, b, hq, hkv, sq, skv, flags, window, 128, words), shown)
+    compare_with_oracle(attn, p, q, k, v)
+
+
+@pytest.mark.parametrize("case", CUT)
+def test_cut_masks_against_oracle(case, plan_dump):
+    b, hq, hkv, sq, skv, _, flags, window, _, block, kind, shown = case
+    bitmap = block_bitmap(case) if kind else None
+    assert_shown(plan_dump(148, b, hq, hkv, sq, skv, flags, window, block, bitmap.ravel() if kind else ()), shown)
+    compare_with_oracle(*make(case[:9], block=block, bitmap=bitmap))
 
 
 def test_interrupted_call_leaves_nothing_behind():

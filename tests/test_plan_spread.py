@@ -1,39 +1,33 @@
 """Plans that pack the heads of a group into query tiles and cut key ranges over CTAs: every key tile that a
 query tile sees is executed exactly once, with the right mask flag, and the parts of a cut tile are numbered
 completely.  The visible tiles come from the mask's definition, row by row.  CPU only."""
-import os
-import subprocess
-
 import numpy as np
 import pytest
 
-HERE = os.path.dirname(os.path.abspath(__file__))
 CAUSAL, WINDOW, BITMAP = 1, 2, 4
 
-CASES = [  # ctas, batch, heads_q, heads_kv, seq_q, seq_kv, flags, window, kept share of a bitmap's blocks
-    (148, 8, 32, 8, 1, 6001, CAUSAL, 0, 0), (148, 1, 8, 1, 3, 1000, CAUSAL, 0, 0), (148, 2, 12, 4, 8, 40, 0, 0, 0),
-    (148, 1, 32, 8, 500, 12500, CAUSAL, 0, 0), (148, 1, 3, 1, 129, 129, CAUSAL, 0, 0),
-    (148, 1, 6, 2, 200, 900, CAUSAL | WINDOW, 150, 0), (148, 1, 4, 1, 40, 5000, WINDOW, 600, 0),
-    (148, 1, 12, 12, 512, 512, 0, 0, 0), (148, 1, 1, 1, 256, 256, CAUSAL, 0, 0), (148, 1, 1, 1, 1, 32768, 0, 0, 0),
-    (148, 1, 2, 1, 300, 100, CAUSAL, 0, 0), (4, 1, 5, 5, 1000, 1000, CAUSAL, 0, 0), (3, 2, 4, 2, 700, 2000, CAUSAL, 0, 0),
-    (148, 1, 2, 1, 2048, 2048, CAUSAL | BITMAP, 0, 0.4), (148, 1, 2, 2, 128, 8192, BITMAP, 0, 0.6),
-    (148, 16, 128, 16, 8, 4096, CAUSAL, 0, 0), (7, 1, 7, 1, 130, 3000, 0, 0, 0), (148, 1, 1, 1, 16384, 16384, CAUSAL, 0, 0),
-    (148, 1, 16, 4, 2048, 2048, CAUSAL, 0, 0), (148, 16, 16, 16, 1, 3000, CAUSAL, 0, 0),
-    (148, 1, 2, 2, 8192, 8192, BITMAP | CAUSAL, 0, 0.3),
+# ctas, batch, heads_q, heads_kv, seq_q, seq_kv, flags, window, kept share of a bitmap's blocks, and what the plan is
+# to show: packed heads, fewest and most parts of a cut query tile (0, 0: none is cut)
+CASES = [
+    (148, 8, 32, 8, 1, 6001, CAUSAL, 0, 0, (1, 4, 4)), (148, 1, 8, 1, 3, 1000, CAUSAL, 0, 0, (1, 0, 0)),
+    (148, 2, 12, 4, 8, 40, 0, 0, 0, (1, 0, 0)), (148, 1, 32, 8, 500, 12500, CAUSAL, 0, 0, (0, 3, 3)),
+    (148, 1, 3, 1, 129, 129, CAUSAL, 0, 0, (1, 0, 0)), (148, 1, 6, 2, 200, 900, CAUSAL | WINDOW, 150, 0, (1, 0, 0)),
+    (148, 1, 4, 1, 40, 5000, WINDOW, 600, 0, (1, 0, 0)), (148, 1, 12, 12, 512, 512, 0, 0, 0, (0, 0, 0)),
+    (148, 1, 1, 1, 256, 256, CAUSAL, 0, 0, (0, 0, 0)), (148, 1, 1, 1, 1, 32768, 0, 0, 0, (0, 64, 64)),
+    (148, 1, 2, 1, 300, 100, CAUSAL, 0, 0, (0, 0, 0)), (4, 1, 5, 5, 1000, 1000, CAUSAL, 0, 0, (0, 0, 0)),
+    (3, 2, 4, 2, 700, 2000, CAUSAL, 0, 0, (1, 0, 0)), (148, 1, 2, 1, 2048, 2048, CAUSAL | BITMAP, 0, 0.4, (0, 0, 0)),
+    (148, 1, 2, 2, 128, 8192, BITMAP, 0, 0.6, (0, 6, 6)), (148, 16, 128, 16, 8, 4096, CAUSAL, 0, 0, (1, 0, 0)),
+    (7, 1, 7, 1, 130, 3000, 0, 0, 0, (1, 0, 0)), (148, 1, 1, 1, 16384, 16384, CAUSAL, 0, 0, (0, 2, 5)),
+    (148, 1, 16, 4, 2048, 2048, CAUSAL, 0, 0, (0, 0, 0)), (148, 16, 16, 16, 1, 3000, CAUSAL, 0, 0, (0, 2, 4)),
+    (148, 1, 2, 2, 8192, 8192, BITMAP | CAUSAL, 0, 0.3, (0, 0, 0)),
+    (148, 1, 4, 2, 300, 9000, CAUSAL | WINDOW, 5000, 0, (1, 6, 7)), (148, 1, 4, 4, 128, 9000, WINDOW, 6000, 0, (0, 8, 8)),
+    (148, 1, 32, 16, 700, 4000, CAUSAL, 0, 0, (1, 2, 2)),
 ]
-
-
-@pytest.fixture(scope="module")
-def plan_dump(tmp_path_factory):
-    exe = str(tmp_path_factory.mktemp("plan") / "plan_dump")
-    subprocess.check_call(["g++", "-std=c++17", "-O1", "-o", exe, os.path.join(HERE, "plan_dump.cpp"),
-                           os.path.join(HERE, "..", "paper_2607_09385_b200", "csrc", "steel_planner.cpp")])
-    return exe
 
 
 @pytest.mark.parametrize("case", CASES)
 def test_every_visible_key_tile_exactly_once(plan_dump, case):
-    ctas, batch, hq, hkv, sq, skv, flags, window, keep = case
+    ctas, batch, hq, hkv, sq, skv, flags, window, keep, shown = case
     tq, tkv = -(-sq // 128), -(-skv // 128)
     bits, words = np.ones((hq, tq, tkv), bool), []
     if flags & BITMAP:
@@ -41,14 +35,15 @@ def test_every_visible_key_tile_exactly_once(plan_dump, case):
         packed_bits = np.zeros((hq, tq, -(-tkv // 32)), np.uint32)
         for h, i, j in zip(*np.nonzero(bits)):
             packed_bits[h, i, j >> 5] |= np.uint32(1 << (j & 31))
-        words = ["%x" % x for x in packed_bits.ravel()]
-    out = subprocess.check_output([plan_dump] + [str(x) for x in (ctas, batch, hq, hkv, sq, skv, flags, window)] + words,
-                                  text=True).split("\n")
+        words = packed_bits.ravel()
+    out = plan_dump(ctas, batch, hq, hkv, sq, skv, flags, window, 128, words)
     grid, packed, n_parts, n_items = (int(x) for x in out[0].split()[1:])
     assert grid <= ctas and n_items == sum(l.startswith("item") for l in out)
     splits = [tuple(int(x) for x in l.split()[1:]) for l in out if l.startswith("split")]
     assert sum(n for _, n in splits) == n_parts and all(2 <= n <= 64 for _, n in splits)
     assert [f for f, _ in splits] == list(np.cumsum([0] + [n for _, n in splits])[:-1])
+    counts = [n for _, n in splits] or [0]
+    assert (packed, min(counts), max(counts)) == shown
     seen, parts, tiles = {}, {}, set()
     for l in out[1:]:
         if l.startswith("item"):
