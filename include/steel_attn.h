@@ -22,6 +22,8 @@
  *     BITMAP : bit (J & 31) of bitmap[(h * T_q + I) * ceil(T_kv / 32) + (J >> 5)] is set,
  *              I = i / block_q, J = j / block_kv, T_q = ceil(seq_q / block_q), T_kv likewise.
  * A query row with no visible key gets O = 0 and LSE = -inf.
+ * A masked key inside an executed 128 x 128 tile has weight 0 exactly; where its V is not finite, 0 times it is NaN
+ * and reaches the O of every row of that tile (a tile may hold rows of several heads of a group).
  *
  * Memory layout: Q and O are [batch, heads_q, seq_q, head_dim], K and V are
  * [batch, heads_kv, seq_kv, head_dim], all contiguous bfloat16; LSE is
@@ -215,7 +217,9 @@ steel_status_t steel_attn_run_noalloc(const steel_attn_params_t *params, const v
  * the bitmap) when batch == 1; the number used is the largest divisor of batch (of heads_kv) not
  * above max_chunks (values below 1 mean 1).  Chunk c is copied host -> device, run through the
  * kernel of steel_attn_run and copied device -> host on separate streams, so the copies of one
- * chunk overlap the kernel of another.  Results equal those of steel_attn_run on the same chunk.
+ * chunk overlap the kernel of another.  More than one chunk: the chunks are planned without cut key ranges and
+ * results agree with those of steel_attn_run within rounding (bit for bit where its plan visits a query's keys
+ * in the same order).  One chunk: the plan and the results of steel_attn_run.
  */
 typedef struct steel_attn_host steel_attn_host_t; /* opaque, owned by the library */
 

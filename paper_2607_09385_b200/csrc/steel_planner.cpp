@@ -88,7 +88,8 @@ struct Ctx {
   }
 
   // Bitmap masks: the entries of query tile I of head h, fully masked tiles (case i) left out.  Word by word:
-  // one tile at a time took most of the planning (8 heads x 4096 tokens, 64-token blocks: 528 us in all, now 55).
+  // one tile at a time took most of the planning (8 heads x 4096 tokens, 64-token blocks, plan of the allocation-free
+  // call without statistics, on the host of a B200: 416 us in all, now 75).
   void entries(int h, int64_t I, std::vector<uint32_t> *out) const {
     int64_t i0, i1, whole_lo, whole_hi;
     rows(I, kTile, i0, i1);
@@ -252,7 +253,7 @@ struct Share {
 
 // Deal the drafts' steps, in order, into one share of at most `quota` per CTA (a piece of a draft at either end
 // of a share).  False if the shares do not suffice.  Only the numbers: the pieces are made once the quota is found
-// (made at every step of the search they took most of the planning: bitmap, 4 heads x 8192, 791 us in all, now 277).
+// (made at every step of the search they took half of the planning: bitmap, 4 heads x 8192, 749 us in all, now 392).
 bool deal_shares(const std::vector<Draft> &drafts, int num_ctas, double quota, double fill, std::vector<Share> *shares) {
   const double overhead = kPieceOverheadSteps + part_write_steps(fill);
   int cta = 0;
@@ -353,7 +354,7 @@ double cut_over_ctas(const std::vector<Draft> &drafts, int num_ctas, double fill
 }
 
 // Statistics of the executed tiles.  Ranges are counted as such: visiting every tile of them took most of the
-// planning of long sequences (32/8 heads x 131072: 154 ms in all, now 6).
+// planning of long sequences (32/8 heads x 131072: 143 ms in all, now 4).
 void count_tiles(const Ctx &c, const Plan &plan, int64_t rows, steel_attn_stats_t *s) {
   for (const WorkItem &w : plan.items) {
     if (w.kind == 1) {
