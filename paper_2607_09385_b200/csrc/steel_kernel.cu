@@ -80,7 +80,10 @@ struct Ctrl {
   long long timeout_cycles;
 };
 
-// Command word (producer -> MMA issuer): one product, S(s, t) or PV(s, t).
+// Command word (producer -> MMA issuer): one product, S(s, t) or PV(s, t).  In the queue its 16 bits stand beside
+// their complement: the issuing warp puts a word together from what each of its lanes has read (warp_uniform), and
+// nothing in the language makes the lanes read at the same moment.  A word that only some lanes have seen fails the
+// check and is read again.
 constexpr uint32_t kCmdValid = 1u << 0, kCmdSlot1 = 1u << 1,
                    kCmdFirst = 1u << 2, kCmdLast = 1u << 3,  // of the slot's steps in this item
                    kCmdRingShift = 4,  // 4 bits: ring slot of the K or V tile
@@ -89,7 +92,8 @@ constexpr uint32_t kCmdValid = 1u << 0, kCmdSlot1 = 1u << 1,
                    kCmdDepPhase = 1u << 10,   // S buffer free (S), P full (PV)
                    kCmdWaitSFree = 1u << 11,  // not the CTA's first S
                    kCmdFinal = 1u << 12,      // S: last reader of the K tile, release the ring slot
-                   kCmdExit = 1u << 31;
+                   kCmdExit = 1u << 13;
+__device__ __forceinline__ bool cmd_complete(uint32_t word) { return ((word ^ (word >> 16)) & 0xFFFFu) == 0xFFFFu; }
 
 __device__ __forceinline__ bool bounded_wait(uint64_t *bar, uint32_t parity, Ctrl &ctrl, int32_t *status) {
   if (mbar_test_wait(bar, parity)) return true;  // the common case: already complete, no suspension
@@ -250,7 +254,7 @@ __device__ __forceinline__ bool fifo_push(Ctrl &ctrl, int s, uint32_t &tail, uin
       }
     }
   }
-  *cell = word;
+  *cell = word | ~word << 16;
   tail = (tail + 1) & (kFifoDepth - 1);
   return true;
 }
@@ -376,13 +380,13 @@ __device__ __forceinline__ uint32_t fifo_pop_warp(Ctrl &ctrl, int s, uint32_t &h
   volatile uint32_t *cell = &ctrl.fifo[s][head];
   __syncwarp();
   uint32_t word = warp_uniform(*cell, lane);
-  if (word == 0) {
+  if (!cmd_complete(word)) {
     const long long start = clock64();
     uint32_t n = 0;
     while (true) {
       __syncwarp();
       word = warp_uniform(*cell, lane);
-      if (word != 0) break;
+      if (cmd_complete(word)) break;
       if ((++n & 63u) == 0) {
         const bool stop = *reinterpret_cast<volatile int *>(&ctrl.abort) != 0 || clock64() - start > ctrl.timeout_cycles;
         if (__any_sync(0xffffffffu, stop)) {
@@ -468,7 +472,7 @@ __device__ void mma_role(const KernelParams &p, Ctrl &ctrl, uint8_t *smem_q, uin
     }
     const uint32_t next = warp_uniform(next_raw, lane);
     if (__any_sync(0xffffffffu, !ok)) break;
-    if (next != 0) {
+    if (cmd_complete(next)) {
       if (lane == 0) *next_cell = 0;
       head = (head + 1) & (kFifoDepth - 1);
       cmd = next;
