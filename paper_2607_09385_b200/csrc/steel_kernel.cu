@@ -775,30 +775,11 @@ __device__ int softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, cons
       mx1 = fmax3(mx1, x[126], x[127]);
       const float ms = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3)) * scale_log2;
 
-      if (t == lo) {
-        m_ref = ms;
-      } else {
-        // the running maximum only has to bound the exponents: rescale O lazily
-        const bool need = ms > m_ref + kRescaleThreshold;
-        if (__any_sync(0xffffffffu, need)) {
-          // PV(s, t - 1) accumulates into O: it must have finished
-          if (!warp_wait(&ctrl.p_free[s], (n_sp - 1u) & 1u, ctrl, p.status, lane)) return k;
-          tc_fence_after();
-          const float v = need ? ex2_approx(m_ref - ms) : 1.0f;
-          l *= v;
-          // rare: kept short, so that the loop around it needs fewer instructions from the cache
-#pragma unroll 1
-          for (int c = 0; c < D / 32; ++c) {
-            uint32_t regs[32];
-            tmem_ld32(t_o + c * 32, regs);
-            tc_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 32; ++i) regs[i] = __float_as_uint(__uint_as_float(regs[i]) * v);
-            tmem_st32(t_o + c * 32, regs);
-          }
-          if (need) m_ref = ms;
-        }
-      }
+      // the running maximum only has to bound the exponents: O is rescaled lazily, once PV(s, t - 1) has finished
+      const float m_old = m_ref;
+      const bool grown = ms > m_ref + kRescaleThreshold;
+      if (grown) m_ref = ms;
+      const bool need = grown && t > lo;
       const float m_use = (m_ref == -CUDART_INF_F) ? 0.0f : m_ref;
       const float2 neg_m2 = make_float2(-m_use, -m_use);
 
@@ -807,13 +788,31 @@ __device__ int softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, cons
       for (int half = 0; half < 2; ++half) {
         uint32_t packed[32];
         exp_half<kEmu>(x, half * 64, scale2, neg_m2, acc_a, acc_b, packed);
-        if (half == 0 && (D == 64 || t > lo)) {
-          // PV(s, t - 1) reads the P columns: it must have finished before they are overwritten (by now it has
-          // had the whole first half of the exponentials to do so).  A slot's first step need not wait, and at
-          // head_dim 64 does all the same: its barrier is complete (or in its initial phase), and the loop is
-          // faster without the test (32 heads x 8192 362 -> 355 us; at head_dim 128, 32/8 heads x 16384, slower:
-          // 1622 -> 1638 us).
-          if (!warp_wait(&ctrl.p_free[s], (n_sp - 1u) & 1u, ctrl, p.status, lane)) return k;
+        if (half == 0) {
+          // PV(s, t - 1) reads the P columns and accumulates into O: it must have finished before either is written
+          // (by now it has had the whole first half of the exponentials to do so; at a slot's first step the barrier
+          // is complete or in its initial phase).  One vote decides about both, the wait and the rare rescale: each
+          // vote and branch in this loop costs the warp about 100 cycles of its 2 700 per tile, and nothing else
+          // of the slot runs in them.  Votes of their own, one before and one within the exponentials -> one here:
+          // VOTETIMES
+          if (!__all_sync(0xffffffffu, mbar_test_wait(&ctrl.p_free[s], (n_sp - 1u) & 1u) && !need)) {
+            if (!warp_wait(&ctrl.p_free[s], (n_sp - 1u) & 1u, ctrl, p.status, lane)) return k;
+            if (__any_sync(0xffffffffu, need)) {
+              tc_fence_after();
+              // kept short, so that the loop around it needs fewer instructions from the cache
+              const float v = need ? ex2_approx(m_old - m_ref) : 1.0f;
+              l *= v;
+#pragma unroll 1
+              for (int c = 0; c < D / 16; ++c) {
+                uint32_t regs[16];
+                tmem_ld16(t_o + c * 16, regs);
+                tc_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 16; ++i) regs[i] = __float_as_uint(__uint_as_float(regs[i]) * v);
+                tmem_st16(t_o + c * 16, regs);
+              }
+            }
+          }
           tc_fence_after();
         }
         tmem_st32(t_p + half * 32, packed);
