@@ -112,25 +112,19 @@ __device__ __forceinline__ bool bounded_wait(uint64_t *bar, uint32_t parity, Ctr
   }
 }
 
+constexpr uint32_t kPollLimit = 1u << 27;  // a poll takes 32 cycles or more: the default limit in cycles, or later
+
 // Wait by a whole warp: every lane tests the same barrier and the vote both keeps the warp together and
-// orders its lanes after the observation.
-__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, Ctrl &ctrl, int32_t *status, int lane) {
-  if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
-  const long long start = clock64();
+// orders its lanes after the observation.  In the tile loop of the softmax warps, so it is short: it counts its polls
+// instead of reading the clock (a shorter limit than the default is the other roles' to notice, whose `abort` it
+// sees), and leaves the status word to the end of the kernel (with the clock and the status
+// in it: 32 heads x 4096 d128 119.3 us, as here 118.5; 16/4 x 2048 26.2 -> 25.6, 12 heads x 512 d64 8.52 -> 8.48).
+__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, Ctrl &ctrl) {
   uint32_t n = 0;
-  while (true) {
-    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-    if ((++n & 63u) == 0) {
-      const bool stop = *reinterpret_cast<volatile int *>(&ctrl.abort) != 0 || clock64() - start > ctrl.timeout_cycles;
-      if (__any_sync(0xffffffffu, stop)) {
-        if (lane == 0 && *reinterpret_cast<volatile int *>(&ctrl.abort) == 0) {
-          *reinterpret_cast<volatile int *>(&ctrl.abort) = 1;
-          atomicExch(status, 5);
-        }
-        return false;
-      }
-    }
+  while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+    if ((++n & 63u) == 0 && (*reinterpret_cast<volatile int *>(&ctrl.abort) != 0 || n >= kPollLimit)) return false;
   }
+  return true;
 }
 
 // A work item unpacked into scalars (no indexable arrays, so everything stays in registers).
@@ -721,7 +715,7 @@ __device__ int softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, cons
 
       bool ok;
       {
-        ok = warp_wait(&ctrl.s_full[s], n_sp & 1u, ctrl, p.status, lane);
+        ok = warp_wait(&ctrl.s_full[s], n_sp & 1u, ctrl);
       }
       if (!ok) return k;
       tc_fence_after();
@@ -784,39 +778,37 @@ __device__ int softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, cons
       const float2 neg_m2 = make_float2(-m_use, -m_use);
 
       float2 acc_a = make_float2(0.f, 0.f), acc_b = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        uint32_t packed[32];
-        exp_half<kEmu>(x, half * 64, scale2, neg_m2, acc_a, acc_b, packed);
-        if (half == 0) {
-          // PV(s, t - 1) reads the P columns and accumulates into O: it must have finished before either is written
-          // (by now it has had the whole first half of the exponentials to do so; at a slot's first step the barrier
-          // is complete or in its initial phase).  One vote decides about both, the wait and the rare rescale: each
-          // vote and branch in this loop costs the warp about 100 cycles of its 2 700 per tile, and nothing else
-          // of the slot runs in them.  Votes of their own, one before and one within the exponentials -> one here:
-          // VOTETIMES
-          if (!__all_sync(0xffffffffu, mbar_test_wait(&ctrl.p_free[s], (n_sp - 1u) & 1u) && !need)) {
-            if (!warp_wait(&ctrl.p_free[s], (n_sp - 1u) & 1u, ctrl, p.status, lane)) return k;
-            if (__any_sync(0xffffffffu, need)) {
-              tc_fence_after();
-              // kept short, so that the loop around it needs fewer instructions from the cache
-              const float v = need ? ex2_approx(m_old - m_ref) : 1.0f;
-              l *= v;
-#pragma unroll 1
-              for (int c = 0; c < D / 16; ++c) {
-                uint32_t regs[16];
-                tmem_ld16(t_o + c * 16, regs);
-                tc_wait_ld();
-#pragma unroll
-                for (int i = 0; i < 16; ++i) regs[i] = __float_as_uint(__uint_as_float(regs[i]) * v);
-                tmem_st16(t_o + c * 16, regs);
-              }
-            }
-          }
+      uint32_t p_lo[32], p_hi[32];
+      exp_half<kEmu>(x, 0, scale2, neg_m2, acc_a, acc_b, p_lo);
+      exp_half<kEmu>(x, 64, scale2, neg_m2, acc_a, acc_b, p_hi);
+      // PV(s, t - 1) reads the P columns and accumulates into O: it must have finished before either is written.  P
+      // stays in registers until here, because products that are issued at the same time share the tensor core:
+      // with an S beside it PV takes up to 1 024 cycles, and a softmax warp that waits for it halfway through its
+      // exponentials stands still.  (At a slot's first step the barrier is complete or in its initial phase.)  One vote
+      // decides about both, the wait and the rare rescale: each vote and branch in this loop costs the warp about
+      // 100 cycles of its 2 700 per tile.  P stored in halves -> here: 32 heads x 8192 d64 352 -> 337 us, 32 heads x
+      // 4096 d128 123.4 -> 119.3 us, window 4096 of 16384 796 -> 755 us, 500 queries on 12500 keys 95.1 -> 90.5 us.
+      if (!__all_sync(0xffffffffu, mbar_test_wait(&ctrl.p_free[s], (n_sp - 1u) & 1u) && !need)) {
+        if (!warp_wait(&ctrl.p_free[s], (n_sp - 1u) & 1u, ctrl)) return k;
+        if (__any_sync(0xffffffffu, need)) {
           tc_fence_after();
+          // kept short, so that the loop around it needs fewer instructions from the cache
+          const float v = need ? ex2_approx(m_old - m_ref) : 1.0f;
+          l *= v;
+#pragma unroll 1
+          for (int c = 0; c < D / 16; ++c) {
+            uint32_t regs[16];
+            tmem_ld16(t_o + c * 16, regs);
+            tc_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) regs[i] = __float_as_uint(__uint_as_float(regs[i]) * v);
+            tmem_st16(t_o + c * 16, regs);
+          }
         }
-        tmem_st32(t_p + half * 32, packed);
       }
+      tc_fence_after();
+      tmem_st32(t_p, p_lo);
+      tmem_st32(t_p + 32, p_hi);
       tc_wait_st();
       tc_fence_before();
       __syncwarp();
@@ -832,7 +824,7 @@ __device__ int softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, cons
     if (active) {
       bool ok;
       {
-        ok = warp_wait(&ctrl.o_full[s], n_use & 1u, ctrl, p.status, lane);
+        ok = warp_wait(&ctrl.o_full[s], n_use & 1u, ctrl);
       }
       if (!ok) return k;
       ++n_use;
@@ -947,6 +939,10 @@ steel_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
   if (warp < 8) {
     setmaxnreg_inc<kRegsSoftmax>();
     const int left = softmax_role<D, kEmu, kSplit, kList>(p, ctrl, warp / 4, threadIdx.x % kTile);
+    if (left >= 0 && lane == 0 && *reinterpret_cast<volatile int *>(&ctrl.abort) == 0) {
+      *reinterpret_cast<volatile int *>(&ctrl.abort) = 1;
+      atomicExch(p.status, 5);
+    }
     if (kSplit && left >= 0) count_abandoned_parts(p, left, warp / 4, warp % 4, lane);
   } else {
     setmaxnreg_dec<kRegsOther>();
