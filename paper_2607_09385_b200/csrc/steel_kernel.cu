@@ -120,6 +120,7 @@ constexpr uint32_t kPollLimit = 1u << 27;  // a poll takes 32 cycles or more: th
 // sees), and leaves the status word to the end of the kernel (with the clock and the status
 // in it: 32 heads x 4096 d128 119.3 us, as here 118.5; 16/4 x 2048 26.2 -> 25.6, 12 heads x 512 d64 8.52 -> 8.48).
 __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, Ctrl &ctrl) {
+  if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
   uint32_t n = 0;
   while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
     if ((++n & 63u) == 0 && (*reinterpret_cast<volatile int *>(&ctrl.abort) != 0 || n >= kPollLimit)) return false;
