@@ -215,6 +215,7 @@ steel_status_t launch_with_params(const steel_attn_params_t &p, KernelParams kp,
     m.v_ptr = v;
   }
   kp.o = o;
+  kp.o_aligned32 = (reinterpret_cast<uintptr_t>(o) & 31u) == 0;
   kp.lse = lse;
   kp.heads_kv = p.heads_kv;
   kp.seq_q = p.seq_q;

@@ -682,6 +682,7 @@ __device__ int softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, cons
   const int k_end = p.cta_begin[blockIdx.x + 1];
   for (int k = p.cta_begin[blockIdx.x]; k < k_end; ++k) {
     const Item w = load_item(p.items, k);
+    if (k + 1 < k_end) prefetch_l1(p.items + k + 1);  // a miss at the start of an item costs 1 000 cycles
     if (w.head(s) < 0) continue;
     const int row = w.qtile(s) * kTile + r;
     const size_t out_row = (size_t(w.batch) * p.heads_q + w.head(s)) * size_t(p.rows_q) + size_t(row);
@@ -692,10 +693,18 @@ __device__ int softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, cons
     // Range items: tiles f_lo .. f_hi need no element-wise mask (case ii).  List items carry it in the entry.
     int f_lo = 0, f_hi = p.seq_kv / kTile - 1;
     const int r0 = w.qtile(s) * kTile, r1 = min(r0 + kTile, p.rows_q) - 1;
-    const bool one_head = r0 / p.seq_q == r1 / p.seq_q;  // else the tile spans all positions
-    if (causal) f_hi = min(f_hi, ((one_head ? r0 % p.seq_q : 0) + off + 1) / kTile - 1);
+    // first and last position in the tile; one that spans several heads spans all positions.  (Divisions only where rows
+    // of several heads are packed: 100 cycles each, and one per partial tile.)
+    int pos0 = r0, pos1 = r1, pos_row = row;
+    if (p.rows_q != p.seq_q) {
+      const bool one_head = r0 / p.seq_q == r1 / p.seq_q;
+      pos0 = one_head ? r0 % p.seq_q : 0;
+      pos1 = one_head ? r1 % p.seq_q : p.seq_q - 1;
+      pos_row = row % p.seq_q;
+    }
+    if (causal) f_hi = min(f_hi, (pos0 + off + 1) / kTile - 1);
     if (windowed) {
-      const int first = (one_head ? r1 % p.seq_q : p.seq_q - 1) + off - p.window + 1;
+      const int first = pos1 + off - p.window + 1;
       f_lo = first > 0 ? (first + kTile - 1) / kTile : 0;
     }
     const uint32_t *entries = reinterpret_cast<const uint32_t *>(p.steps + w.list_off()) + s;
@@ -737,7 +746,7 @@ __device__ int softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, cons
 
       if (partial) {
         // visible columns of this row form one interval [c_lo, c_hi] of the tile
-        const int pos = row % p.seq_q + off, jb = j * kTile;  // key position aligned with the row's query
+        const int pos = pos_row + off, jb = j * kTile;  // key position aligned with the row's query
         int c_hi = min(kTile - 1, p.seq_kv - 1 - jb), c_lo = 0;
         if (causal) c_hi = min(c_hi, pos - jb);
         if (windowed) c_lo = max(c_lo, pos - p.window + 1 - jb);
@@ -856,15 +865,23 @@ __device__ int softmax_role(const KernelParams &p, Ctrl &ctrl, const int s, cons
           tmem_ld32(t_o + c * 32, regs);
           tc_wait_ld();
           if (valid) {
-            uint4 *dst = reinterpret_cast<uint4 *>(o_base + out_row * D + c * 32);
+            // A row's 64 bytes as two 32-byte stores: whole sectors, and half as many passes through L1 (each lane
+            // writes a line of its own, and what bounds the epilogue is one line per cycle).  16-byte stores ->
+            // here: batch 4 24/8 x 1777 79.8 -> 77.8 us, window 4096 of 16384 744 -> 731 us.  Turning pieces
+            // among four lanes by shuffles, for whole lines, took longer than it saved (95 us).
+            __nv_bfloat16 *dst = o_base + out_row * D + c * 32;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              uint4 v;
-              v.x = pack_bf16x2(__uint_as_float(regs[8 * i + 0]) * inv, __uint_as_float(regs[8 * i + 1]) * inv);
-              v.y = pack_bf16x2(__uint_as_float(regs[8 * i + 2]) * inv, __uint_as_float(regs[8 * i + 3]) * inv);
-              v.z = pack_bf16x2(__uint_as_float(regs[8 * i + 4]) * inv, __uint_as_float(regs[8 * i + 5]) * inv);
-              v.w = pack_bf16x2(__uint_as_float(regs[8 * i + 6]) * inv, __uint_as_float(regs[8 * i + 7]) * inv);
-              dst[i] = v;
+            for (int i = 0; i < 2; ++i) {
+              uint32_t v[8];
+#pragma unroll
+              for (int e = 0; e < 8; ++e)
+                v[e] = pack_bf16x2(__uint_as_float(regs[16 * i + 2 * e]) * inv, __uint_as_float(regs[16 * i + 2 * e + 1]) * inv);
+              if (p.o_aligned32) {
+                store_global32(dst + 16 * i, v);
+              } else {
+                reinterpret_cast<uint4 *>(dst)[2 * i] = make_uint4(v[0], v[1], v[2], v[3]);
+                reinterpret_cast<uint4 *>(dst)[2 * i + 1] = make_uint4(v[4], v[5], v[6], v[7]);
+              }
             }
           }
         }

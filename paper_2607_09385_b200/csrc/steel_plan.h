@@ -56,6 +56,7 @@ struct KernelParams {
   const StepPair *steps;       // list-kind step entries
   void *o;                   // bf16 [batch, heads_q, seq_q, head_dim]
   float *lse;                // fp32 [batch, heads_q, seq_q] or null
+  bool o_aligned32;          // `o` is a multiple of 32 (16 is what callers promise)
   int32_t *status;           // device status word (0 ok, else STEEL_ERR_TIMEOUT)
   const SplitTile *split_tiles;  // null: no query tile is split
   float *parts;              // per part: O as float4 [head_dim / 4][part_rows], then (m, l) [part_rows]

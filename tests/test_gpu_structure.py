@@ -136,3 +136,22 @@ def test_rows_masked_in_their_first_tile():
     assert not torch.isnan(o.float()).any() and not torch.isnan(lse).any()
     H.assert_parity(w, data, o, lse, H.all_rows(w))
     attn.close()
+
+
+@pytest.mark.parametrize("head_dim", [64, 128])
+@pytest.mark.parametrize("seq", [1, 129, 300])
+def test_output_at_any_16_byte_boundary(head_dim, seq):
+    """O may start at any multiple of 16 bytes; where it is no multiple of 32 the stores are narrower, the bytes the same."""
+    g = torch.Generator(device="cuda").manual_seed(head_dim + seq)
+    q, k, v = (torch.randn((2, 3, seq, head_dim), generator=g, device="cuda").to(torch.bfloat16) for _ in "qkv")
+    attn = binding.SteelAttention(2, 3, 3, seq, seq, head_dim, 0.125, CAUSAL)
+    outs = []
+    for offset in (0, 8):  # elements of 2 bytes
+        room = torch.full((q.numel() + 16,), float("nan"), dtype=torch.bfloat16, device="cuda")
+        o = room[offset:offset + q.numel()].view(q.shape)
+        assert o.data_ptr() % 32 == 2 * offset
+        attn.run(q, k, v, o)
+        assert attn.last_status() == binding.STEEL_OK
+        assert room[:offset].isnan().all() and room[offset + q.numel():].isnan().all()  # nothing beside it
+        outs.append(o)
+    assert torch.equal(outs[0], outs[1])
