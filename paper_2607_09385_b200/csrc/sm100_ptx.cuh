@@ -253,6 +253,11 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
+__device__ __forceinline__ float fmax_nan(float a, float b) {  // NaN if either is
+  float d;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
 // Releases the caller's (and, after a barrier, its warp's) writes and acquires those of earlier arrivals.
 __device__ __forceinline__ int atomic_add_acq_rel(int *p, int v) {
   int old;
