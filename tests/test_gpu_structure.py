@@ -155,3 +155,41 @@ def test_output_at_any_16_byte_boundary(head_dim, seq):
         assert room[:offset].isnan().all() and room[offset + q.numel():].isnan().all()  # nothing beside it
         outs.append(o)
     assert torch.equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("head_dim", [64, 128])
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+def test_a_score_that_is_no_number_reaches_its_rows_from_every_column(head_dim, value):
+    """At head_dim 64 some columns of a tile take another exponential than the others.  A key that is NaN or infinite must
+    show in every row that sees it, whatever its column, and in no other row."""
+    g = torch.Generator(device="cuda").manual_seed(head_dim)
+    q, k, v = (torch.rand((1, 1, 128, head_dim), generator=g, device="cuda").to(torch.bfloat16) for _ in "qkv")  # q > 0
+    attn = binding.SteelAttention(1, 1, 1, 128, 128, head_dim, 0.125, CAUSAL)
+    o_ref, lse_ref = attn.run(q, k, v)
+    for j in range(128):
+        bad = k.clone()
+        bad[0, 0, j] = value
+        o, lse = attn.run(q, bad, v)
+        assert o[0, 0, j:].isnan().all(), j
+        assert torch.equal(o[0, 0, :j], o_ref[0, 0, :j]) and torch.equal(lse[0, 0, :j], lse_ref[0, 0, :j]), j
+
+
+def test_far_apart_scores_at_head_dim_64():
+    """Scores from one to far below the smallest number's logarithm beneath the maximum, in every column: weights that
+    vanish are exactly 0, the others right to bf16's rounding (V is one-hot in the key's column, so O is the weight)."""
+    n, d = 64, 64
+    q = torch.zeros((1, 1, 128, d), device="cuda")
+    q[0, 0, :, 0] = torch.arange(128, device="cuda") * 2.0   # steepness per row
+    k = torch.zeros((1, 1, n, d), device="cuda")
+    k[0, 0, :, 0] = -torch.arange(n, device="cuda")          # score of key j: -2 * row * j (exact in bf16)
+    v = torch.eye(n, device="cuda")[None, None]
+    attn = binding.SteelAttention(1, 1, 1, 128, n, d, 0.5, 0)
+    o, lse = attn.run(q.to(torch.bfloat16), k.to(torch.bfloat16), v.to(torch.bfloat16))
+    y = -(torch.arange(128, dtype=torch.float64)[:, None] * torch.arange(n, dtype=torch.float64)[None])
+    p = torch.softmax(y, 1)
+    got = o[0, 0].double().cpu()
+    # P and O are rounded to bf16: 8 significant bits, so at most half of 2^-7 each, relative, and (1 + 2^-8)^2 together;
+    # the exponentials and the fp32 row sum add less than 2^-20
+    assert (got - p).abs().le(p * (2.0 ** -7 + 2.0 ** -16 + 2.0 ** -20) + 1e-37).all()
+    assert (got[p < 1e-45] == 0).all()
+    assert torch.allclose(lse[0, 0].double().cpu(), torch.logsumexp(y, 1), rtol=0, atol=2e-6)  # fp32 values up to 4.2
