@@ -25,7 +25,7 @@ constexpr size_t kMaxItems = 16384;   // work items (64 bytes each)
 constexpr size_t kMaxCtas = 1024;     // persistent CTAs (+1 range entry)
 constexpr size_t kMaxSteps = 131072;  // explicit step-list entries of bitmap masks (8 bytes each)
 // The call's lists are packed one behind the other, so that one copy brings them: status word, per-CTA
-// ranges, items, steps.
+// ranges, items, steps (or the bitmap, behind which the device writes the steps).
 constexpr size_t kOffCtaBegin = 256;
 constexpr size_t round16(size_t n) { return (n + 15) / 16 * 16; }
 constexpr size_t kScratchBytes = kOffCtaBegin + round16((kMaxCtas + 1) * sizeof(int32_t)) +
@@ -59,6 +59,25 @@ steel_status_t setup_device(int device, unsigned char **base, int *sm_count) {
   return STEEL_OK;
 }
 
+// The step lists of single query tiles, from the bitmap: one warp per item, one lane per key tile, 32 at a time; a vote
+// gives each visible tile its place, in ascending order.  Bound by the latency of its few loads.  With the entries
+// made and copied by the host the call took 175 us (8 heads x 4096 d64, 64-token blocks), as here 144.
+constexpr int kListWarps = 8;
+__global__ void write_lists(const WorkItem *items, int n_items, const uint32_t *bitmap, BitmapMask mask, StepPair *steps) {
+  const int n = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
+  if (n >= n_items || items[n].kind != 1) return;
+  const WorkItem &w = items[n];
+  const uint32_t *rows = bitmap + size_t(w.head[0]) * mask.blocks_q * mask.words;
+  StepPair *out = steps + w.j0[0];
+  for (int j0 = 0, at = 0; j0 < mask.key_tiles() && at < w.n_steps; j0 += 32) {
+    const uint32_t e = j0 + lane < mask.key_tiles() ? mask.entry(rows, w.qtile[0], j0 + lane) : 0u;
+    const uint32_t seen = __ballot_sync(0xffffffffu, e != 0);
+    const int place = at + __popc(seen & ((1u << lane) - 1u));
+    if (e != 0 && place < w.n_steps) out[place] = StepPair{{e, 0u}};
+    at += __popc(seen);
+  }
+}
+
 }  // namespace
 
 extern "C" steel_status_t steel_attn_run_noalloc(const steel_attn_params_t *params, const void *q, const void *k,
@@ -86,33 +105,55 @@ extern "C" steel_status_t steel_attn_run_noalloc(const steel_attn_params_t *para
 
   // Host memory only.  One query tile per item can need more list entries than pairs: where the fixed array
   // has no room for it, the paired plan is taken.  What fits in neither way is refused, not truncated.
+  // Where the items of a bitmap mask are single query tiles, their lists are written on the device, from the bitmap,
+  // if that fits into the array beside them; else here.
   Plan plan;
   bool fits = false;
-  std::vector<unsigned char> lists;
-  size_t off_items = 0, off_steps = 0;
+  std::vector<unsigned char> lists;  // what is copied: all but the status word's rest and device-written lists
+  size_t off_items = 0, off_steps = 0, off_bitmap = 0;
+  const BitmapMask mask = bitmap_mask(*params);
+  const size_t bitmap_bytes =
+      (params->mask.flags & STEEL_MASK_BITMAP) ? size_t(params->heads_q) * mask.blocks_q * mask.words * sizeof(uint32_t) : 0;
+  bool device_lists = false;
   try {
-    for (Spread spread : {Spread::kTiles, Spread::kNone}) {
-      st = build_plan(params, sm_count, &plan, /*stats=*/false, spread);
-      if (st != STEEL_OK) return st;
-      fits = plan.items.size() <= kMaxItems && plan.steps.size() <= kMaxSteps && plan.cta_begin.size() <= kMaxCtas + 1;
-      if (fits) break;
-    }
+    auto plan_as = [&](Spread spread, bool on_device) {
+      st = build_plan(params, sm_count, &plan, /*stats=*/false, spread, nullptr, on_device);
+      if (st != STEEL_OK) return;
+      fits = plan.items.size() <= kMaxItems && size_t(plan.n_steps) <= kMaxSteps && plan.cta_begin.size() <= kMaxCtas + 1;
+      off_items = kOffCtaBegin + round16(plan.cta_begin.size() * sizeof(int32_t));
+      off_steps = off_bitmap = off_items + plan.items.size() * sizeof(WorkItem);
+      device_lists = plan.steps.empty() && plan.n_steps > 0;
+      if (device_lists) off_steps += round16(bitmap_bytes);
+    };
+    plan_as(Spread::kTiles, bitmap_bytes > 0);
+    if (st == STEEL_OK && fits && device_lists && off_steps + size_t(plan.n_steps) * sizeof(StepPair) > kScratchBytes)
+      plan_as(Spread::kTiles, false);
+    if (st == STEEL_OK && !fits) plan_as(Spread::kNone, false);
+    if (st != STEEL_OK) return st;
     if (!fits) return STEEL_ERR_UNSUPPORTED;
-    off_items = kOffCtaBegin + round16(plan.cta_begin.size() * sizeof(int32_t));
-    off_steps = off_items + plan.items.size() * sizeof(WorkItem);
-    lists.resize(off_steps + plan.steps.size() * sizeof(StepPair));
+    lists.resize(device_lists ? off_bitmap + bitmap_bytes : off_steps + plan.steps.size() * sizeof(StepPair));
   } catch (const std::bad_alloc &) {
     return STEEL_ERR_ALLOC;
   }
   std::memcpy(lists.data() + kOffCtaBegin, plan.cta_begin.data(), plan.cta_begin.size() * sizeof(int32_t));
-  if (!plan.items.empty()) std::memcpy(lists.data() + off_items, plan.items.data(), off_steps - off_items);
-  if (!plan.steps.empty()) std::memcpy(lists.data() + off_steps, plan.steps.data(), lists.size() - off_steps);
+  if (!plan.items.empty()) std::memcpy(lists.data() + off_items, plan.items.data(), plan.items.size() * sizeof(WorkItem));
+  if (device_lists)
+    std::memcpy(lists.data() + off_bitmap, params->mask.bitmap, bitmap_bytes);
+  else if (!plan.steps.empty())
+    std::memcpy(lists.data() + off_steps, plan.steps.data(), plan.steps.size() * sizeof(StepPair));
 
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   // The array still holds the previous call's lists and status word: overwrite both (the word with 0).
   if (cudaMemcpyAsync(base, lists.data(), lists.size(), cudaMemcpyHostToDevice, stream) != cudaSuccess) {
     cudaGetLastError();
     return STEEL_ERR_CUDA;
+  }
+  if (device_lists) {
+    const int n_items = int(plan.items.size());
+    write_lists<<<(n_items + kListWarps - 1) / kListWarps, kListWarps * 32, 0, stream>>>(
+        reinterpret_cast<const WorkItem *>(base + off_items), n_items, reinterpret_cast<const uint32_t *>(base + off_bitmap),
+        mask, reinterpret_cast<StepPair *>(base + off_steps));
+    if (cudaGetLastError() != cudaSuccess) return STEEL_ERR_CUDA;
   }
   KernelParams kp{};  // no split query tiles: their buffers have no room in the array
   kp.items = reinterpret_cast<const WorkItem *>(base + off_items);

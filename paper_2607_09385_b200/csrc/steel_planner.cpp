@@ -95,6 +95,35 @@ struct Ctx {
     rows(I, kTile, i0, i1);
     whole_range(i0, i1, kTile, &whole_lo, &whole_hi);
     const bool ragged = p->seq_kv % kTile != 0;
+    kept_words(h, I, [&](int64_t w, uint32_t inside, const uint32_t (&set)[2], bool two_rows, uint32_t kept) {
+      const int per = int(kTile / bq);
+      for (; kept; kept &= kept - 1) {
+        const int bit0 = __builtin_ctz(kept);
+        const int64_t J = (32 * w + bit0) / per;
+        uint32_t sub = 0xF;
+        bool full = J >= whole_lo && J <= whole_hi;
+        if (per == 2) {  // sub-blocks TL, TR, BL, BR; those outside the problem do not make a tile partial
+          const uint32_t a = (set[0] >> bit0) & 3u, b = (set[1] >> bit0) & 3u, in = (inside >> bit0) & 3u;
+          sub = a | b << 2;
+          full = full && a == in && (!two_rows || b == in);
+        }
+        uint32_t e = uint32_t(J) | kEntryPresent | (sub << kEntrySubShift);
+        if (!full || (ragged && J == tkv128 - 1)) e |= kEntryPartial;
+        out->push_back(e);
+      }
+    });
+  }
+  // Their number.
+  int64_t count_entries(int h, int64_t I) const {
+    int64_t n = 0;
+    kept_words(h, I, [&](int64_t, uint32_t, const uint32_t (&)[2], bool, uint32_t kept) { n += __builtin_popcount(kept); });
+    return n;
+  }
+
+  // The words of query tile I's blocks that hold visible ones: visit(word, bits inside the problem, bits of the tile's
+  // rows of blocks, whether there are two, one bit per visible key tile).
+  template <class Visit>
+  void kept_words(int h, int64_t I, Visit &&visit) const {
     const int per = int(kTile / bq);  // blocks of a tile in each direction: 1 or 2
     const uint32_t *row[2] = {nullptr, nullptr};
     int64_t lo[2] = {0, 0}, hi[2] = {-1, -1};
@@ -116,20 +145,7 @@ struct Ctx {
           kept |= set[a] & range_bits(w, lo[a], hi[a]);
         }
       if (per == 2) kept = (kept | kept >> 1) & 0x55555555u;
-      for (; kept; kept &= kept - 1) {
-        const int bit0 = __builtin_ctz(kept);
-        const int64_t J = (32 * w + bit0) / per;
-        uint32_t sub = 0xF;
-        bool full = J >= whole_lo && J <= whole_hi;
-        if (per == 2) {  // sub-blocks TL, TR, BL, BR; those outside the problem do not make a tile partial
-          const uint32_t a = (set[0] >> bit0) & 3u, b = (set[1] >> bit0) & 3u, in = (inside >> bit0) & 3u;
-          sub = a | b << 2;
-          full = full && a == in && (!row[1] || b == in);
-        }
-        uint32_t e = uint32_t(J) | kEntryPresent | (sub << kEntrySubShift);
-        if (!full || (ragged && J == tkv128 - 1)) e |= kEntryPartial;
-        out->push_back(e);
-      }
+      visit(w, inside, set, row[1] != nullptr, kept);
     }
   }
 };
@@ -465,20 +481,21 @@ steel_status_t place_items(const steel_attn_params_t &p, int num_ctas, std::vect
     for (int id : per_cta[cta]) {
       Draft &d = drafts[id];
       if (d.w.kind == 1) {
-        d.w.j0[0] = int32_t(plan->steps.size());
+        d.w.j0[0] = int32_t(plan->n_steps);
+        plan->n_steps += d.list.empty() ? int64_t(d.w.n_steps) : int64_t(d.list.size());
         plan->steps.insert(plan->steps.end(), d.list.begin(), d.list.end());
       }
       plan->items.push_back(d.w);
     }
     plan->cta_begin.push_back(int32_t(plan->items.size()));
   }
-  if (plan->steps.size() >= (size_t(1) << 31)) return STEEL_ERR_UNSUPPORTED;
+  if (plan->n_steps >= (int64_t(1) << 31)) return STEEL_ERR_UNSUPPORTED;
 
   // ---- statistics of the executed plan
   steel_attn_stats_t &s = plan->stats;
   s.work_items = int64_t(plan->items.size());
   s.grid = grid;
-  s.list_entries = int64_t(plan->steps.size());
+  s.list_entries = plan->n_steps;
   s.max_cta_steps = 0;
   for (int cta = 0; cta < grid; ++cta) {
     int64_t st_sum = 0;
@@ -514,7 +531,7 @@ steel_status_t validate_params(const steel_attn_params_t *p) {
 }
 
 steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan, bool stats, Spread spread,
-                          Plan *whole) {
+                          Plan *whole, bool device_lists) {
   steel_status_t st = validate_params(p);
   if (st != STEEL_OK) return st;
   const int policy = p->policy;
@@ -538,6 +555,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
 
   plan->items.clear();
   plan->steps.clear();
+  plan->n_steps = 0;
   plan->split_tiles.clear();
   plan->n_parts = 0;
   plan->packed = false;
@@ -602,17 +620,57 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
   }
   const int64_t rows_q = plan_rows_q(*p, *plan);
   std::vector<std::vector<Task>> tasks(heads);  // [h][I]
-  const size_t key_words = size_t(c.tkv128 + 63) / 64;
-  std::vector<uint32_t> entries;
-  std::vector<uint64_t> keys;  // bitmap masks: the key tiles of each task as bits
-  if (c.bitmap) keys.assign(size_t(heads) * size_t(c.tq128) * key_words, 0);
+  // Bitmap masks: the search for partners takes most of the planning, so where no key range may be cut the
+  // choice between pairs and single tiles is made on the lengths alone (partners are of similar length).
+  const bool on_lengths = spread == Spread::kTiles && c.bitmap && int64_t(p->batch) * heads * c.tq128 < 8 * num_ctas;
   for (int h = 0; h < heads; ++h) {
     tasks[h].resize(c.tq128);
     for (int64_t I = 0; I < c.tq128; ++I) {
       Task &t = tasks[h][I];
       t.h = h;
       t.I = I;
-      if (c.bitmap) {
+      if (on_lengths) {
+        t.entries.n = size_t(c.count_entries(h, I));
+      } else if (!c.bitmap && h > 0) {
+        t.jlo = tasks[0][I].jlo;
+        t.jhi = tasks[0][I].jhi;
+      } else if (!c.bitmap) {
+        // kept key tiles of a row of tiles form one contiguous range under causal / window masks
+        key_range(c, rows_q, I, &t.jlo, &t.jhi);
+      }
+    }
+  }
+  bool pair = true;
+  if (on_lengths) {
+    std::vector<double> paired, single;
+    double work = 0.0;
+    std::vector<int64_t> count;
+    for (int g = 0; g < p->heads_kv; ++g) {
+      count.clear();
+      for (int h = g * G; h < (g + 1) * G; ++h)
+        for (const Task &t : tasks[h])
+          if (t.count() > 0) count.push_back(t.count());
+      std::sort(count.begin(), count.end(), std::greater<int64_t>());
+      for (int batch = 0; batch < p->batch; ++batch)
+        for (size_t n = 0; n < count.size(); ++n) {
+          single.push_back(kSingleStep * double(count[n]) + kItemOverheadSteps);
+          if (n % 2) continue;
+          paired.push_back((n + 1 < count.size() ? 1.0 : kSingleStep) * double(count[n]) + kItemOverheadSteps);
+          work += paired.back();
+        }
+    }
+    const double load = makespan(std::move(paired), num_ctas);
+    pair = !(load > 1.1 * work / num_ctas && makespan(std::move(single), num_ctas) < 0.95 * load);
+  }
+  device_lists = device_lists && on_lengths && !pair && !stats;
+  const size_t key_words = size_t(c.tkv128 + 63) / 64;
+  std::vector<uint32_t> entries;
+  std::vector<uint64_t> keys;  // the key tiles of each task as bits
+  if (c.bitmap && !device_lists) {
+    keys.assign(size_t(heads) * size_t(c.tq128) * key_words, 0);
+    for (int h = 0; h < heads; ++h)
+      for (int64_t I = 0; I < c.tq128; ++I) {
+        Task &t = tasks[h][I];
         t.entries.at = entries.size();
         c.entries(h, I, &entries);
         t.entries.n = entries.size() - t.entries.at;
@@ -620,22 +678,13 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
           const uint32_t J = entries[n] & kEntryTileMask;
           keys[size_t(h * c.tq128 + I) * key_words + J / 64] |= uint64_t(1) << (J % 64);
         }
-      } else if (h > 0) {
-        t.jlo = tasks[0][I].jlo;
-        t.jhi = tasks[0][I].jhi;
-      } else {
-        // kept key tiles of a row of tiles form one contiguous range under causal / window masks
-        key_range(c, rows_q, I, &t.jlo, &t.jhi);
       }
-    }
+    for (std::vector<Task> &row : tasks)
+      for (Task &t : row) t.entries.first = entries.data() + t.entries.at;
   }
-
-  for (std::vector<Task> &row : tasks)
-    for (Task &t : row) t.entries.first = entries.data() + t.entries.at;
 
   // ---- work items: pair query tiles that can share K/V loads
   std::vector<Draft> drafts, uncut;  // `uncut`: for `whole`
-  bool pair = true;
   auto finish_range = [&](const Task *a, const Task *b, int batch, int g) {
     Draft d{};
     d.group = g;
@@ -702,8 +751,10 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
       ea.insert(ea.end(), rest_a.begin(), rest_a.end());
       eb.insert(eb.end(), rest_b.begin(), rest_b.end());
     } else {
-      d.list.reserve(na);
-      for (uint32_t e : a->entries) d.list.push_back(StepPair{{e, 0u}});
+      if (!device_lists) {
+        d.list.reserve(na);
+        for (uint32_t e : a->entries) d.list.push_back(StepPair{{e, 0u}});
+      }
       drafts.push_back(std::move(d));
       return;
     }
@@ -752,7 +803,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
           std::vector<Length> by_length;
           by_length.reserve(live.size());
           for (const Task *t : live)
-            by_length.push_back({t->count(), &keys[size_t(t->h * c.tq128 + t->I) * key_words], t});
+            by_length.push_back({t->count(), pair ? &keys[size_t(t->h * c.tq128 + t->I) * key_words] : nullptr, t});
           if (pair)
             std::stable_sort(by_length.begin(), by_length.end(), [](const Length &a, const Length &b) { return a.n > b.n; });
           // among the next few tasks of similar length, take the partner with the most key tiles in common
@@ -800,31 +851,6 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
       }
     }
   };
-  // Bitmap masks: the search for partners takes most of the planning, so where no key range may be cut the
-  // choice between pairs and single tiles is made on the lengths alone (partners are of similar length).
-  bool chosen = false;
-  if (spread == Spread::kTiles && c.bitmap && int64_t(p->batch) * heads * c.tq128 < 8 * num_ctas) {
-    std::vector<double> paired, single;
-    double work = 0.0;
-    std::vector<int64_t> count;
-    for (int g = 0; g < p->heads_kv; ++g) {
-      count.clear();
-      for (int h = g * G; h < (g + 1) * G; ++h)
-        for (const Task &t : tasks[h])
-          if (t.count() > 0) count.push_back(t.count());
-      std::sort(count.begin(), count.end(), std::greater<int64_t>());
-      for (int batch = 0; batch < p->batch; ++batch)
-        for (size_t n = 0; n < count.size(); ++n) {
-          single.push_back(kSingleStep * double(count[n]) + kItemOverheadSteps);
-          if (n % 2) continue;
-          paired.push_back((n + 1 < count.size() ? 1.0 : kSingleStep) * double(count[n]) + kItemOverheadSteps);
-          work += paired.back();
-        }
-    }
-    const double load = makespan(std::move(paired), num_ctas);
-    chosen = true;
-    pair = !(load > 1.1 * work / num_ctas && makespan(std::move(single), num_ctas) < 0.95 * load);
-  }
   drafts.reserve(size_t(p->batch) * size_t(heads) * size_t(c.tq128));
   build_drafts();
 
@@ -833,7 +859,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
   // tenth more than the mean.)  Kernel time, paired -> chosen plan: 500 queries on 12500 keys, 32/8 heads,
   // 161 -> 96 us (cut); a decode step of batch 8 on 6001 keys, 32/8 heads, 82 -> 39 us (packed and cut);
   // 12 heads x 512 d64 11.8 -> 9.6 us, 16/4 heads x 2048 d128 35.2 -> 30.7 us (one query tile per item).
-  if (spread != Spread::kNone && !chosen && drafts.size() < size_t(8 * num_ctas)) {
+  if (spread != Spread::kNone && !on_lengths && drafts.size() < size_t(8 * num_ctas)) {
     const double fill = double(std::min<int64_t>(rows_q, kTile)) / kTile;
     double work = 0.0;
     for (const Draft &d : drafts) work += step_cost(d.w) * d.w.n_steps + kItemOverheadSteps;
@@ -879,6 +905,21 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
   if (st != STEEL_OK) return st;
   if (stats) count_tiles(c, *plan, rows_q, &s);
   return STEEL_OK;
+}
+
+BitmapMask bitmap_mask(const steel_attn_params_t &p) {
+  BitmapMask m;
+  m.seq_q = p.seq_q;
+  m.seq_kv = p.seq_kv;
+  m.off = int64_t(p.seq_kv) - p.seq_q;
+  m.window = p.mask.window;
+  m.block = p.mask.block_q ? p.mask.block_q : kTile;
+  m.blocks_q = (p.seq_q + m.block - 1) / m.block;
+  m.blocks_kv = (p.seq_kv + m.block - 1) / m.block;
+  m.words = (m.blocks_kv + 31) / 32;
+  m.causal = (p.mask.flags & STEEL_MASK_CAUSAL) != 0;
+  m.windowed = (p.mask.flags & STEEL_MASK_WINDOW) != 0;
+  return m;
 }
 
 int64_t plan_rows_q(const steel_attn_params_t &p, const Plan &plan) {

@@ -5,6 +5,7 @@
 #include <vector>
 
 #include "../../include/steel_attn.h"
+#include "steel_bitmap.h"
 #include "steel_plan.h"
 
 namespace steel {
@@ -42,6 +43,7 @@ struct Plan {
   std::vector<WorkItem> items;     // in CTA order
   std::vector<int32_t> cta_begin;  // grid + 1
   std::vector<StepPair> steps;     // list-kind entries
+  int64_t n_steps = 0;             // their number; `steps` is empty where the lists are left to the device
   std::vector<SplitTile> split_tiles;
   int32_t n_parts = 0;             // part buffers of all split tiles
   bool packed = false;             // query tiles hold rows of all heads of a group (KernelParams::rows_q)
@@ -59,8 +61,12 @@ enum class Spread {
 // Scheduling policy and the other options come from `p`.  Without `stats` the plan's statistics stay 0 (they
 // take a walk over every block).  Where `plan` cuts key ranges, `whole` (if not null)
 // becomes the plan that would be taken without cuts: items, steps and the statistics of its items.
+// `device_lists`: where the items of a bitmap mask are single query tiles, the plan holds the lengths and places of
+// their lists only; the entry of tile J is BitmapMask::entry, in ascending order of J (Spread::kTiles, no `stats`).
 steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan, bool stats = true,
-                          Spread spread = Spread::kNone, Plan *whole = nullptr);
+                          Spread spread = Spread::kNone, Plan *whole = nullptr, bool device_lists = false);
+
+BitmapMask bitmap_mask(const steel_attn_params_t &p);
 
 // steel_attn_create with a limit on what the plan may do (implemented in steel_attn.cu).
 steel_status_t create_attention(const steel_attn_params_t *params, Spread most, steel_attn_t **out);

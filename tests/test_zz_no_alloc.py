@@ -97,6 +97,34 @@ def test_noalloc_with_packed_heads(shape):
     attn.close()
 
 
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("shape,flags,window", [((2, 4, 2, 700, 1333, 64), CAUSAL | BITMAP, 0), ((1, 3, 3, 1000, 300, 128), BITMAP, 0),
+                                                ((1, 6, 1, 129, 2001, 64), CAUSAL | WINDOW | BITMAP, 900)])
+def test_noalloc_lists_written_on_the_device(shape, flags, window, block):
+    # single query tiles under a bitmap: ragged and unequal lengths, tiles and rows without any visible key
+    b, hq, hkv, sq, skv, d = shape
+    rng = np.random.default_rng(44)
+    q, k, v = (torch.from_numpy(rng.standard_normal(s, np.float32)).to(torch.bfloat16).cuda()
+               for s in ((b, hq, sq, d), (b, hkv, skv, d), (b, hkv, skv, d)))
+    words = -(-(-(-skv // block)) // 32)
+    bits = rng.integers(0, 2 ** 32, (hq, -(-sq // block), words), np.uint32) & rng.integers(0, 2 ** 32, (words,), np.uint32)
+    bits[0, 0] = 0
+    params, keep = B.make_params(b, hq, hkv, sq, skv, d, d ** -0.5, flags, block, block, window, bits)
+    o = torch.full_like(q, float("nan"))
+    lse = torch.full(q.shape[:3], float("nan"), device="cuda")
+    st = B.steel_attn_run_noalloc(params, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(),
+                                  torch.cuda.current_stream().cuda_stream)
+    assert st == B.STEEL_OK, B.steel_status_string(st)
+    attn = B.SteelAttention(b, hq, hkv, sq, skv, d, d ** -0.5, flags, block=block, window=window, bitmap=bits)
+    o_ref, lse_ref = attn.run(q, k, v)
+    assert attn.last_status() == B.STEEL_OK
+    err = (o.float() - o_ref.float()).abs()
+    assert not torch.isnan(o).any() and float(err.max()) <= H.TOL_O_MAX and float(err.mean()) <= H.TOL_O_MEAN
+    fin = torch.isfinite(lse_ref)
+    assert torch.equal(torch.isfinite(lse), fin) and float((lse[fin] - lse_ref[fin]).abs().max()) <= H.TOL_LSE
+    attn.close()
+
+
 def test_noalloc_rejects_plans_beyond_the_fixed_array():
     # 32 heads x 2048 query tiles = 32768 work items > 16384: refused, nothing launched
     params, _ = B.make_params(1, 32, 32, 262144, 262144, 128, 0.1, CAUSAL)
