@@ -432,7 +432,7 @@ steel_status_t steel_attn_debug_clock_probe(steel_attn_t *h, int64_t *device_pai
 steel_status_t steel_attn_debug_stall(steel_attn_t *h, int32_t cta, int64_t timeout_cycles) {
   if (!h || cta >= h->plan.grid) return STEEL_ERR_INVALID_ARG;
   h->stall_cta = cta < 0 ? -1 : cta;
-  h->timeout_cycles = timeout_cycles > 0 ? timeout_cycles : kDefaultTimeoutCycles;
+  h->timeout_cycles = timeout_cycles > 0 ? std::min<int64_t>(timeout_cycles, kMaxTimeoutCycles) : kDefaultTimeoutCycles;
   return STEEL_OK;
 }
 

@@ -40,6 +40,7 @@
 #include "sm100_ptx.cuh"
 #include "steel_kernel.h"
 #include "steel_plan.h"
+#include "steel_wait.cuh"
 
 namespace steel {
 
@@ -110,22 +111,6 @@ __device__ __forceinline__ bool bounded_wait(uint64_t *bar, uint32_t parity, Ctr
       }
     }
   }
-}
-
-constexpr uint32_t kPollLimit = 1u << 27;  // a poll takes 32 cycles or more: the default limit in cycles, or later
-
-// Wait by a whole warp: every lane tests the same barrier and the vote both keeps the warp together and
-// orders its lanes after the observation.  In the tile loop of the softmax warps, so it is short: it counts its polls
-// instead of reading the clock (a shorter limit than the default is the other roles' to notice, whose `abort` it
-// sees), and leaves the status word to the end of the kernel (with the clock and the status
-// in it: 32 heads x 4096 d128 119.3 us, as here 118.5; 16/4 x 2048 26.2 -> 25.6, 12 heads x 512 d64 8.52 -> 8.48).
-__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, Ctrl &ctrl) {
-  if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
-  uint32_t n = 0;
-  while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
-    if ((++n & 63u) == 0 && (*reinterpret_cast<volatile int *>(&ctrl.abort) != 0 || n >= kPollLimit)) return false;
-  }
-  return true;
 }
 
 // A work item unpacked into scalars (no indexable arrays, so everything stays in registers).

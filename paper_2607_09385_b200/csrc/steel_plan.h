@@ -9,6 +9,7 @@ namespace steel {
 
 constexpr int kTile = 128;  // query rows per tile and keys per tile
 constexpr long long kDefaultTimeoutCycles = 4000000000ll;  // about two seconds of SM clock
+constexpr long long kMaxTimeoutCycles = 1ll << 46;       // about ten hours: waits may keep time in 32 bits of 65 536 cycles
 
 // One step entry of one query tile ("slot") in a list-kind item.
 constexpr uint32_t kEntryTileMask = 0x00FFFFFFu;  // key-tile index

@@ -58,3 +58,25 @@ def test_status_is_read_and_cleared_on_its_own_stream():
         torch.cuda.synchronize()
     binding.steel_attn_debug_stall(attn.handle, -1)
     attn.close()
+
+
+@pytest.mark.parametrize("limit", [30_000_000, 300_000_000])
+def test_the_bound_holds_where_only_softmax_warps_wait(limit):
+    """Two key tiles per query tile: the stalled CTA's producer finds room for all of them in its ring and leaves, and so do
+    the issuers, so that nothing but the softmax warps' own bound ends the launch."""
+    q, k, v = (torch.randn((1, 1, 256, 128), device="cuda").to(torch.bfloat16) for _ in "qkv")
+    attn = binding.SteelAttention(1, 1, 1, 256, 256, 128, 0.1, 0)
+    o_ref, lse_ref = attn.run(q, k, v)
+    torch.cuda.synchronize()
+    binding.steel_attn_debug_stall(attn.handle, 0, limit)
+    t0 = time.time()
+    attn.run(q, k, v)
+    assert attn.last_status() == binding.STEEL_ERR_TIMEOUT
+    elapsed = time.time() - t0
+    # below the highest clock (1.965 GHz) and above a low one; a wait is looked at after its first 64 polls
+    assert limit / 2.0e9 * 0.99 < elapsed < limit / 0.3e9 + 2.0
+    binding.steel_attn_debug_stall(attn.handle, -1, 0)
+    o, lse = attn.run(q, k, v)
+    assert attn.last_status() == binding.STEEL_OK
+    assert torch.equal(o, o_ref) and torch.equal(lse, lse_ref)
+    attn.close()
