@@ -8,7 +8,8 @@
 // runs in the same kernel as steel_attn_run: this file only plans chunks, owns the staging buffers
 // and orders copies and launches with events.
 //
-// One stream brings the operands.  Three in turn, so that a copy's start-up hides behind the one before it, also let
+// One stream brings the operands.  Three in turn (measured while every chunk was copied back as soon as its kernel had
+// ended), so that a copy's start-up hides behind the one before it, also let
 // a later chunk's copies share the link with an earlier chunk's, which then ends later: us, one stream -> three,
 // head_dim 128, causal, 8 chunks: 32/8 heads x 4096 1 548 -> 1 410, 20/5 heads x 4096 (5 chunks) 1 005 -> 868, but
 // batch 8, 32/8 heads x 2048 4 674 -> 5 036, batch 16, 32/8 x 1024 4 581 -> 4 956, batch 4, 24/8 x 1777 1 841 -> 1 994,
@@ -26,6 +27,7 @@ struct steel_attn_host {
   int device = 0;
   int n_chunks = 1;
   size_t q_chunk_bytes = 0, kv_chunk_bytes = 0, lse_chunk_bytes = 0;
+  bool back_after_next = false;  // a chunk's copy back waits for the next chunk's operands
   std::vector<steel_attn_t *> child;  // one per chunk (bitmap masks) or a single shared one
   unsigned char *dq = nullptr, *dk = nullptr, *dv = nullptr, *dout = nullptr;
   float *dlse = nullptr;
@@ -35,6 +37,16 @@ struct steel_attn_host {
 };
 
 namespace {
+
+// Copies in both directions at once hinder each other, and by how much depends on where in a copy in the copy back
+// starts: with its start moved by 0, 5, 60, 100 and 130 us the call on 32 heads x 4096 d128 in 8 chunks took 2 340,
+// 2 230, 2 500, 2 300 and 2 470 us, so a kernel that became faster made the call slower (2 293 -> 2 354 us).  Started when
+// the next chunk's operands are in, beside the copies of the chunk after it, the copy back keeps its place.  Us, started
+// after the kernel -> here: 2 354 -> 2 200 (32/8 heads: 1 560 -> 1 290; 12 heads x 6000 dense, 6 chunks: 1 423 -> 1 316;
+// 32 heads x 1024 d64, 4 chunks: 378 -> 376).  It waits up to one chunk longer, which large chunks do not get back: batch
+// 2, 32/8 heads x 4096 (33.6 MB of Q each) 2 882 -> 3 231, batch 2 x 16 x 5000 (20.5 MB) 2 958 -> 3 076, batch 4, 24/8 x
+// 1777 (10.9 MB) 1 896 -> 1 936; at 8.4 MB (32 heads x 4096, 4 chunks) still 2 328 -> 2 253.
+constexpr size_t kSmallChunkBytes = size_t(8) << 20;
 
 int largest_divisor_up_to(int n, int limit) {
   int best = 1;
@@ -99,6 +111,7 @@ extern "C" steel_status_t steel_attn_host_create(const steel_attn_params_t *para
   h->q_chunk_bytes = static_cast<size_t>(cp.batch) * cp.heads_q * params->seq_q * row_bytes;
   h->kv_chunk_bytes = static_cast<size_t>(cp.batch) * cp.heads_kv * params->seq_kv * row_bytes;
   h->lse_chunk_bytes = static_cast<size_t>(cp.batch) * cp.heads_q * params->seq_q * sizeof(float);
+  h->back_after_next = h->q_chunk_bytes <= kSmallChunkBytes;
 
   // The bitmap is indexed by query head and shared across the batch: a head chunk needs its own
   // slice and plan, every other chunking runs all chunks through one plan.
@@ -119,10 +132,9 @@ extern "C" steel_status_t steel_attn_host_create(const steel_attn_params_t *para
       p.mask.bitmap = params->mask.bitmap + static_cast<int64_t>(c) * cp.heads_q * words_per_head;
     }
     steel_attn_t *child = nullptr;
-    // A chunk's kernel hides behind the copies, so what spreading it over all SMs changes is only when the copy back
-    // starts, and the call gets slower or faster with that (8 chunks, head_dim 128, paired query tiles / spread:
-    // 32 heads x 4096 2.29 / 2.42 ms, 12 heads x 6000 dense 1.43 / 1.30 ms, most others within 2 %): paired, and
-    // chunks stay without part buffers.
+    // A chunk's kernel hides behind the copies: paired query tiles / spread over all SMs, us, 8 chunks, head_dim 128:
+    // 32 heads x 4096 2 202 / 2 201, 12 heads x 6000 dense 1 311 / 1 303, 2 heads x 2043 dense 145 / 142, most
+    // others within 0.5 %.  Paired, and chunks stay without part buffers.
     st = steel::create_attention(&p, h->n_chunks > 1 ? steel::Spread::kNone : steel::Spread::kCut, &child);
     if (st == STEEL_OK) h->child.push_back(child);
   }
@@ -183,27 +195,34 @@ extern "C" steel_status_t steel_attn_host_run(steel_attn_host_t *h, const void *
   // everything below starts after the work already queued on the caller's stream
   STEEL_HOST_CHECK(cudaEventRecord(h->ev_begin, user));
   STEEL_HOST_CHECK(cudaStreamWaitEvent(h->s_in, h->ev_begin, 0));
+  auto copy_back = [&](int c) -> steel_status_t {
+    const size_t qo = c * h->q_chunk_bytes, lo = c * h->lse_chunk_bytes;
+    STEEL_HOST_CHECK(cudaStreamWaitEvent(h->s_out, h->ev_run[c], 0));
+    if (h->back_after_next && c + 1 < h->n_chunks) STEEL_HOST_CHECK(cudaStreamWaitEvent(h->s_out, h->ev_in[c + 1], 0));
+    STEEL_HOST_CHECK(cudaMemcpyAsync(ho + qo, h->dout + qo, h->q_chunk_bytes, cudaMemcpyDeviceToHost, h->s_out));
+    if (lse)
+      STEEL_HOST_CHECK(cudaMemcpyAsync(reinterpret_cast<unsigned char *>(lse) + lo,
+                                       reinterpret_cast<unsigned char *>(h->dlse) + lo, h->lse_chunk_bytes,
+                                       cudaMemcpyDeviceToHost, h->s_out));
+    return STEEL_OK;
+  };
   for (int c = 0; c < h->n_chunks; ++c) {
     const size_t qo = c * h->q_chunk_bytes, ko = c * h->kv_chunk_bytes, lo = c * h->lse_chunk_bytes;
     STEEL_HOST_CHECK(cudaMemcpyAsync(h->dq + qo, hq + qo, h->q_chunk_bytes, cudaMemcpyHostToDevice, h->s_in));
     STEEL_HOST_CHECK(cudaMemcpyAsync(h->dk + ko, hk + ko, h->kv_chunk_bytes, cudaMemcpyHostToDevice, h->s_in));
     STEEL_HOST_CHECK(cudaMemcpyAsync(h->dv + ko, hv + ko, h->kv_chunk_bytes, cudaMemcpyHostToDevice, h->s_in));
     STEEL_HOST_CHECK(cudaEventRecord(h->ev_in[c], h->s_in));
+    steel_status_t st = h->back_after_next && c > 0 ? copy_back(c - 1) : STEEL_OK;
+    if (st != STEEL_OK) return st;
 
     STEEL_HOST_CHECK(cudaStreamWaitEvent(h->s_run, h->ev_in[c], 0));
     steel_attn_t *child = h->child[h->child.size() == 1 ? 0 : c];
-    const steel_status_t st =
-        steel_attn_run(child, h->dq + qo, h->dk + ko, h->dv + ko, h->dout + qo,
-                       reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(h->dlse) + lo), h->s_run);
+    st = steel_attn_run(child, h->dq + qo, h->dk + ko, h->dv + ko, h->dout + qo,
+                        reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(h->dlse) + lo), h->s_run);
     if (st != STEEL_OK) return st;
     STEEL_HOST_CHECK(cudaEventRecord(h->ev_run[c], h->s_run));
-
-    STEEL_HOST_CHECK(cudaStreamWaitEvent(h->s_out, h->ev_run[c], 0));
-    STEEL_HOST_CHECK(cudaMemcpyAsync(ho + qo, h->dout + qo, h->q_chunk_bytes, cudaMemcpyDeviceToHost, h->s_out));
-    if (lse)
-      STEEL_HOST_CHECK(cudaMemcpyAsync(reinterpret_cast<unsigned char *>(lse) + lo,
-                                       reinterpret_cast<unsigned char *>(h->dlse) + lo, h->lse_chunk_bytes,
-                                       cudaMemcpyDeviceToHost, h->s_out));
+    if (!h->back_after_next || c + 1 == h->n_chunks) st = copy_back(c);
+    if (st != STEEL_OK) return st;
   }
   // the caller's stream continues once the last chunk is back in host memory
   STEEL_HOST_CHECK(cudaEventRecord(h->ev_end, h->s_out));

@@ -173,3 +173,28 @@ def test_chunks_of_few_queries_and_many_keys():
     assert float((lse - lse_dev.cpu()).abs().max()) <= H.TOL_LSE
     host.close()
     attn.close()
+
+
+@pytest.mark.parametrize("by_batch", [False, True])
+@pytest.mark.parametrize("seq", [32768, 32769])
+def test_copies_back_of_small_and_large_chunks(seq, by_batch):
+    """Chunks of 8 MiB of Q are copied back after the next chunk's operands have come, larger ones after their kernel.  Each
+    call has new operands, so rows that are copied too early or not at all show as the call's before."""
+    n, d = 3, 128
+    batch, heads = (n, 1) if by_batch else (1, n)
+    args = (batch, heads, heads, seq, seq, d, d ** -0.5, CAUSAL | WINDOW)
+    host, attn = B.SteelAttentionHost(*args, window=64, max_chunks=n), B.SteelAttention(*args, window=64)
+    assert host.chunks == n
+    q, k, v, o = (torch.empty((batch, heads, seq, d), dtype=torch.bfloat16, pin_memory=True) for _ in range(4))
+    lse = torch.empty((batch, heads, seq), pin_memory=True)
+    g = torch.Generator(device="cuda").manual_seed(seq)
+    for _ in range(3):
+        dev = [torch.randn(q.shape, generator=g, device="cuda").to(torch.bfloat16) for _ in "qkv"]
+        for t, x in zip((q, k, v), dev):
+            t.copy_(x)
+        host.run(q, k, v, o, lse)
+        assert host.last_status() == B.STEEL_OK
+        o_dev, lse_dev = attn.run(*dev)
+        assert torch.equal(o, o_dev.cpu()) and torch.equal(lse, lse_dev.cpu())
+    host.close()
+    attn.close()
