@@ -641,6 +641,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
     }
   }
   bool pair = true;
+  int64_t n_lists = 0, n_entries = 0;  // of single query tiles
   if (on_lengths) {
     std::vector<double> paired, single;
     double work = 0.0;
@@ -654,6 +655,8 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
       for (int batch = 0; batch < p->batch; ++batch)
         for (size_t n = 0; n < count.size(); ++n) {
           single.push_back(kSingleStep * double(count[n]) + kItemOverheadSteps);
+          ++n_lists;
+          n_entries += count[n];
           if (n % 2) continue;
           paired.push_back((n + 1 < count.size() ? 1.0 : kSingleStep) * double(count[n]) + kItemOverheadSteps);
           work += paired.back();
@@ -662,7 +665,7 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
     const double load = makespan(std::move(paired), num_ctas);
     pair = !(load > 1.1 * work / num_ctas && makespan(std::move(single), num_ctas) < 0.95 * load);
   }
-  device_lists = device_lists && on_lengths && !pair && !stats;
+  device_lists = device_lists && on_lengths && !pair && !stats && lists_on_device(n_lists, n_entries);
   const size_t key_words = size_t(c.tkv128 + 63) / 64;
   std::vector<uint32_t> entries;
   std::vector<uint64_t> keys;  // the key tiles of each task as bits

@@ -32,6 +32,12 @@ constexpr double combine_steps(double fill, int parts) { return 1.5 + 0.7 * fill
 // Shorter pieces (in key tiles) cost more to start and combine than they take.
 constexpr int min_piece_tiles(double fill) { return int(4 + 8 * fill); }
 
+// Whether a small kernel writes the lists of single query tiles, `entries` in all: its launch costs 2.5 us, and it saves
+// the host 0.06 us per list and 0.01 us per entry (steel_attn_run_noalloc at 110 shapes).  Us, lists from the host /
+// from the device: 4 lists of 10 entries 33.7 / 35.7, 16 of 37 36.7 / 37.8, 24 of 36 37.8 / 37.8, 24 of 117 51.0 / 51.0,
+// 32 of 73 39.8 / 38.8, 48 of 110 44.0 / 42.8, 128 of 825 79.8 / 67.2, 32 of 391 67.4 / 64.6.
+constexpr bool lists_on_device(int64_t lists, int64_t entries) { return 6 * lists + entries >= 240; }
+
 struct Draft {  // a work item before it is placed
   WorkItem w;
   std::vector<StepPair> list;
@@ -61,8 +67,8 @@ enum class Spread {
 // Scheduling policy and the other options come from `p`.  Without `stats` the plan's statistics stay 0 (they
 // take a walk over every block).  Where `plan` cuts key ranges, `whole` (if not null)
 // becomes the plan that would be taken without cuts: items, steps and the statistics of its items.
-// `device_lists`: where the items of a bitmap mask are single query tiles, the plan holds the lengths and places of
-// their lists only; the entry of tile J is BitmapMask::entry, in ascending order of J (Spread::kTiles, no `stats`).
+// `device_lists`: where the items of a bitmap mask are single query tiles and lists_on_device says so, the plan holds the
+// lengths and places of their lists only; the entry of tile J is BitmapMask::entry, in ascending order of J (Spread::kTiles, no `stats`).
 steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan, bool stats = true,
                           Spread spread = Spread::kNone, Plan *whole = nullptr, bool device_lists = false);
 
