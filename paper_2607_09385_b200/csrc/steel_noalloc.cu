@@ -40,25 +40,6 @@ std::mutex g_mutex;
 unsigned char *g_scratch_addr[kMaxDevices] = {};
 int g_sm_count[kMaxDevices] = {};
 
-// Once per device, with that device current: resolve the array's device address, read the SM
-// count, opt the kernels in to their shared-memory size.
-steel_status_t setup_device(int device, unsigned char **base, int *sm_count) {
-  std::lock_guard<std::mutex> lock(g_mutex);
-  if (!g_scratch_addr[device]) {
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return STEEL_ERR_CUDA;
-    if (prop.major != 10) return STEEL_ERR_CUDA;
-    void *ptr = nullptr;
-    if (cudaGetSymbolAddress(&ptr, g_scratch) != cudaSuccess || !ptr) return STEEL_ERR_CUDA;
-    if (configure_kernels() != cudaSuccess) return STEEL_ERR_CUDA;
-    g_sm_count[device] = prop.multiProcessorCount;
-    g_scratch_addr[device] = static_cast<unsigned char *>(ptr);
-  }
-  *base = g_scratch_addr[device];
-  *sm_count = g_sm_count[device];
-  return STEEL_OK;
-}
-
 // The step lists of single query tiles, from the bitmap: one warp per item, one lane per key tile, 32 at a time; a vote
 // gives each visible tile its place, in ascending order.  Bound by the latency of its few loads.  With the entries
 // made and copied by the host the call took 175 us (8 heads x 4096 d64, 64-token blocks), as here 144.
@@ -76,6 +57,28 @@ __global__ void write_lists(const WorkItem *items, int n_items, const uint32_t *
     if (e != 0 && place < w.n_steps) out[place] = StepPair{{e, 0u}};
     at += __popc(seen);
   }
+}
+
+// Once per device, with that device current: resolve the array's device address, read the SM
+// count, load every kernel that a later call may launch (code is loaded lazily, which can allocate device memory and wait
+// for the device) and opt the attention kernels in to their shared-memory size.
+steel_status_t setup_device(int device, unsigned char **base, int *sm_count) {
+  std::lock_guard<std::mutex> lock(g_mutex);
+  if (!g_scratch_addr[device]) {
+    cudaDeviceProp prop;
+    if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return STEEL_ERR_CUDA;
+    if (prop.major != 10) return STEEL_ERR_CUDA;
+    void *ptr = nullptr;
+    if (cudaGetSymbolAddress(&ptr, g_scratch) != cudaSuccess || !ptr) return STEEL_ERR_CUDA;
+    cudaFuncAttributes loaded;
+    if (configure_kernels() != cudaSuccess || cudaFuncGetAttributes(&loaded, write_lists) != cudaSuccess)
+      return STEEL_ERR_CUDA;
+    g_sm_count[device] = prop.multiProcessorCount;
+    g_scratch_addr[device] = static_cast<unsigned char *>(ptr);
+  }
+  *base = g_scratch_addr[device];
+  *sm_count = g_sm_count[device];
+  return STEEL_OK;
 }
 
 }  // namespace

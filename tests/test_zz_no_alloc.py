@@ -7,6 +7,9 @@ call and keeps the previous call's contents, so the test makes two calls in a ro
 problems and checks each against steel_attn_run on the same inputs.  This file is collected last
 on purpose: a run that stops at the first failure has then already run every other test.
 """
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -123,6 +126,28 @@ def test_noalloc_lists_written_on_the_device(shape, flags, window, block):
     fin = torch.isfinite(lse_ref)
     assert torch.equal(torch.isfinite(lse), fin) and float((lse[fin] - lse_ref[fin]).abs().max()) <= H.TOL_LSE
     attn.close()
+
+
+FIRST_CALLS = """
+import numpy as np, torch
+from paper_2607_09385_b200 import binding as B
+q, k, v = (torch.randn((1, 8, 1024, 64), device="cuda").to(torch.bfloat16) for _ in "qkv")
+o = torch.empty_like(q)
+free = []
+for flags, bits in ((B.STEEL_MASK_CAUSAL, None), (B.STEEL_MASK_CAUSAL | B.STEEL_MASK_BITMAP, np.full((8, 16, 1), 0xFFFFFFFF, np.uint32))):
+    params, keep = B.make_params(1, 8, 8, 1024, 1024, 64, 0.125, flags, 64, 64, 0, bits)
+    st = B.steel_attn_run_noalloc(params, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), None,
+                                  torch.cuda.current_stream().cuda_stream)
+    assert st == B.STEEL_OK, st
+    free.append(torch.cuda.mem_get_info()[0])
+assert free[0] == free[1], free
+"""
+
+
+def test_noalloc_sets_up_in_the_first_call_only(repo_root):
+    # the first call of a process has no bitmap; the first one with lists written on the device takes no memory either
+    out = subprocess.run([sys.executable, "-c", FIRST_CALLS], cwd=repo_root, capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr
 
 
 def test_noalloc_rejects_plans_beyond_the_fixed_array():
