@@ -193,3 +193,28 @@ def test_far_apart_scores_at_head_dim_64():
     assert (got - p).abs().le(p * (2.0 ** -7 + 2.0 ** -16 + 2.0 ** -20) + 1e-37).all()
     assert (got[p < 1e-45] == 0).all()
     assert torch.allclose(lse[0, 0].double().cpu(), torch.logsumexp(y, 1), rtol=0, atol=2e-6)  # fp32 values up to 4.2
+
+
+@pytest.mark.parametrize("head_dim", [64, 128])
+@pytest.mark.parametrize("size", [2.0 ** 33, 2.0 ** 37, 2.0 ** 44])
+def test_weights_beyond_the_largest_number_are_infinite_in_every_column(head_dim, size):
+    """Scaled scores so large that rounding the running maximum leaves exponents of 128 and more: 2 to their power is
+    infinite, and the row must show it (no row of such scores is right), whatever the column of the key."""
+    d, scale = head_dim, 1.1
+    a = 1.0 + torch.arange(128, device="cuda") / 128.0                    # exact in bf16
+    q, k, v = (torch.zeros((1, 1, 128, d), device="cuda") for _ in "qkv")
+    q[0, 0, :, 0] = a
+    v[0, 0, :, 1] = 1.0
+    # the exponent that is left of the largest score: its product with scale * log2(e) less that product rounded
+    scale_log2 = float(np.float32(scale) * np.float32(1.4426950408889634))
+    product = (a.double().cpu() * size * scale_log2).numpy()              # 8 and 24 bits: exact
+    left = torch.from_numpy(product - product.astype(np.float32).astype(np.float64))
+    rows = left >= 128.5
+    assert rows.sum() > 20
+    attn = binding.SteelAttention(1, 1, 1, 128, 128, d, scale, 0)
+    for j in range(128):
+        k.zero_()
+        k[0, 0, j, 0] = size
+        o, lse = attn.run(q.to(torch.bfloat16), k.to(torch.bfloat16), v.to(torch.bfloat16))
+        assert not o[0, 0].cpu()[rows][:, 1].isfinite().any(), j
+        assert (lse[0, 0].cpu()[rows] == float("inf")).all(), j
