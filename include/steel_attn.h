@@ -198,8 +198,9 @@ steel_status_t steel_attn_debug_clock_probe(steel_attn_t *handle, int64_t *devic
  * causal case that fits).  Arguments as for steel_attn_create and steel_attn_run.
  *
  * The call is blocking: it plans on the host (transient host memory only), copies the lists on
- * `cuda_stream`, runs the kernel, waits for the stream and returns the device status (STEEL_OK or
- * STEEL_ERR_TIMEOUT).  All calls in the process share the one array per GPU, which still holds the
+ * `cuda_stream`, runs the kernel, waits for the stream and returns the device status (STEEL_OK,
+ * STEEL_ERR_TIMEOUT, or STEEL_ERR_CUDA if step lists written on the device are not as long as planned: a defect of the
+ * library, or a bitmap that was changed during the call; outputs are undefined).  All calls in the process share the one array per GPU, which still holds the
  * previous call's lists when a call starts: the call rewrites the lists and clears the status word,
  * so two calls that overlap on the same GPU (from two threads or streams) race and must be
  * serialised by the caller.  The first call on each device also resolves the array's device

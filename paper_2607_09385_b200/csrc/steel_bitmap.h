@@ -1,5 +1,7 @@
-// The step entry of one (query tile, key tile) pair under a bitmap mask, from the mask's words: the same code for the
-// host and for the kernel that writes the step lists of steel_attn_run_noalloc.
+// The step entry of one (query tile, key tile) pair under a bitmap mask, from the mask's words, and the list of a query
+// tile made of them: what the kernel does that writes the step lists of steel_attn_run_noalloc.  The planner counts, and
+// makes its own lists, word by word (Ctx::kept_words); tests/list_entries.cpp compares the two, and a list that is not as
+// long as the planner has counted is reported (ListWriter::finish).
 #pragma once
 #include <stdint.h>
 
@@ -50,6 +52,35 @@ struct BitmapMask {
     if (j1 - j0 + 1 < kTile) full = false;  // a ragged last tile is masked element by element
     if (per == 1) sub = 0xFu;
     return uint32_t(J) | kEntryPresent | (sub << kEntrySubShift) | (full ? 0u : kEntryPartial);
+  }
+};
+
+STEEL_HOST_DEVICE inline int bits(uint32_t word) {
+#ifdef __CUDA_ARCH__
+  return __popc(word);
+#else
+  return __builtin_popcount(word);
+#endif
+}
+
+// One lane's part in writing a query tile's list, 32 key tiles at a time in ascending order.  Only the list's own
+// `n_steps` places are written.
+struct ListWriter {
+  StepPair *out;
+  int n_steps;
+  int at = 0;  // entries found so far, by all lanes
+
+  // `e`: the lane's entry (0 if its tile is not visible), `seen`: the lanes that have one.
+  STEEL_HOST_DEVICE void place(int lane, uint32_t e, uint32_t seen) {
+    const int here = at + bits(seen & ((1u << lane) - 1u));
+    if (e != 0 && here < n_steps) out[here] = StepPair{{e, 0u}};
+    at += bits(seen);
+  }
+  // After the last key tile: whether the list is as long as planned.  Places without an entry become key tile 0, so that
+  // the steps that the attention kernel expects are there whatever has gone wrong.
+  STEEL_HOST_DEVICE bool finish(int lane) {
+    for (int n = at + lane; n < n_steps; n += 32) out[n] = StepPair{{kEntryPresent | (0xFu << kEntrySubShift) | kEntryPartial, 0u}};
+    return at == n_steps;
   }
 };
 

@@ -42,21 +42,22 @@ int g_sm_count[kMaxDevices] = {};
 
 // The step lists of single query tiles, from the bitmap: one warp per item, one lane per key tile, 32 at a time; a vote
 // gives each visible tile its place, in ascending order.  Bound by the latency of its few loads.  With the entries
-// made and copied by the host the call took 175 us (8 heads x 4096 d64, 64-token blocks), as here 144.
+// made and copied by the host the call took 175 us (8 heads x 4096 d64, 64-token blocks), as here 144.  A list that is
+// not as long as the planner has counted sets the status word.
 constexpr int kListWarps = 8;
-__global__ void write_lists(const WorkItem *items, int n_items, const uint32_t *bitmap, BitmapMask mask, StepPair *steps) {
+constexpr int32_t kListMismatch = STEEL_ERR_CUDA;  // beside STEEL_ERR_TIMEOUT of the attention kernel
+__global__ void write_lists(const WorkItem *items, int n_items, const uint32_t *bitmap, BitmapMask mask, StepPair *steps,
+                            int32_t *status) {
   const int n = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
   if (n >= n_items || items[n].kind != 1) return;
   const WorkItem &w = items[n];
   const uint32_t *rows = bitmap + size_t(w.head[0]) * mask.blocks_q * mask.words;
-  StepPair *out = steps + w.j0[0];
-  for (int j0 = 0, at = 0; j0 < mask.key_tiles() && at < w.n_steps; j0 += 32) {
+  ListWriter list{steps + w.j0[0], w.n_steps};
+  for (int j0 = 0; j0 < mask.key_tiles(); j0 += 32) {
     const uint32_t e = j0 + lane < mask.key_tiles() ? mask.entry(rows, w.qtile[0], j0 + lane) : 0u;
-    const uint32_t seen = __ballot_sync(0xffffffffu, e != 0);
-    const int place = at + __popc(seen & ((1u << lane) - 1u));
-    if (e != 0 && place < w.n_steps) out[place] = StepPair{{e, 0u}};
-    at += __popc(seen);
+    list.place(lane, e, __ballot_sync(0xffffffffu, e != 0));
   }
+  if (!list.finish(lane) && lane == 0) atomicExch(status, kListMismatch);
 }
 
 // Once per device, with that device current: resolve the array's device address, read the SM
@@ -155,7 +156,7 @@ extern "C" steel_status_t steel_attn_run_noalloc(const steel_attn_params_t *para
     const int n_items = int(plan.items.size());
     write_lists<<<(n_items + kListWarps - 1) / kListWarps, kListWarps * 32, 0, stream>>>(
         reinterpret_cast<const WorkItem *>(base + off_items), n_items, reinterpret_cast<const uint32_t *>(base + off_bitmap),
-        mask, reinterpret_cast<StepPair *>(base + off_steps));
+        mask, reinterpret_cast<StepPair *>(base + off_steps), reinterpret_cast<int32_t *>(base));
     if (cudaGetLastError() != cudaSuccess) return STEEL_ERR_CUDA;
   }
   KernelParams kp{};  // no split query tiles: their buffers have no room in the array
@@ -177,5 +178,5 @@ extern "C" steel_status_t steel_attn_run_noalloc(const steel_attn_params_t *para
     cudaGetLastError();
     return STEEL_ERR_CUDA;
   }
-  return word == 0 ? STEEL_OK : STEEL_ERR_TIMEOUT;
+  return static_cast<steel_status_t>(word);  // 0, or set by one of the kernels
 }

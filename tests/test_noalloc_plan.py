@@ -28,3 +28,12 @@ def noalloc_plan(tmp_path_factory, repo_root):
 def test_short_lists_are_written_by_the_host(noalloc_plan, shape, items, entries, device):
     # a launch of its own costs a call of few entries more than writing them here
     assert noalloc_plan(*shape) == [items, entries, device]
+
+
+def test_a_list_of_another_length_than_planned_is_noticed(tmp_path, repo_root):
+    # and nothing is written beside it, and every planned place holds an entry that the attention kernel can walk
+    exe = str(tmp_path / "list_writer")
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-o", exe, os.path.join(repo_root, "tests", "list_writer.cpp"),
+                           os.path.join(repo_root, "paper_2607_09385_b200", "csrc", "steel_planner.cpp")])
+    out = subprocess.run([exe], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout
