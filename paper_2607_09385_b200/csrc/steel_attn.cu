@@ -105,18 +105,18 @@ void free_device(steel_attn *h) {
   if (h->roaming_done) cudaEventDestroy(h->roaming_done);
 }
 
-constexpr size_t round16(size_t n) { return (n + 15) / 16 * 16; }
+constexpr size_t round16(size_t n) { return round_up(n, 16); }
 
 // Append a plan's lists to `image`; `lists` receives offsets, which place_lists makes addresses.
 void append_lists(const Plan &plan, std::vector<unsigned char> *image, DeviceLists *lists) {
-  auto put = [image](const void *data, size_t bytes) {
-    const size_t at = image->size();
+  auto put = [image](const void *data, size_t bytes, size_t align = 16) {
+    const size_t at = round_up(image->size(), align);
     image->resize(at + round16(bytes));
     if (bytes) std::memcpy(image->data() + at, data, bytes);
     return at;
   };
   lists->cta_begin = reinterpret_cast<int32_t *>(put(plan.cta_begin.data(), plan.cta_begin.size() * sizeof(int32_t)));
-  lists->items = reinterpret_cast<WorkItem *>(put(plan.items.data(), plan.items.size() * sizeof(WorkItem)));
+  lists->items = reinterpret_cast<WorkItem *>(put(plan.items.data(), plan.items.size() * sizeof(WorkItem), 64));
   lists->steps = reinterpret_cast<StepPair *>(put(plan.steps.data(), plan.steps.size() * sizeof(StepPair)));
   lists->grid = plan.grid;
   lists->overlap_launch = plan.stats.max_cta_steps <= kOverlapSteps;

@@ -21,19 +21,9 @@ using namespace steel;
 
 namespace {
 
-constexpr size_t kMaxItems = 16384;   // work items (64 bytes each)
-constexpr size_t kMaxCtas = 1024;     // persistent CTAs (+1 range entry)
-constexpr size_t kMaxSteps = 131072;  // explicit step-list entries of bitmap masks (8 bytes each)
-// The call's lists are packed one behind the other, so that one copy brings them: status word, per-CTA
-// ranges, items, steps (or the bitmap, behind which the device writes the steps).
-constexpr size_t kOffCtaBegin = 256;
-constexpr size_t round16(size_t n) { return (n + 15) / 16 * 16; }
-constexpr size_t kScratchBytes = kOffCtaBegin + round16((kMaxCtas + 1) * sizeof(int32_t)) +
-                                 kMaxItems * sizeof(WorkItem) + kMaxSteps * sizeof(StepPair);  // about 2.0 MiB
-
 // In host code this name is only a handle for the symbol, never a device address: the address the
 // kernel needs comes from cudaGetSymbolAddress below.
-static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
+static __device__ __align__(256) unsigned char g_scratch[kNoallocBytes];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mutex;
@@ -107,44 +97,24 @@ extern "C" steel_status_t steel_attn_run_noalloc(const steel_attn_params_t *para
     return st;
   }
 
-  // Host memory only.  One query tile per item can need more list entries than pairs: where the fixed array
-  // has no room for it, the paired plan is taken.  What fits in neither way is refused, not truncated.
-  // Where the items of a bitmap mask are single query tiles, their lists are written on the device, from the bitmap,
-  // if that fits into the array beside them; else here.
-  Plan plan;
-  bool fits = false;
+  // Host memory only.
+  NoallocPlan np;
   std::vector<unsigned char> lists;  // what is copied: all but the status word's rest and device-written lists
-  size_t off_items = 0, off_steps = 0, off_bitmap = 0;
-  const BitmapMask mask = bitmap_mask(*params);
-  const size_t bitmap_bytes =
-      (params->mask.flags & STEEL_MASK_BITMAP) ? size_t(params->heads_q) * mask.blocks_q * mask.words * sizeof(uint32_t) : 0;
-  bool device_lists = false;
   try {
-    auto plan_as = [&](Spread spread, bool on_device) {
-      st = build_plan(params, sm_count, &plan, /*stats=*/false, spread, nullptr, on_device);
-      if (st != STEEL_OK) return;
-      fits = plan.items.size() <= kMaxItems && size_t(plan.n_steps) <= kMaxSteps && plan.cta_begin.size() <= kMaxCtas + 1;
-      off_items = kOffCtaBegin + round16(plan.cta_begin.size() * sizeof(int32_t));
-      off_steps = off_bitmap = off_items + plan.items.size() * sizeof(WorkItem);
-      device_lists = plan.steps.empty() && plan.n_steps > 0;
-      if (device_lists) off_steps += round16(bitmap_bytes);
-    };
-    plan_as(Spread::kTiles, bitmap_bytes > 0);
-    if (st == STEEL_OK && fits && device_lists && off_steps + size_t(plan.n_steps) * sizeof(StepPair) > kScratchBytes)
-      plan_as(Spread::kTiles, false);
-    if (st == STEEL_OK && !fits) plan_as(Spread::kNone, false);
+    st = plan_noalloc(params, sm_count, &np);
     if (st != STEEL_OK) return st;
-    if (!fits) return STEEL_ERR_UNSUPPORTED;
-    lists.resize(device_lists ? off_bitmap + bitmap_bytes : off_steps + plan.steps.size() * sizeof(StepPair));
+    lists.resize(np.copy_bytes);
   } catch (const std::bad_alloc &) {
     return STEEL_ERR_ALLOC;
   }
-  std::memcpy(lists.data() + kOffCtaBegin, plan.cta_begin.data(), plan.cta_begin.size() * sizeof(int32_t));
-  if (!plan.items.empty()) std::memcpy(lists.data() + off_items, plan.items.data(), plan.items.size() * sizeof(WorkItem));
-  if (device_lists)
-    std::memcpy(lists.data() + off_bitmap, params->mask.bitmap, bitmap_bytes);
-  else if (!plan.steps.empty())
-    std::memcpy(lists.data() + off_steps, plan.steps.data(), plan.steps.size() * sizeof(StepPair));
+  const Plan &plan = np.plan;
+  auto put = [&lists](size_t at, const void *data, size_t bytes) {
+    if (bytes) std::memcpy(lists.data() + at, data, bytes);
+  };
+  put(np.off_cta_begin, plan.cta_begin.data(), plan.cta_begin.size() * sizeof(int32_t));
+  put(np.off_items, plan.items.data(), plan.items.size() * sizeof(WorkItem));
+  put(np.off_bitmap, params->mask.bitmap, np.bitmap_bytes);
+  put(np.off_steps, plan.steps.data(), plan.steps.size() * sizeof(StepPair));
 
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   // The array still holds the previous call's lists and status word: overwrite both (the word with 0).
@@ -152,17 +122,17 @@ extern "C" steel_status_t steel_attn_run_noalloc(const steel_attn_params_t *para
     cudaGetLastError();
     return STEEL_ERR_CUDA;
   }
-  if (device_lists) {
+  if (np.device_lists) {
     const int n_items = int(plan.items.size());
     write_lists<<<(n_items + kListWarps - 1) / kListWarps, kListWarps * 32, 0, stream>>>(
-        reinterpret_cast<const WorkItem *>(base + off_items), n_items, reinterpret_cast<const uint32_t *>(base + off_bitmap),
-        mask, reinterpret_cast<StepPair *>(base + off_steps), reinterpret_cast<int32_t *>(base));
+        reinterpret_cast<const WorkItem *>(base + np.off_items), n_items, reinterpret_cast<const uint32_t *>(base + np.off_bitmap),
+        bitmap_mask(*params), reinterpret_cast<StepPair *>(base + np.off_steps), reinterpret_cast<int32_t *>(base));
     if (cudaGetLastError() != cudaSuccess) return STEEL_ERR_CUDA;
   }
   KernelParams kp{};  // no split query tiles: their buffers have no room in the array
-  kp.items = reinterpret_cast<const WorkItem *>(base + off_items);
-  kp.cta_begin = reinterpret_cast<const int32_t *>(base + kOffCtaBegin);
-  kp.steps = reinterpret_cast<const StepPair *>(base + off_steps);
+  kp.items = reinterpret_cast<const WorkItem *>(base + np.off_items);
+  kp.cta_begin = reinterpret_cast<const int32_t *>(base + np.off_cta_begin);
+  kp.steps = reinterpret_cast<const StepPair *>(base + np.off_steps);
   kp.status = reinterpret_cast<int32_t *>(base);
   set_query_view(*params, plan.packed, &kp);
   kp.overlap_launch = plan.stats.max_cta_steps <= kOverlapSteps;

@@ -925,6 +925,38 @@ BitmapMask bitmap_mask(const steel_attn_params_t &p) {
   return m;
 }
 
+steel_status_t plan_noalloc(const steel_attn_params_t *p, int num_ctas, NoallocPlan *np) {
+  const BitmapMask mask = bitmap_mask(*p);
+  const size_t bitmap_bytes =
+      (p->mask.flags & STEEL_MASK_BITMAP) ? size_t(p->heads_q) * mask.blocks_q * mask.words * sizeof(uint32_t) : 0;
+  Plan &plan = np->plan;
+  bool fits = false;
+  auto plan_as = [&](Spread spread, bool on_device) {
+    const steel_status_t st = build_plan(p, num_ctas, &plan, /*stats=*/false, spread, nullptr, on_device);
+    if (st != STEEL_OK) return st;
+    fits = plan.items.size() <= kNoallocItems && size_t(plan.n_steps) <= kNoallocSteps &&
+           plan.cta_begin.size() <= kNoallocCtas + 1;
+    np->device_lists = plan.steps.empty() && plan.n_steps > 0;
+    np->bitmap_bytes = np->device_lists ? bitmap_bytes : 0;
+    np->off_cta_begin = kNoallocStatusBytes;
+    // items start on 64 bytes, so that each lies in one cache line
+    np->off_items = round_up(np->off_cta_begin + plan.cta_begin.size() * sizeof(int32_t), 64);
+    np->off_bitmap = np->off_items + plan.items.size() * sizeof(WorkItem);
+    np->off_steps = np->off_bitmap + round_up(np->bitmap_bytes, 16);
+    np->end = np->off_steps + size_t(plan.n_steps) * sizeof(StepPair);
+    np->copy_bytes = np->device_lists ? np->off_bitmap + np->bitmap_bytes : np->end;
+    return STEEL_OK;
+  };
+  // One query tile per item can need more list entries than pairs: where the array has no room for it, the paired plan
+  // is taken.  Where the items of a bitmap mask are single query tiles, their lists are written on the device if the
+  // bitmap fits into the array beside them; else by the host.  What fits in no way is refused, not truncated.
+  steel_status_t st = plan_as(Spread::kTiles, bitmap_bytes > 0);
+  if (st == STEEL_OK && fits && np->device_lists && np->end > kNoallocBytes) st = plan_as(Spread::kTiles, false);
+  if (st == STEEL_OK && !fits) st = plan_as(Spread::kNone, false);
+  if (st != STEEL_OK) return st;
+  return fits ? STEEL_OK : STEEL_ERR_UNSUPPORTED;
+}
+
 int64_t plan_rows_q(const steel_attn_params_t &p, const Plan &plan) {
   return plan.packed ? int64_t(p.heads_q / p.heads_kv) * p.seq_q : p.seq_q;
 }

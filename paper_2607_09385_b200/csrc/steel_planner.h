@@ -74,6 +74,26 @@ steel_status_t build_plan(const steel_attn_params_t *p, int num_ctas, Plan *plan
 
 BitmapMask bitmap_mask(const steel_attn_params_t &p);
 
+// steel_attn_run_noalloc: the fixed array, and a call's plan and places in it, one behind the other so that one copy
+// brings them: status word, per-CTA ranges, items, then the bitmap where the device writes the step lists, then those.
+constexpr size_t kNoallocItems = 16384;   // work items (64 bytes each)
+constexpr size_t kNoallocCtas = 1024;     // persistent CTAs (+1 range entry)
+constexpr size_t kNoallocSteps = 131072;  // explicit step-list entries of bitmap masks (8 bytes each)
+constexpr size_t round_up(size_t n, size_t to) { return (n + to - 1) / to * to; }
+constexpr size_t kNoallocStatusBytes = 256;
+constexpr size_t kNoallocBytes = kNoallocStatusBytes + round_up((kNoallocCtas + 1) * sizeof(int32_t), 64) +
+                                 kNoallocItems * sizeof(WorkItem) + kNoallocSteps * sizeof(StepPair);  // about 2.0 MiB
+struct NoallocPlan {
+  Plan plan;
+  bool device_lists = false;
+  size_t off_cta_begin = 0, off_items = 0, off_bitmap = 0, off_steps = 0;
+  size_t bitmap_bytes = 0;  // 0 unless device_lists
+  size_t copy_bytes = 0;    // from the array's start, host -> device
+  size_t end = 0;           // of all that the call keeps in the array
+};
+// STEEL_ERR_UNSUPPORTED: no plan fits.  Host only; may throw std::bad_alloc.
+steel_status_t plan_noalloc(const steel_attn_params_t *p, int num_ctas, NoallocPlan *np);
+
 // steel_attn_create with a limit on what the plan may do (implemented in steel_attn.cu).
 steel_status_t create_attention(const steel_attn_params_t *params, Spread most, steel_attn_t **out);
 

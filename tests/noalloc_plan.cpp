@@ -1,6 +1,7 @@
-// Prints where the step lists of steel_attn_run_noalloc are written, for tests/test_noalloc_plan.py.  Host code only.
+// Prints how steel_attn_run_noalloc lays out a call, for tests/test_noalloc_plan.py, after checking that what it keeps
+// lies in the fixed array in order, aligned and without overlap.  Host code only.
 // usage: noalloc_plan batch heads_q heads_kv seq_q seq_kv flags window block words-value (hex, for every word)
-// prints: items, list entries, 1 if the device writes them
+// prints: items, list entries, 1 if the device writes them; or "refused"
 #include <cstdio>
 #include <cstdlib>
 
@@ -22,9 +23,22 @@ int main(int argc, char **argv) {
   const steel::BitmapMask m = steel::bitmap_mask(p);
   const std::vector<uint32_t> words(size_t(p.heads_q) * m.blocks_q * m.words, uint32_t(std::strtoul(argv[9], nullptr, 16)));
   p.mask.bitmap = words.data();
-  steel::Plan plan;
-  const steel_status_t st = steel::build_plan(&p, 148, &plan, false, steel::Spread::kTiles, nullptr, true);
+  steel::NoallocPlan np;
+  const steel_status_t st = steel::plan_noalloc(&p, 148, &np);
+  if (st == STEEL_ERR_UNSUPPORTED) return std::puts("refused"), 0;
   if (st != STEEL_OK) return 3;
-  std::printf("%zu %lld %d\n", plan.items.size(), (long long)plan.n_steps, int(plan.steps.empty() && plan.n_steps > 0));
+  const steel::Plan &plan = np.plan;
+  const size_t steps = size_t(plan.n_steps) * sizeof(steel::StepPair), bitmap = words.size() * sizeof(uint32_t);
+  const bool in_order = np.off_cta_begin >= sizeof(int32_t) &&
+                        np.off_items >= np.off_cta_begin + plan.cta_begin.size() * sizeof(int32_t) &&
+                        np.off_bitmap >= np.off_items + plan.items.size() * sizeof(steel::WorkItem) &&
+                        np.off_steps >= np.off_bitmap + np.bitmap_bytes && np.end >= np.off_steps + steps &&
+                        np.end <= steel::kNoallocBytes && np.copy_bytes <= np.end;
+  const bool aligned = np.off_cta_begin % 4 == 0 && np.off_items % 64 == 0 && np.off_bitmap % 4 == 0 && np.off_steps % 16 == 0;
+  const bool copied = np.device_lists ? np.bitmap_bytes == bitmap && np.copy_bytes == np.off_bitmap + bitmap && plan.steps.empty()
+                                      : np.bitmap_bytes == 0 && np.copy_bytes >= np.off_steps + steps &&
+                                            plan.steps.size() == size_t(plan.n_steps);
+  if (!in_order || !aligned || !copied) return std::printf("layout %d %d %d\n", in_order, aligned, copied), 4;
+  std::printf("%zu %lld %d\n", plan.items.size(), (long long)plan.n_steps, int(np.device_lists));
   return 0;
 }

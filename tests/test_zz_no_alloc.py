@@ -18,6 +18,7 @@ from paper_2607_09385_b200 import binding as B
 from paper_2607_09385_b200 import inputs
 
 import helpers as H
+from test_noalloc_plan import DEVICE_LISTS
 
 pytestmark = pytest.mark.gpu
 CAUSAL, WINDOW, BITMAP = inputs.MASK_CAUSAL, inputs.MASK_WINDOW, inputs.MASK_BITMAP
@@ -119,6 +120,29 @@ def test_noalloc_lists_written_on_the_device(shape, flags, window, block):
                                   torch.cuda.current_stream().cuda_stream)
     assert st == B.STEEL_OK, B.steel_status_string(st)
     attn = B.SteelAttention(b, hq, hkv, sq, skv, d, d ** -0.5, flags, block=block, window=window, bitmap=bits)
+    o_ref, lse_ref = attn.run(q, k, v)
+    assert attn.last_status() == B.STEEL_OK
+    err = (o.float() - o_ref.float()).abs()
+    assert not torch.isnan(o).any() and float(err.max()) <= H.TOL_O_MAX and float(err.mean()) <= H.TOL_O_MEAN
+    fin = torch.isfinite(lse_ref)
+    assert torch.equal(torch.isfinite(lse), fin) and float((lse[fin] - lse_ref[fin]).abs().max()) <= H.TOL_LSE
+    attn.close()
+
+
+@pytest.mark.parametrize("shape", DEVICE_LISTS)
+def test_noalloc_longer_lists_written_on_the_device(shape):
+    b, hq, hkv, sq, skv, flags, window, block = shape
+    g = torch.Generator(device="cuda").manual_seed(sq)
+    q, k, v = (torch.randn(s, generator=g, device="cuda").to(torch.bfloat16) for s in ((b, hq, sq, 64), (b, hkv, skv, 64), (b, hkv, skv, 64)))
+    rng = np.random.default_rng(skv)
+    bits = rng.integers(0, 2 ** 32, (hq, -(-sq // block), -(-(-(-skv // block)) // 32)), np.uint32)
+    bits[0, 0] = 0
+    params, keep = B.make_params(b, hq, hkv, sq, skv, 64, 0.125, flags, block, block, window, bits)
+    o, lse = torch.full_like(q, float("nan")), torch.full(q.shape[:3], float("nan"), device="cuda")
+    st = B.steel_attn_run_noalloc(params, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(),
+                                  torch.cuda.current_stream().cuda_stream)
+    assert st == B.STEEL_OK, B.steel_status_string(st)
+    attn = B.SteelAttention(b, hq, hkv, sq, skv, 64, 0.125, flags, block=block, window=window, bitmap=bits)
     o_ref, lse_ref = attn.run(q, k, v)
     assert attn.last_status() == B.STEEL_OK
     err = (o.float() - o_ref.float()).abs()
