@@ -462,7 +462,7 @@ __device__ void mma_role(const KernelParams &p, Ctrl &ctrl, uint8_t *smem_q, uin
   }
   // Leaving on an expired wait: everything this warp issued must have retired before the CTA frees
   // its tensor memory, so commit to a spare barrier and wait for it (bounded).
-  if (*reinterpret_cast<volatile int *>(&ctrl.abort)) {
+  if (warp_aborted(ctrl)) {
     if (elect_one()) {
       tc_commit(&ctrl.drain[who]);
       const long long start = clock64();

@@ -9,6 +9,12 @@
 
 namespace steel {
 
+// Whether a lane has seen a role give up: the same answer in every lane.
+template <class Ctrl>
+__device__ __forceinline__ bool warp_aborted(Ctrl &ctrl) {
+  return __any_sync(0xffffffffu, *reinterpret_cast<volatile int *>(&ctrl.abort) != 0);
+}
+
 // Every lane tests the same barrier; the vote both keeps the warp together and orders its lanes after the
 // observation.  In the tile loop of the softmax warps, so it is short: the clock and `abort` are looked at once in 64
 // polls (every poll that fails may suspend its thread, so polls are no measure of time), and the status word is left to

@@ -1,6 +1,6 @@
-"""The wait that the 32 lanes of a softmax warp make together, on host threads: all of them leave it in the same way whatever
-moment each one reads the abort flag at, it ends within the bound that the kernel was given however long a poll takes, and
-it passes as soon as the phase is complete.  CPU only."""
+"""The wait that the 32 lanes of a softmax warp make together, and the question whether a role has given up, on host
+threads: all lanes get the same answer whatever moment each one reads the abort flag at, a wait ends within the bound that
+the kernel was given however long a poll takes, and it passes as soon as the phase is complete.  CPU only."""
 import os
 import subprocess
 
@@ -15,7 +15,7 @@ def warp_wait(tmp_path_factory, repo_root):
     return exe
 
 
-@pytest.mark.parametrize("what", ["abort", "bound", "full"])
+@pytest.mark.parametrize("what", ["abort", "bound", "full", "leave"])
 def test_lanes_wait_together(warp_wait, what):
     out = subprocess.run([warp_wait, what], capture_output=True, text=True, timeout=120)
     assert out.returncode == 0, out.stdout

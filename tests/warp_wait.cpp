@@ -74,17 +74,16 @@ struct Ctrl {
   long long timeout_cycles = 0;
 };
 
-// Runs the wait in every lane; its result, which has to be the same in all.
-bool run(Warp &w, Ctrl &ctrl, long long *polls) {
+// Runs `call` in every lane; its result, which has to be the same in all.
+bool run(Warp &w, const std::function<bool()> &call, long long *polls) {
   g_warp = &w;
-  uint64_t bar = 0;
   int passed = 0;
   std::vector<std::thread> lanes;
   for (int lane = 0; lane < 32; ++lane)
     lanes.emplace_back([&, lane] {
       g_lane = lane;
       g_polls = g_clock = 0;
-      const bool ok = steel::warp_wait(&bar, 0u, ctrl);
+      const bool ok = call();
       std::lock_guard<std::mutex> lock(w.m);
       ++w.left;
       passed += ok;
@@ -101,6 +100,8 @@ int main(int argc, char **argv) {
   Warp w;
   Ctrl ctrl;
   long long polls = 0;
+  uint64_t bar = 0;
+  const auto wait = [&] { return steel::warp_wait(&bar, 0u, ctrl); };
   ctrl.timeout_cycles = 200'000'000;
   g_most_polls = 1 << 20;
   g_cycles_per_poll = 100;
@@ -116,20 +117,31 @@ int main(int argc, char **argv) {
       ctrl.abort = 1;
       self.cv.notify_all();
     };
-    if (run(w, ctrl, nullptr)) fail("the wait passed");
+    if (run(w, wait, nullptr)) fail("the wait passed");
   } else if (!std::strcmp(what, "bound")) {
     // a poll may suspend its thread for long: 500 polls to the limit, and the clock is looked at once in 64
     g_full_at = 1 << 20;
     g_cycles_per_poll = 400'000;
     g_most_polls = 500 + 3 * 64;
-    if (run(w, ctrl, &polls)) fail("the wait passed");
+    if (run(w, wait, &polls)) fail("the wait passed");
     if (polls < 490) fail("the wait ended before its bound");  // the clock is read in units of 65 536 cycles
   } else if (!std::strcmp(what, "full")) {
     for (long long at : {0, 1, 63, 64, 65, 200}) {
       Warp again;
       g_full_at = at;
-      if (!run(again, ctrl, &polls)) fail("the wait expired");
+      if (!run(again, wait, &polls)) fail("the wait expired");
       if (polls != at) fail("polls after the phase was complete");
+    }
+  } else if (!std::strcmp(what, "leave")) {
+    // the flag is set while lanes read it: each has a reading of its own
+    for (int seen_by : {0, 16, 32}) {
+      Warp again;
+      const auto aborted = [&] {
+        Ctrl mine;
+        mine.abort = g_lane < seen_by;
+        return steel::warp_aborted(mine);
+      };
+      if (run(again, aborted, nullptr) != (seen_by > 0)) fail("the flag was not seen");
     }
   } else {
     return 2;
