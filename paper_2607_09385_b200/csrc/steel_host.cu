@@ -43,10 +43,11 @@ namespace {
 // 2 230, 2 500, 2 300 and 2 470 us, so a kernel that became faster made the call slower (2 293 -> 2 354 us).  Started when
 // the next chunk's operands are in, beside the copies of the chunk after it, the copy back keeps its place.  Us, started
 // after the kernel -> here: 2 354 -> 2 200 (32/8 heads: 1 560 -> 1 290; 12 heads x 6000 dense, 6 chunks: 1 423 -> 1 316;
-// 32 heads x 1024 d64, 4 chunks: 378 -> 376).  It waits up to one chunk longer, which large chunks do not get back: batch
-// 2, 32/8 heads x 4096 (33.6 MB of Q each) 2 882 -> 3 231, batch 2 x 16 x 5000 (20.5 MB) 2 958 -> 3 076, batch 4, 24/8 x
-// 1777 (10.9 MB) 1 896 -> 1 936; at 8.4 MB (32 heads x 4096, 4 chunks) still 2 328 -> 2 253.
-constexpr size_t kSmallChunkBytes = size_t(8) << 20;
+// 32 heads x 1024 d64, 4 chunks: 378 -> 376; of 30 more shapes in 4 to 8 chunks most 1 to 9 % faster, one, batch 4 x 16 x
+// 681 d64, 471 -> 476).  It waits up to one chunk longer, which large or few chunks do not get back: batch 4, 24/8 x 1777
+// (10.9 MB of Q each) 1 896 -> 1 936, at 8.4 MB (32 heads x 4096, 4 chunks) still 2 328 -> 2 253; three chunks of 8.2 MB
+// 1 030 -> 1 054; two chunks of 0.8 MB 140 -> 146, 4.4 MB 428 -> 452, 33.6 MB 2 882 -> 3 231.
+bool back_after_next(int n_chunks, size_t q_chunk_bytes) { return n_chunks > 3 && q_chunk_bytes <= size_t(8) << 20; }
 
 int largest_divisor_up_to(int n, int limit) {
   int best = 1;
@@ -111,7 +112,7 @@ extern "C" steel_status_t steel_attn_host_create(const steel_attn_params_t *para
   h->q_chunk_bytes = static_cast<size_t>(cp.batch) * cp.heads_q * params->seq_q * row_bytes;
   h->kv_chunk_bytes = static_cast<size_t>(cp.batch) * cp.heads_kv * params->seq_kv * row_bytes;
   h->lse_chunk_bytes = static_cast<size_t>(cp.batch) * cp.heads_q * params->seq_q * sizeof(float);
-  h->back_after_next = h->q_chunk_bytes <= kSmallChunkBytes;
+  h->back_after_next = back_after_next(h->n_chunks, h->q_chunk_bytes);
 
   // The bitmap is indexed by query head and shared across the batch: a head chunk needs its own
   // slice and plan, every other chunking runs all chunks through one plan.

@@ -176,11 +176,11 @@ def test_chunks_of_few_queries_and_many_keys():
 
 
 @pytest.mark.parametrize("by_batch", [False, True])
-@pytest.mark.parametrize("seq", [32768, 32769])
-def test_copies_back_of_small_and_large_chunks(seq, by_batch):
-    """Chunks of 8 MiB of Q are copied back after the next chunk's operands have come, larger ones after their kernel.  Each
-    call has new operands, so rows that are copied too early or not at all show as the call's before."""
-    n, d = 3, 128
+@pytest.mark.parametrize("n,seq", [(3, 32768), (4, 32768), (4, 32769), (7, 700)])
+def test_copies_back_of_small_and_large_chunks(n, seq, by_batch):
+    """Four or more chunks of up to 8 MiB of Q are copied back after the next chunk's operands have come, others after
+    their kernel.  Each call has new operands, so rows that are copied too early or not at all show as the call's before."""
+    d = 128
     batch, heads = (n, 1) if by_batch else (1, n)
     args = (batch, heads, heads, seq, seq, d, d ** -0.5, CAUSAL | WINDOW)
     host, attn = B.SteelAttentionHost(*args, window=64, max_chunks=n), B.SteelAttention(*args, window=64)
