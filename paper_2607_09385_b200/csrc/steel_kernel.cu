@@ -524,8 +524,8 @@ __device__ __forceinline__ float2 exp2_full(float2 y) {
 // exponent the paper uses on the NPU generation that has no exponent unit).
 // kShare: one pair in eight by exp2_full.  At head_dim 64 the special-function unit is what a tile waits for (2 048
 // cycles for two tiles, their products take 1 024): 32 heads x 8192 340 -> 330 us, 2 x 12 heads x 4096 147 -> 144 us
-// (one in six: 335, 145.6; degree 5, as exact as ex2.approx but no more: 328, 143).  At head_dim 128 the products take as long as the exponentials and
-// it is slower (32 heads x 4096 121 -> 131 us).
+// (one in six: 335, 145.6; degree 5, as exact as ex2.approx but no more: 328, 143).  At head_dim 128 the products take
+// as long as the exponentials and it is slower (32 heads x 4096 121 -> 131 us).
 template <int kEmu, bool kShare>
 __device__ __forceinline__ void exp_half(const float (&x)[kTile], int base, float2 scale2, float2 neg_m2,
                                          float2 &acc_a, float2 &acc_b, uint32_t (&packed)[32]) {
