@@ -105,7 +105,8 @@ def test_noalloc_with_packed_heads(shape):
 @pytest.mark.parametrize("shape,flags,window", [((2, 4, 2, 700, 1333, 64), CAUSAL | BITMAP, 0), ((1, 3, 3, 1000, 300, 128), BITMAP, 0),
                                                 ((1, 6, 1, 129, 2001, 64), CAUSAL | WINDOW | BITMAP, 900)])
 def test_noalloc_lists_written_on_the_device(shape, flags, window, block):
-    # single query tiles under a bitmap: ragged and unequal lengths, tiles and rows without any visible key
+    # single query tiles under a bitmap: ragged and unequal lengths, tiles and rows without any visible key (the last two
+    # shapes have so few entries that the host writes them; DEVICE_LISTS below has longer ones)
     b, hq, hkv, sq, skv, d = shape
     rng = np.random.default_rng(44)
     q, k, v = (torch.from_numpy(rng.standard_normal(s, np.float32)).to(torch.bfloat16).cuda()
