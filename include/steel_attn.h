@@ -168,7 +168,7 @@ steel_status_t steel_attn_plan_host(const steel_attn_params_t *params, steel_att
 /*
  * Test hook for the bounded device-side waits.  With cta >= 0, CTA `cta` of the handle's following
  * runs withholds the commands its producer would publish, so the waits of its other roles expire
- * after `timeout_cycles` SM cycles (<= 0: the default, about two seconds): the kernel then returns
+ * after `timeout_cycles` SM cycles (<= 0: the default, about two seconds; at most 2^46): the kernel then returns
  * normally, outputs are undefined and steel_attn_last_status reports STEEL_ERR_TIMEOUT.  Nothing
  * faults or hangs; the context stays usable.  cta < 0 switches the hook off.
  */
